@@ -3,6 +3,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <functional>
 #include <new>
 #include <vector>
 
@@ -102,11 +103,12 @@ extern "C" vc_status vc_f2sp_create(uint64_t v, uint64_t h, int device, vc_f2sp 
     s->device = device;
     s->v = v;
     s->h = h;
-    // the transform's geometry: dimension d has size q[d]; slot = sum of
-    // digit_d stride_d, the last dimension innermost
+    // the transform's geometry: dimension d has size q[d], largest first; slot
+    // = sum of digit_d stride_d, the last dimension innermost
+    std::sort(q.begin(), q.end(), std::greater<u32>());
     const u32 m = (u32)q.size();
     std::vector<u32> stride(m), N(m), t(m);
-    u32 nroots = 0;
+    u32 ncs = 0;
     for (int d = (int)m - 1; d >= 0; d--) stride[d] = (d == (int)m - 1) ? 1 : stride[d + 1] * q[d + 1];
     SpFftHost &F = s->F;
     F.h = (u32)h;
@@ -116,22 +118,21 @@ extern "C" vc_status vc_f2sp_create(uint64_t v, uint64_t h, int device, vc_f2sp 
         t[d] = 0;
         while ((u64)N[d] * t[d] % q[d] != 1 % q[d]) t[d]++;  // (h / q_d)^{-1} mod q_d
         F.q[d] = q[d];
-        F.magic[d] = ((1u << 20) + q[d] - 1) / q[d];
-        F.twoff[d] = nroots;
-        nroots += q[d];
+        F.st[d] = stride[d];
+        F.magic[d] = (u32)(((u64(1) << 32) + stride[d] - 1) / stride[d]);  // (unused, 0, for stride 1)
+        F.cso[d] = ncs;
+        ncs += ((q[d] - 1) / 2) * ((q[d] - 1) / 2);
     }
-    F.nroots = nroots;
+    F.ncs = ncs;
     s->nparts = sp_prove_ctas(v);
     const u64 n2 = 2 * h;
-    u32 *d_pin = nullptr, *d_perm = nullptr, *d_idx = nullptr;
-    u64 *d_fw = nullptr, *d_bw = nullptr, *d_twist = nullptr;
+    u32 *d_pin = nullptr, *d_idx = nullptr;
+    u64 *d_cs = nullptr, *d_twist = nullptr;
     auto carve = [&](Arena &A) {
         d_pin = A.take<u32>(h);
-        d_perm = A.take<u32>(h);
         d_idx = A.take<u32>(h);
         d_twist = A.take<u64>(h);
-        d_fw = A.take<u64>(nroots + 1);
-        d_bw = A.take<u64>(nroots + 1);
+        d_cs = A.take<u64>(2 * ncs + 2);
         s->pw = A.take<u64>(n2);
         s->L = A.take<u64>(h);
         s->M = A.take<u64>(n2);
@@ -155,17 +156,22 @@ extern "C" vc_status vc_f2sp_create(uint64_t v, uint64_t h, int device, vc_f2sp 
         // 2h, w = u^2 the one of order h; root of dimension d = w^{h / q_d}
         const u64 u = h_pow(37, (FP_P - 1) / n2), w = h_mul(u, u);
         s->inv_h = h_inv(h);
-        std::vector<u64> pw(n2), fw(nroots + 1, 0), bw(nroots + 1, 0), twist(h);
-        std::vector<u32> pin(h), perm(h), idx(h);
+        std::vector<u64> pw(n2), cs(2 * ncs + 2, 0), twist(h);
+        std::vector<u32> pin(h), idx(h);
         u64 tpow = 1;
         for (u64 k = 0; k < n2; k++, tpow = h_mul(tpow, u)) pw[k] = tpow;
         for (u32 d = 0; d < m; d++) {
-            const u64 root = h_pow(w, N[d]), iroot = h_inv(root);
-            u64 f = 1, b = 1;
-            for (u32 e2 = 0; e2 < q[d]; e2++, f = h_mul(f, root), b = h_mul(b, iroot)) {
-                fw[F.twoff[d] + e2] = f;
-                bw[F.twoff[d] + e2] = b;
-            }
+            const u64 root = h_pow(w, N[d]);
+            std::vector<u64> pr(q[d], 1);
+            for (u32 e2 = 1; e2 < q[d]; e2++) pr[e2] = h_mul(pr[e2 - 1], root);
+            const u32 n = (q[d] - 1) / 2;
+            for (u32 k = 1; k <= n; k++)
+                for (u32 j = 1; j <= n; j++) {  // (root^{jk} +- root^{-jk}) / 2
+                    const u64 a = pr[j * k % q[d]], b = pr[(q[d] - j * k % q[d]) % q[d]];
+                    u64 *o = cs.data() + 2 * (F.cso[d] + (k - 1) * n + (j - 1));
+                    o[0] = h_mul(f_add(a, b), FP_INV2);
+                    o[1] = h_mul(f_sub(a, b), FP_INV2);
+                }
         }
         auto slot_of_input = [&](u64 y) {  // digits y t_d mod q_d
             u64 p = 0;
@@ -173,27 +179,24 @@ extern "C" vc_status vc_f2sp_create(uint64_t v, uint64_t h, int device, vc_f2sp 
             return (u32)p;
         };
         for (u64 y = 0; y < h; y++) pin[y] = slot_of_input(y);
-        for (u64 P = 0; P < h; P++) {  // output slot: digits k_d = j mod q_d; j by CRT
-            u64 j = 0;
+        for (u64 P = 0; P < h; P++) {
+            // digits: of the coefficient j, j mod q_d (j by CRT); of the output k = sum k_d N_d
+            u64 j = 0, k = 0;
             for (u32 d = 0; d < m; d++) {
                 const u64 kd = (P / stride[d]) % q[d];
                 j = (j + kd * N[d] % h * t[d]) % h;
+                k = (k + kd * N[d]) % h;
             }
-            idx[P] = (u32)j;
-            perm[P] = slot_of_input(j);
+            idx[P] = (u32)k;
             twist[P] = h_mul(pw[j], s->inv_h);
         }
         e = upload(d_pin, pin);
-        if (e == cudaSuccess) e = upload(d_perm, perm);
         if (e == cudaSuccess) e = upload(d_idx, idx);
         if (e == cudaSuccess) e = upload(d_twist, twist);
-        if (e == cudaSuccess) e = upload(d_fw, fw);
-        if (e == cudaSuccess) e = upload(d_bw, bw);
+        if (e == cudaSuccess) e = upload(d_cs, cs);
         if (e == cudaSuccess) e = upload(s->pw, pw);
-        F.fw = d_fw;
-        F.bw = d_bw;
+        F.cs = d_cs;
         F.pin = d_pin;
-        F.perm = d_perm;
         F.idx = d_idx;
         F.twist = d_twist;
     }

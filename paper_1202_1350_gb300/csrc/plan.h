@@ -427,14 +427,13 @@ u32 pergate_gpt();  // gates (and line entries) per CTA
 // transform (built by vc_f2sp_create): h = q_0 ... q_{m-1}, pairwise coprime
 // prime powers <= 61; device tables.
 struct SpFftHost {
-    u32 h, m, nroots;
-    u32 q[8], magic[8], twoff[8];
-    const u64 *fw, *bw;      // per dimension: its root's powers and inverse powers
-    const u32 *pin, *perm, *idx;
+    u32 h, m, ncs;
+    u32 q[8], st[8], magic[8], cso[8];
+    const u64 *cs;  // per dimension: its root's (c, s) pairs
+    const u32 *pin, *idx;
     const u64 *twist;
 };
 void sp_init();
-size_t sp_prove_smem(u64 h, u32 nroots);
 u32 sp_prove_ctas(u64 v);
 void launch_sp_prove(const u64 *a, u64 v, const SpFftHost &H, u64 *part, u32 nparts, u64 *proof, u32 *status,
                      cudaStream_t st);
