@@ -75,8 +75,8 @@ bool sp_factor(u64 h, std::vector<u32> &q)
 
 static vc_status sp_status(vc_f2sp *s, cudaStream_t st)
 {
-    cudaError_t e = cudaMemcpyAsync(s->h_res, s->res, 4 * sizeof(u64), cudaMemcpyDeviceToHost, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(s->h_res + 4, s->status, sizeof(u32), cudaMemcpyDeviceToHost, st);
+    // the status word follows the results: one copy
+    cudaError_t e = cudaMemcpyAsync(s->h_res, s->res, 5 * sizeof(u64), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return cuda_status(e);
     const u32 stv = (u32)(s->h_res[4] & 0xFFFFFFFFu);
@@ -139,8 +139,8 @@ extern "C" vc_status vc_f2sp_create(uint64_t v, uint64_t h, int device, vc_f2sp 
         s->acc = A.take<u64>(v);
         s->part = A.take<u64>((u64)s->nparts * n2);
         s->proof = A.take<u64>(n2);
-        s->res = A.take<u64>(4);
-        s->status = A.take<u32>(1);
+        s->res = A.take<u64>(5);
+        s->status = reinterpret_cast<u32 *>(s->res + 4);
     };
     Arena A0;
     carve(A0);
@@ -298,13 +298,16 @@ extern "C" vc_status vc_f2sp_prove(vc_f2sp *s, const uint64_t *a, uint64_t *proo
     if (!s || !a || !proof) return VC_EINVAL;
     DevGuard guard(s->device);
     cudaStream_t st = (cudaStream_t)stream;
-    if (ptr_kind(proof, s->device) < 0) return VC_EINVAL;
+    const int kp = ptr_kind(proof, s->device);
+    if (kp < 0) return VC_EINVAL;
     vc_status err;
     const u64 *da = sp_device_input(s, a, s->v * s->h, st, &err);
     if (!da) return err;
-    launch_sp_prove(da, s->v, s->F, s->part, s->nparts, s->proof, s->status, st);
+    // a proof buffer on the device is written in place
+    launch_sp_prove(da, s->v, s->F, s->part, s->nparts, kp ? proof : s->proof, s->status, st);
     cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess) e = cudaMemcpyAsync(proof, s->proof, 2 * s->h * sizeof(u64), cudaMemcpyDefault, st);
+    if (e == cudaSuccess && !kp)
+        e = cudaMemcpyAsync(proof, s->proof, 2 * s->h * sizeof(u64), cudaMemcpyDefault, st);
     if (e != cudaSuccess) return cuda_status(e);
     return sp_status(s, st);
 }

@@ -146,13 +146,22 @@ __device__ __forceinline__ u64 acc_red(const acc128 &a)
     return wred(t);
 }
 
-// Product of two W values, result in W.
+// The same for a below 7 * 2^122 (six products of W values and a 64-bit
+// term): a = (a div 2^61) 2^61 + (a mod 2^61), and the quotient, below
+// 7 * 2^61, is one funnel shift: half of acc_red's instructions.
+__device__ __forceinline__ u64 acc_red7(const acc128 &a)
+{
+    return wred((a.lo & FP_P) + ((a.hi << 3) | (a.lo >> 61)));
+}
+
+// Product of two values whose product is below 7 * 2^122 (W values, or
+// one below 2^63 and one canonical), result in W.
 __device__ __forceinline__ u64 wmul(u64 x, u64 y)
 {
     acc128 a;
     a.lo = x * y;
     a.hi = __umul64hi(x, y);
-    return acc_red(a);
+    return acc_red7(a);
 }
 
 // u0 + r (u1 - u0) for u0, u1 in W and canonical r given as 31/30-bit limbs

@@ -38,7 +38,12 @@
 #include "plan.h"
 
 #define SP_NT 256
-#define SP_PNT 512  // prover CTA
+// Prover CTA: 1024 threads (64 registers each) when every dimension is at most
+// 13, whose lines fit that; 512 (128 registers) otherwise.  A line's products
+// are dependent chains, so warps in flight matter: at 4995 x 5005 16 warps an
+// SM issued in 42 % of the cycles.
+#define SP_PNT 1024
+#define SP_PNT_BIG 512
 
 // Geometry and tables of the prover's transform (device pointers; built on
 // the host by vc_f2sp_create).
@@ -58,6 +63,9 @@ struct SpFft {
 // the factor 1/Q, swaps outputs k and Q - k), in place; with TW times
 // tw[slot].  Up to 13 values the sums and differences stay in registers
 // together; beyond, the differences wait in shared memory for the sums' half.
+// Values between passes are below 3 2^61 (lazy sums of two W values, or a
+// difference plus 2 p): the next pass's sums and differences, below 2^64, are
+// brought back to W.
 template <int Q, bool INV, bool TW>
 __device__ __forceinline__ void sp_line(u64 *p, u32 st, const ulonglong2 *cs, const u64 *__restrict__ tw)
 {
@@ -67,18 +75,18 @@ __device__ __forceinline__ void sp_line(u64 *p, u32 st, const ulonglong2 *cs, co
     u64 s[N];
     if constexpr (Q <= 13) {
         u64 d[N];
-        u64 t = x0;
+        u64 t = wred(x0);
 #pragma unroll
         for (int j = 0; j < N; j++) {
             const u64 a = p[(j + 1) * st], b = p[(Q - 1 - j) * st];
             s[j] = wred(a + b);
-            d[j] = wred(a + (2 * FP_P) - b);
+            d[j] = wred(a + (4 * FP_P) - b);
             t += s[j];  // at most seven W values: below 2^64
         }
         put(0, wred(t));
-#pragma unroll 2
+#pragma unroll 1
         for (int k = 1; k <= N; k++) {
-            acc128 c, e;
+            acc128 c, e;  // at most six products and x0
             c.lo = x0;
             c.hi = 0;
             acc_zero(e);
@@ -88,17 +96,17 @@ __device__ __forceinline__ void sp_line(u64 *p, u32 st, const ulonglong2 *cs, co
                 mac(c, s[j], w.x);
                 mac(e, d[j], w.y);
             }
-            const u64 C = acc_red(c), S = acc_red(e);
-            put(INV ? Q - k : k, wred(C + S));
-            put(INV ? k : Q - k, wred(C + (2 * FP_P) - S));
+            const u64 C = acc_red7(c), S = acc_red7(e);
+            put(INV ? Q - k : k, C + S);
+            put(INV ? k : Q - k, C + (2 * FP_P) - S);
         }
     } else {
-        u64 t = x0;
+        u64 t = wred(x0);
 #pragma unroll
         for (int j = 0; j < N; j++) {
             const u64 a = p[(j + 1) * st], b = p[(Q - 1 - j) * st];
             s[j] = wred(a + b);
-            p[(Q - 1 - j) * st] = wred(a + (2 * FP_P) - b);
+            p[(Q - 1 - j) * st] = wred(a + (4 * FP_P) - b);
             t += s[j];
             if ((j & 3) == 3) t = wred(t);
         }
@@ -123,8 +131,8 @@ __device__ __forceinline__ void sp_line(u64 *p, u32 st, const ulonglong2 *cs, co
 #pragma unroll
             for (int j = 0; j < N; j++) mac((j & 1) ? e1 : e0, s[j], cs[(k - 1) * N + j].y);
             const u64 C = p[k * st], S = wred(acc_red(e0) + acc_red(e1));
-            put(INV ? Q - k : k, wred(C + S));
-            put(INV ? k : Q - k, wred(C + (2 * FP_P) - S));
+            put(INV ? Q - k : k, C + S);
+            put(INV ? k : Q - k, C + (2 * FP_P) - S);
         }
     }
 }
@@ -136,12 +144,12 @@ enum { SP_INV = 0, SP_FWD = 1, SP_MID = 2 };
 
 // One pass over `nrows` rows in buf: a thread per line.  Lines of all the rows
 // are numbered together (line J starts at (J / st) q st + J mod st).
-template <int Q, int KIND>
+template <int Q, int KIND, int NT>
 __device__ __forceinline__ void sp_pass_q(u64 *buf, u32 nrows, const SpFft &F, u32 d, const ulonglong2 *cs)
 {
     const u32 st = F.st[d], n = nrows * (F.h / Q);
     const ulonglong2 *w = cs + F.cso[d];
-    for (u32 J = threadIdx.x; J < n; J += SP_PNT) {
+    for (u32 J = threadIdx.x; J < n; J += NT) {
         const u32 o = st == 1 ? J : __umulhi(J, F.magic[d]), in = J - o * st;
         u64 *p = buf + o * Q * st + in;
         if (KIND == SP_MID) {  // outermost digit: o is the row, `in` the line's first slot
@@ -155,42 +163,46 @@ __device__ __forceinline__ void sp_pass_q(u64 *buf, u32 nrows, const SpFft &F, u
     }
 }
 
-template <int KIND>
+template <int KIND, int NT>
 __device__ __noinline__ void sp_pass(u64 *buf, u32 nrows, const SpFft &F, u32 d, const ulonglong2 *cs)
 {
     switch (F.q[d]) {
-    case 3: sp_pass_q<3, KIND>(buf, nrows, F, d, cs); break;
-    case 5: sp_pass_q<5, KIND>(buf, nrows, F, d, cs); break;
-    case 7: sp_pass_q<7, KIND>(buf, nrows, F, d, cs); break;
-    case 9: sp_pass_q<9, KIND>(buf, nrows, F, d, cs); break;
-    case 11: sp_pass_q<11, KIND>(buf, nrows, F, d, cs); break;
-    case 13: sp_pass_q<13, KIND>(buf, nrows, F, d, cs); break;
-    case 25: sp_pass_q<25, KIND>(buf, nrows, F, d, cs); break;
-    case 31: sp_pass_q<31, KIND>(buf, nrows, F, d, cs); break;
-    case 41: sp_pass_q<41, KIND>(buf, nrows, F, d, cs); break;
-    case 61: sp_pass_q<61, KIND>(buf, nrows, F, d, cs); break;
-    default: break;  // vc_f2sp_create admits no other size
+    case 3: sp_pass_q<3, KIND, NT>(buf, nrows, F, d, cs); break;
+    case 5: sp_pass_q<5, KIND, NT>(buf, nrows, F, d, cs); break;
+    case 7: sp_pass_q<7, KIND, NT>(buf, nrows, F, d, cs); break;
+    case 9: sp_pass_q<9, KIND, NT>(buf, nrows, F, d, cs); break;
+    case 11: sp_pass_q<11, KIND, NT>(buf, nrows, F, d, cs); break;
+    case 13: sp_pass_q<13, KIND, NT>(buf, nrows, F, d, cs); break;
+    default:
+        if constexpr (NT == SP_PNT_BIG) switch (F.q[d]) {
+            case 25: sp_pass_q<25, KIND, NT>(buf, nrows, F, d, cs); break;
+            case 31: sp_pass_q<31, KIND, NT>(buf, nrows, F, d, cs); break;
+            case 41: sp_pass_q<41, KIND, NT>(buf, nrows, F, d, cs); break;
+            case 61: sp_pass_q<61, KIND, NT>(buf, nrows, F, d, cs); break;
+            default: break;  // vc_f2sp_create admits no other size
+            }
     }
 }
 
 // Column partials of the proof for the CTA's rows (consecutive, F.rb at a
 // time): part[cta][2y] = sum a(x, y)^2, part[cta][2k + 1] = sum f_x(u w^k)^2.
-__global__ void __launch_bounds__(SP_PNT, 1) k_sp_prove(const u64 *__restrict__ a, u64 v, SpFft F, u64 *part,
+template <int NT>
+__global__ void __launch_bounds__(NT, 1) k_sp_prove(const u64 *__restrict__ a, u64 v, SpFft F, u64 *part,
                                                         u32 *status)
 {
     extern __shared__ __align__(16) u64 sp_dyn[];
     const u32 h = F.h, gh = F.groups * h;
     ulonglong2 *cs = reinterpret_cast<ulonglong2 *>(sp_dyn);
     u64 *buf = sp_dyn + 2 * F.ncs, *acc_e = buf + F.rb * h, *acc_o = acc_e + gh;
-    for (u32 i = threadIdx.x; i < gh; i += SP_PNT) acc_e[i] = acc_o[i] = 0;
-    for (u32 i = threadIdx.x; i < F.ncs; i += SP_PNT) cs[i] = make_ulonglong2(F.cs[2 * i], F.cs[2 * i + 1]);
+    for (u32 i = threadIdx.x; i < gh; i += NT) acc_e[i] = acc_o[i] = 0;
+    for (u32 i = threadIdx.x; i < F.ncs; i += NT) cs[i] = make_ulonglong2(F.cs[2 * i], F.cs[2 * i + 1]);
     bool bad = false;
     const u64 x0 = v * blockIdx.x / gridDim.x, x1 = v * (blockIdx.x + 1) / gridDim.x;
     for (u64 x = x0; x < x1; x += F.rb) {
         const u32 nr = (u32)(x1 - x < F.rb ? x1 - x : F.rb);
         const u64 *rows = a + x * h;
         __syncthreads();  // the previous rows are done with the buffer
-        for (u32 e = threadIdx.x; e < gh; e += SP_PNT) {
+        for (u32 e = threadIdx.x; e < gh; e += NT) {
             const u32 g = F.groups == 1 ? 0 : e / h, y = e - g * h;
             const u32 slot = __ldg(F.pin + y);
             u64 sum = acc_e[e];
@@ -207,30 +219,30 @@ __global__ void __launch_bounds__(SP_PNT, 1) k_sp_prove(const u64 *__restrict__ 
         if (x + F.rb < x1) {
             const u64 *nx = rows + (u64)F.rb * h;
             const u64 left = (x1 - x - F.rb) * h, want = (u64)F.rb * h;
-            for (u64 o = threadIdx.x * 16; o < (left < want ? left : want); o += SP_PNT * 16)
+            for (u64 o = threadIdx.x * 16; o < (left < want ? left : want); o += NT * 16)
                 asm volatile("prefetch.global.L2 [%0];" ::"l"(nx + o));
         }
         __syncthreads();
         if (F.m == 0) {  // h = 1: only the twist (u^0 / 1)
-            for (u32 i = threadIdx.x; i < nr; i += SP_PNT) buf[i] = wmul(buf[i], F.twist[0]);
+            for (u32 i = threadIdx.x; i < nr; i += NT) buf[i] = wmul(buf[i], F.twist[0]);
             __syncthreads();
         } else {
             for (u32 d = F.m - 1; d > 0; d--) {
-                sp_pass<SP_INV>(buf, nr, F, d, cs);
+                sp_pass<SP_INV, NT>(buf, nr, F, d, cs);
                 __syncthreads();
             }
-            sp_pass<SP_MID>(buf, nr, F, 0, cs);
+            sp_pass<SP_MID, NT>(buf, nr, F, 0, cs);
             __syncthreads();
             for (u32 d = 1; d < F.m; d++) {
-                sp_pass<SP_FWD>(buf, nr, F, d, cs);
+                sp_pass<SP_FWD, NT>(buf, nr, F, d, cs);
                 __syncthreads();
             }
         }
-        for (u32 e = threadIdx.x; e < gh; e += SP_PNT) {
+        for (u32 e = threadIdx.x; e < gh; e += NT) {
             const u32 g = F.groups == 1 ? 0 : e / h, i = e - g * h;
             u64 sum = acc_o[e];
             for (u32 r = g; r < nr; r += F.groups) {
-                const u64 f = buf[r * h + i];
+                const u64 f = wred(buf[r * h + i]);
                 sum = wred(sum + wmul(f, f));
             }
             acc_o[e] = sum;
@@ -238,7 +250,7 @@ __global__ void __launch_bounds__(SP_PNT, 1) k_sp_prove(const u64 *__restrict__ 
     }
     if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(status, ST_BAD_INPUT);
     u64 *out = part + (u64)blockIdx.x * 2 * h;
-    for (u32 i = threadIdx.x; i < h; i += SP_PNT) {
+    for (u32 i = threadIdx.x; i < h; i += NT) {
         u64 se = 0, so = 0;
         for (u32 g = 0; g < F.groups; g++) {
             se = wred(se + acc_e[g * h + i]);
@@ -336,20 +348,24 @@ __global__ void __launch_bounds__(SP_VNT) k_sp_vabsorb(const u64 *__restrict__ r
         const u64 *row = rows + x * h;
         u64 red = 0;
         bool bad = false;
-        for (u32 y0 = lane; y0 < n; y0 += 32 * SP_VU) {
-            u64 val[SP_VU], l[SP_VU];
+        u64 val[SP_VU];
+        auto load = [&](u32 y0) {
 #pragma unroll
-            for (u32 u = 0; u < SP_VU; u++) {
-                const u32 y = y0 + 32 * u;
-                val[u] = y < n ? __ldcs(row + y) : 0;
-                l[u] = y < n ? __ldg(L + y) : 0;
-            }
+            for (u32 u = 0; u < SP_VU; u++) val[u] = y0 + 32 * u < n ? __ldcs(row + y0 + 32 * u) : 0;
+        };
+        load(lane);
+        for (u32 y0 = lane; y0 < n; y0 += 32 * SP_VU) {
+            u64 cur[SP_VU];
+#pragma unroll
+            for (u32 u = 0; u < SP_VU; u++) cur[u] = val[u];
+            load(y0 + 32 * SP_VU);  // the next entries arrive during this batch's products
             acc128 s;
             acc_zero(s);
 #pragma unroll
             for (u32 u = 0; u < SP_VU; u++) {
-                bad |= val[u] >= FP_P;
-                mac(s, val[u] >= FP_P ? 0 : val[u], l[u]);
+                const u32 y = y0 + 32 * u;
+                bad |= cur[u] >= FP_P;
+                mac(s, cur[u] >= FP_P ? 0 : cur[u], y < n ? __ldg(L + y) : 0);
             }
             red = wred(red + acc_red(s));
         }
@@ -362,7 +378,7 @@ __global__ void __launch_bounds__(SP_VNT) k_sp_vabsorb(const u64 *__restrict__ r
 // Verifier end (one CTA): res[0] = accept, res[1] = F2 answer (the even
 // points), res[2] = s(r), res[3] = sum_x f_x(r)^2.
 #define SP_ENT 1024
-#define SP_EU 4
+#define SP_EU 8
 __global__ void __launch_bounds__(SP_ENT) k_sp_vend(const u64 *__restrict__ proof, u64 v, u64 h,
                                                     const u64 *__restrict__ M, const u64 *__restrict__ acc, u64 *res)
 {
@@ -420,10 +436,10 @@ __global__ void __launch_bounds__(SP_ENT) k_sp_vend(const u64 *__restrict__ proo
 
 // Rows a CTA transforms together, its accumulators per column and its shared
 // memory.  About 14,000 values at once: at h = 5005 two rows, whose lines
-// (2 x 385 of size 13 up to 2 x 1001 of size 5) fill the 512 threads better
-// than one row's and halve the barriers; short rows many at a time.  At most
-// the CTA's share of the rows, and what 227 KB hold.
-void sp_prove_shape(u64 v, u64 h, u32 ncs, u32 *rb, u32 *groups, size_t *smem)
+// (2 x 385 of size 13 up to 2 x 1001 of size 5) fill the threads better than
+// one row's and halve the barriers; short rows many at a time.  At most the
+// CTA's share of the rows, and what 227 KB hold.
+static void sp_prove_shape(u64 v, u64 h, u32 nt, u32 ncs, u32 *rb, u32 *groups, size_t *smem)
 {
     const u64 ctas = sp_prove_ctas(v), share = (v + ctas - 1) / ctas;
     const u64 room = 227 * 1024 / 8 - 2 * ncs;
@@ -431,7 +447,7 @@ void sp_prove_shape(u64 v, u64 h, u32 ncs, u32 *rb, u32 *groups, size_t *smem)
     if (r > share) r = share;
     if (r < 1) r = 1;
     while (true) {
-        g = SP_PNT / h;
+        g = nt / h;
         if (g > r) g = r;
         if (g < 1) g = 1;
         if (r == 1 || (r + 2 * g) * h <= room) break;
@@ -446,7 +462,8 @@ u32 sp_prove_ctas(u64 v) { return (u32)(v < (u64)device_sms() ? v : (u64)device_
 
 void sp_init()
 {
-    cudaFuncSetAttribute(k_sp_prove, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    cudaFuncSetAttribute(k_sp_prove<SP_PNT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+    cudaFuncSetAttribute(k_sp_prove<SP_PNT_BIG>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
 }
 
 void launch_sp_prove(const u64 *a, u64 v, const SpFftHost &H, u64 *part, u32 nparts, u64 *proof, u32 *status,
@@ -467,8 +484,12 @@ void launch_sp_prove(const u64 *a, u64 v, const SpFftHost &H, u64 *part, u32 npa
     F.twist = H.twist;
     F.idx = H.idx;
     size_t smem = 0;
-    sp_prove_shape(v, H.h, H.ncs, &F.rb, &F.groups, &smem);
-    k_sp_prove<<<nparts, SP_PNT, smem, st>>>(a, v, F, part, status);
+    const bool big = H.m && H.q[0] > 13;  // the largest dimension is first
+    sp_prove_shape(v, H.h, big ? SP_PNT_BIG : SP_PNT, H.ncs, &F.rb, &F.groups, &smem);
+    if (big)
+        k_sp_prove<SP_PNT_BIG><<<nparts, SP_PNT_BIG, smem, st>>>(a, v, F, part, status);
+    else
+        k_sp_prove<SP_PNT><<<nparts, SP_PNT, smem, st>>>(a, v, F, part, status);
     k_sp_reduce<<<(unsigned)((2 * H.h + 31) / 32), SP_NT, 0, st>>>(part, nparts, 2 * H.h, proof);
 }
 
