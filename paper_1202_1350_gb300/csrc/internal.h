@@ -10,7 +10,7 @@
 #include "vc.h"
 
 constexpr u32 WV_LOG = 7;                  // log2 of the threads of a wave CTA
-constexpr u32 PR_CHUNK_LOG = PR_M + WV_LOG;  // rounds of one PROD chunk (2^PR_M entries per thread)
+constexpr u32 PR_CHUNK_LOG = PR_C + PR_R;    // rounds of one PROD chunk
 constexpr u32 GN_CHUNK_LOG = GN_M + WV_LOG;  // rounds of one GEN chunk (2^GN_M entries per thread)
 constexpr u32 LN_CHUNK0_LOG = 6 + WV_LOG;    // coordinates of a first line-wave chunk (64 entries per thread)
 constexpr u32 LN_CHUNKW_LOG = WV_LOG;        // coordinates of a later line-wave chunk (one polynomial per thread)
@@ -52,7 +52,10 @@ constexpr u32 VC_VALUES_SLOTTED = VC_VALUES_STAGED | VC_VALUES_WINDOWED;
 
 // Which layers' phase-2/3 tables are built by k_build23 (the rest are formed
 // on the fly or never stored).
-inline bool needs_tables(u32 kind) { return kind != W_SQUARE && kind != W_TREE; }
+// Layers whose phases 2 and 3 run over tables built by k_build23, and those
+// whose phase 2 looks up eq(r_P, .).
+inline bool needs_tables(u32 kind) { return kind == W_EXPLICIT; }
+inline bool needs_eq_rp(u32 kind) { return kind != W_TREE && kind != W_MATMULT; }
 
 // Bump allocator over one device allocation (base 0: sizing pass).
 struct Arena {
@@ -106,13 +109,14 @@ struct Plan {
     Globals *d_G = nullptr;
     std::vector<Globals> h_G;  // members' globals (merged plans: uploaded to d_G)
     std::vector<Item> checks;  // canonical-input checks (circuit, 2048-input block)
+    std::vector<Item> setups;  // coin setup CTAs (circuit, slice)
     std::vector<EqJob> eqjobs;
     std::vector<EvalSeg> segs;
     std::vector<LayerEval> levs;
     std::vector<std::vector<Item>> seg_items, lev_items;  // per evaluation step
     std::vector<u32> seg_maxblock;                         // per step: largest block of its runs
     std::vector<LineWaveDev> lw;
-    std::vector<BuildItem> builds;
+    std::vector<BuildItem> builds, mms;  // k_build23 (EXPLICIT), k_mm_tables (MATMULT)
     std::vector<HeavyItem> heavy;  // explicit layers' entries with long gate lists (k_build_heavy)
     std::vector<SciDev> scis;
     std::vector<ProdWave> pw;
@@ -124,7 +128,7 @@ struct Plan {
     u32 nbig = 0;
     std::vector<u32> outs;
     // device copies
-    Item *d_checks = nullptr;
+    Item *d_checks = nullptr, *d_setups = nullptr;
     EqJob *d_eqjobs = nullptr;
     EvalSeg *d_segs = nullptr;
     LayerEval *d_levs = nullptr;
@@ -132,7 +136,7 @@ struct Plan {
     std::vector<Task *> d_groupsA, d_groupsB;
     u32 *d_ctr = nullptr;  // two task counters per wave launch (A groups, then B groups)
     LineWaveDev *d_lw = nullptr;
-    BuildItem *d_builds = nullptr;
+    BuildItem *d_builds = nullptr, *d_mms = nullptr;
     HeavyItem *d_heavy = nullptr;
     SciDev *d_scis = nullptr;
     ProdWave *d_pw = nullptr;
@@ -251,8 +255,8 @@ struct vc_circuit {
                                                           // group g, list ng = every iteration between
                                                           // narrow layers
     std::vector<std::vector<Task *>> d_stA, d_stB;
-    std::vector<std::vector<BuildItem>> stBuild;  // [list]
-    std::vector<BuildItem *> d_stBuild;
+    std::vector<std::vector<BuildItem>> stMm;  // [list]
+    std::vector<BuildItem *> d_stMm;
     std::vector<std::vector<Item>> stEval;  // [layer]: 256-gate blocks of k_eval_layer
     std::vector<Item *> d_stEval;
     LayerEval *d_stLev = nullptr;  // one descriptor per layer

@@ -85,8 +85,7 @@ __global__ void __launch_bounds__(256, MINB) k_pair_rate(u64 iters, u64 *sink)
         y[c] = ((t + 7) * 0xBF58476D1CE4E5B9ull + 3 * c) & FP_P;
         w[c] = ((t + 11) * 0x94D049BB133111EBull + 5 * c) & FP_P;
     }
-    u32 r0, r1;
-    limbs31(0x123456789ABCDEull + t, r0, r1);
+    const u64 r = 0x123456789ABCDEull + t;
     acc128 a0, a1;
     acc_zero(a0);
     acc_zero(a1);
@@ -96,7 +95,7 @@ __global__ void __launch_bounds__(256, MINB) k_pair_rate(u64 iters, u64 *sink)
         for (int c = 0; c < CH; c++) {
             mac(a0, w[c], x[c]);
             mac(a1, w[c], y[c]);
-            const u64 f = wfold(x[c], y[c], r0, r1);
+            const u64 f = wfold(x[c], y[c], r);
             y[c] = x[c];
             x[c] = f;
         }

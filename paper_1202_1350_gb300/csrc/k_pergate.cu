@@ -230,10 +230,8 @@ __global__ void __launch_bounds__(PG_NT) k_pg_step(const Globals *G, const PgLay
         const u64 *F = (j == 0) ? L.Vn : ((j & 1) ? Q.fa : Q.fb);
         u64 *Fo = ((j + 1) & 1) ? Q.fa : Q.fb;
         const u64 nout = 1ull << (Q.sn - j - 1);
-        u32 c0l, c1l;
-        limbs31(ch, c0l, c1l);
         for (u64 y = gid; y < nout; y += gs) {
-            const u64 v = wcanon(wfold(F[2 * y], F[2 * y + 1], c0l, c1l));
+            const u64 v = wcanon(wfold(F[2 * y], F[2 * y + 1], ch));
             Fo[y] = v;
             if (nout == 1 && r == Q.s + Q.sn - 1) *Q.v1 = v;  // V~_{i+1}(r1)
         }

@@ -469,12 +469,15 @@ void prove_kernels_init()
 }
 
 // --------------------------------------------------------------------------------
-// Phase-2/3 tables over layer i+1, gathered per entry w (no atomics).
+// Phase-2/3 tables of an EXPLICIT layer over layer i+1, gathered per entry w
+// (no atomics; the structured kinds need none, see the PK_* and GS_* lists).
 //   w_g = eq(z, r_P) eq(r_P, g),   u_g = w_g eq(r1, in1(g))
 //   P2[w] = sum_{g: in1=w} w_g [ADD: 1, MUL: V(in2)],   B2[w] = sum_{ADD g: in1=w} w_g V(in2)
 //   A2[w] = sum_{ADD g: in2=w} u_g,   M2[w] = sum_{MUL g: in2=w} u_g
 //   P3 = A2 + v1 M2,   B3 = v1 A2,   v1 = V~_{i+1}(r1)
-// Phase-2 message: sum P2 V + B2; phase-3 message: sum P3 V + B3.
+// Phase-2 message: sum P2 V + B2; phase-3 message: sum P3 V + B3.  An entry
+// read by more than BUILD_HEAVY gates is summed by a whole CTA afterwards
+// (k_build_heavy), which adds to what is written here.
 // --------------------------------------------------------------------------------
 
 __global__ void __launch_bounds__(256) k_build23(const Globals *Gs, const BuildItem *items)
@@ -484,118 +487,28 @@ __global__ void __launch_bounds__(256) k_build23(const Globals *Gs, const BuildI
     const u32 i = bi.layer;
     const LayerDev &L = G.layers[i];
     const u64 w = (u64)bi.block * blockDim.x + threadIdx.x;
-    const u64 Sn = 1ull << L.sn;
+    if (w >= (1ull << L.sn)) return;
     const u64 ez = G.scal[SCAL_EQZRP(i)];
     const u64 v1 = G.scal[SCAL_V1(i)];
     const u64 *V = L.Vn;
-    if (L.kind == W_F0_PAIR || L.kind == W_F0_FINAL) {
-        // a thread per pair of entries 2q, 2q+1 (their gates share operands;
-        // a thread per entry left half of each warp idle on the other path)
-        const u64 q = w;
-        if (2 * q >= Sn) return;
-        u64 P2a, P2b, M2;
-        if (L.kind == W_F0_PAIR) {  // gate 2q = v_2q^2, gate 2q+1 = v_2q+1 v_2q
-            const u64 wg0 = f_mul(ez, eq_at(L.trp, 2 * q)), wg1 = f_mul(ez, eq_at(L.trp, 2 * q + 1));
-            const u64 x = V[2 * q];
-            P2a = f_mul(wg0, x);
-            P2b = f_mul(wg1, x);
-            M2 = f_add(f_mul(wg0, eq_at(L.tr1, 2 * q)), f_mul(wg1, eq_at(L.tr1, 2 * q + 1)));
-        } else {  // gate q = v_2q+1^2: only entry 2q+1 is read
-            const u64 wg = f_mul(ez, eq_at(L.trp, q));
-            P2a = f_mul(wg, V[2 * q + 1]);
-            M2 = f_mul(wg, eq_at(L.tr1, 2 * q + 1));
-        }
-        // PAIR: entry 2q carries the products with in1 = 2q (P2 and, with in1
-        // = in2 = 2q or in1 = 2q+1, in2 = 2q, M2 at 2q); FINAL: all at 2q+1
-        ulonglong2 *P2 = reinterpret_cast<ulonglong2 *>(L.P2), *P3 = reinterpret_cast<ulonglong2 *>(L.P3);
-        if (L.kind == W_F0_PAIR) {
-            P2[q] = make_ulonglong2(P2a, P2b);
-            P3[q] = make_ulonglong2(f_mul(v1, M2), 0);
-        } else {
-            P2[q] = make_ulonglong2(0, P2a);
-            P3[q] = make_ulonglong2(0, f_mul(v1, M2));
-        }
-        return;
-    }
-    if (w >= Sn) return;
     u64 P2 = 0, B2 = 0, A2 = 0, M2 = 0;
-    switch (L.kind) {
-    case W_SQUARE: {
-        const u64 wg = f_mul(ez, eq_at(L.trp, w));
-        P2 = f_mul(wg, V[w]);
-        M2 = f_mul(wg, eq_at(L.tr1, w));
-        break;
-    }
-    case W_TREE: {
-        if ((w & 1) == 0) {
-            const u64 wg = f_mul(ez, eq_at(L.trp, w >> 1));
-            P2 = wg;
-            B2 = f_mul(wg, V[w + 1]);
+    const u32 a0 = L.by1_off[w], a1 = L.by1_off[w + 1];
+    for (u32 q = a0; q < a1 && a1 - a0 <= BUILD_HEAVY; q++) {
+        const u32 g = L.by1_g[q];
+        const u64 wg = f_mul(ez, eq_at(L.trp, g));
+        if (L.type[g]) {
+            P2 = f_add(P2, f_mul(wg, V[L.in2[g]]));
         } else {
-            const u64 g = w >> 1;
-            const u64 wg = f_mul(ez, eq_at(L.trp, g));
-            A2 = f_mul(wg, eq_at(L.tr1, w - 1));
+            P2 = f_add(P2, wg);
+            B2 = f_add(B2, f_mul(wg, V[L.in2[g]]));
         }
-        break;
     }
-    case W_F0_FIRST: {
-        const u64 wm = f_mul(ez, eq_at(L.trp, 2 * w));      // MUL gate 2w
-        const u64 wa = f_mul(ez, eq_at(L.trp, 2 * w + 1));  // ADD gate 2w+1
-        const u64 e1 = eq_at(L.tr1, w);
-        P2 = f_add(f_mul(wm, V[w]), wa);
-        B2 = f_mul(wa, V[w]);
-        A2 = f_mul(wa, e1);
-        M2 = f_mul(wm, e1);
-        break;
-    }
-    case W_MATMULT: {
-        const u32 Lb = L.s / 3;
-        const u64 n = 1ull << Lb, msk = n - 1;
-        if (w < (1ull << (2 * Lb))) {
-            // gates with in1 = w: k = w mod n, i = w >> L, all j
-            const u64 k = w & msk, ii = w >> Lb;
-            u64 acc = 0;
-            for (u64 j = 0; j < n; j++) {
-                const u64 g = k | (j << Lb) | (ii << (2 * Lb));
-                const u64 bidx = (1ull << (2 * Lb)) | (k << Lb) | j;
-                acc = f_add(acc, f_mul(eq_at(L.trp, g), V[bidx]));
-            }
-            P2 = f_mul(ez, acc);
-        } else {
-            // gates with in2 = w: j = w mod n, k = (w >> L) mod n, all i
-            const u64 j = w & msk, k = (w >> Lb) & msk;
-            u64 acc = 0;
-            for (u64 ii = 0; ii < n; ii++) {
-                const u64 g = k | (j << Lb) | (ii << (2 * Lb));
-                acc = f_add(acc, f_mul(eq_at(L.trp, g), eq_at(L.tr1, (ii << Lb) | k)));
-            }
-            M2 = f_mul(ez, acc);
-        }
-        break;
-    }
-    default: {  // explicit wiring, gates grouped by in1 and by in2
-        // an entry read by more than BUILD_HEAVY gates is summed by a whole
-        // CTA afterwards (k_build_heavy), which adds to what is written here
-        const u32 a0 = L.by1_off[w], a1 = L.by1_off[w + 1];
-        for (u32 q = a0; q < a1 && a1 - a0 <= BUILD_HEAVY; q++) {
-            const u32 g = L.by1_g[q];
-            const u64 wg = f_mul(ez, eq_at(L.trp, g));
-            if (L.type[g]) {
-                P2 = f_add(P2, f_mul(wg, V[L.in2[g]]));
-            } else {
-                P2 = f_add(P2, wg);
-                B2 = f_add(B2, f_mul(wg, V[L.in2[g]]));
-            }
-        }
-        const u32 b0 = L.by2_off[w], b1 = L.by2_off[w + 1];
-        for (u32 q = b0; q < b1 && b1 - b0 <= BUILD_HEAVY; q++) {
-            const u32 g = L.by2_g[q];
-            const u64 ug = f_mul(f_mul(ez, eq_at(L.trp, g)), eq_at(L.tr1, L.in1[g]));
-            if (L.type[g]) M2 = f_add(M2, ug);
-            else A2 = f_add(A2, ug);
-        }
-        break;
-    }
+    const u32 b0 = L.by2_off[w], b1 = L.by2_off[w + 1];
+    for (u32 q = b0; q < b1 && b1 - b0 <= BUILD_HEAVY; q++) {
+        const u32 g = L.by2_g[q];
+        const u64 ug = f_mul(f_mul(ez, eq_at(L.trp, g)), eq_at(L.tr1, L.in1[g]));
+        if (L.type[g]) M2 = f_add(M2, ug);
+        else A2 = f_add(A2, ug);
     }
     L.P2[w] = P2;
     L.P3[w] = f_add(A2, f_mul(v1, M2));
@@ -603,6 +516,48 @@ __global__ void __launch_bounds__(256) k_build23(const Globals *Gs, const BuildI
         L.B2[w] = B2;
         L.B3[w] = f_mul(v1, A2);
     }
+}
+
+// Phase 2 of a MATMULT layer: the gates with in1 = (k, i) are (k, j, i) for
+// every j, so P2[(k, i)] = sum_j w V[(j, k, 1)] = u[k] ei[i] with
+//   u[k] = eq(z, r_P) eq(r_P over k, k) sum_j eq(r_P over j, j) V[n^2 + k n + j],
+//   ei[i] = eq(r_P over i, i):
+// n products for each of n rows, where a sum of its own per entry took n^3.  A
+// warp a row; the first item also writes ei.
+__global__ void __launch_bounds__(256) k_mm_tables(const Globals *Gs, const BuildItem *items)
+{
+    __shared__ u64 ej[1024];
+    const BuildItem bi = items[blockIdx.x];
+    const Globals &G = Gs[bi.circ];
+    const LayerDev &L = G.layers[bi.layer];
+    const u32 Lb = L.s / 3, n = 1u << Lb, lane = threadIdx.x & 31;
+    const u64 *rP = G.chal + L.chal_off;
+    auto eq_bits = [&](u32 off, u32 x) {
+        u64 v = 1;
+#pragma unroll 1
+        for (u32 m = 0; m < Lb; m++) v = f_mul(v, ((x >> m) & 1) ? rP[off + m] : f_sub(1, rP[off + m]));
+        return v;
+    };
+#pragma unroll 1
+    for (u32 x = threadIdx.x; x < n; x += 256) {
+        ej[x] = eq_bits(Lb, x);
+        if (bi.block == 0) L.mei[x] = eq_bits(2 * Lb, x);
+    }
+    __syncthreads();
+    const u32 k = bi.block * MM_ROWS + (threadIdx.x >> 5);
+    if (k >= n) return;
+    const u64 *row = L.Vn + ((u64)n << Lb) + ((u64)k << Lb);
+    acc128 a;  // at most 32 products a lane
+    acc_zero(a);
+#pragma unroll 4
+    for (u32 j = lane; j < n; j += 32) mac(a, ej[j], row[j]);
+    const u64 s = warp_wsum(acc_red(a));
+    if (lane == 0) L.mu[k] = f_mul(f_mul(G.scal[SCAL_EQZRP(bi.layer)], eq_bits(0, k)), wcanon(s));
+}
+
+void launch_mm_tables(const Globals *Gs, const BuildItem *items, int nitems, cudaStream_t st)
+{
+    if (nitems > 0) k_mm_tables<<<nitems, 256, 0, st>>>(Gs, items);
 }
 
 void launch_build23(const Globals *Gs, const BuildItem *items, int nitems, cudaStream_t st)

@@ -11,15 +11,14 @@
 //      g_j(t) = kappa_j L_j(t) h_j(t),  h_j(t) = sum_y E_j(y) V_j(t, y),
 //    with kappa_j = sigma prod_{m<j} L_m(r_m), E_j(y) = prod_{m>j} L_m(y_m) and
 //    V_j the value table folded with r_0..r_{j-1}; h_j is linear in t, so only
-//    h_j(0), h_j(1) are summed.  Per pair of entries: two multiply-adds and one
-//    fold.  Used for phase 1 of every layer (P = eq(z_i, .)) and for phase 3 of
-//    TREE and SQUARE layers.
+//    h_j(0), h_j(1) are summed.  Used for phase 1 of every layer (P = eq(z_i,
+//    .)), phase 2 of TREE layers and phase 3 of every structured kind.
 //  * general (GEN): P, V, B are tables folded every round; the message needs
 //    P(t)V(t) + B(t) at t = 0, 1, 2.  Chunks sum the values at 0 and 1 and the
 //    leading coefficient (P1 - P0)(V1 - V0) of each pair, which shares its
 //    differences with the folds; k_final turns the three sums into the value
-//    at 2.  The first wave builds P and B from the wiring on the fly (SQUARE,
-//    TREE phase 2) or reads tables built by k_build23.
+//    at 2.  The first wave forms P and B from the wiring on the fly (phase 2 of
+//    SQUARE, F0 and MATMULT layers) or reads tables built by k_build23.
 //
 // Arithmetic is lazy: table values stay in W = [0, 2^61 + 8), products
 // accumulate exactly in 128 bits and are reduced once per round per thread;
@@ -89,19 +88,15 @@ __device__ __forceinline__ u64 warp_sum32(u64 (&v)[32])
 // --------------------------------------------------------------------------------
 
 #define WV_NT 128
-#define PR_SUB 16  // PROD runs of 16 entries (rounds 0..3 per run)
 
 struct ProdSmem {
-    u32 r[32][2];
-    u64 Q[64];
-    u64 E[256];
-    u64 lvl[WV_NT / 32];
-    u64 w[WV_NT / 32][32];
-    u64 echunk;
+    u64 u[8][1 << PR_C];       // row groups' column sums
+    u64 f[16][(1 << PR_R) + 1];  // column groups' row sums
+    u64 U[1 << PR_C], F[1 << PR_R];
 };
 
 struct GenSmem {
-    u32 r[32][2];
+    u64 r[32];
     u64 lvl[3][WV_NT / 32];
     u64 w[WV_NT / 32][40];
     u64 hs[9][WV_NT];  // per-thread sums of in-register rounds 2..4 (kept out of registers)
@@ -112,7 +107,7 @@ struct GenSmem {
 #define LN_BUFB 1024  // wave's first level is 64 pairs x <= 32 coefficients
 
 struct LineSmem {
-    u32 la[32][2], lb[32][2];  // limbs of a_k and b_k for the wave's coordinates
+    u64 la[32], lb[32];  // a_k and b_k for the wave's coordinates
     u64 bufA[LN_BUFA];
     u64 bufB[LN_BUFB];
 };
@@ -123,12 +118,23 @@ union WaveSmem {
     LineSmem line;
 };
 
+extern __shared__ __align__(16) unsigned char wv_dyn[];  // a WaveSmem
+
 // Load of a wave's input.  A first wave's input (layer values, or tables built
 // by an earlier launch) is read-only for the whole launch and goes through
 // L1, where the prefetch of the next run lands; a later wave's input is
 // written by other CTAs of this launch and is read through L2.
 __device__ __forceinline__ ulonglong2 ld_in(const ulonglong2 *p, bool ext) { return ext ? __ldg(p) : __ldcg(p); }
 __device__ __forceinline__ u64 ld_in(const u64 *p, bool ext) { return ext ? __ldg(p) : __ldcg(p); }
+
+// A load that stays where it is written: weights that a loop needs in every
+// pass and that cost more as registers kept through it than as L1 hits.
+__device__ __forceinline__ ulonglong2 ld_again(const ulonglong2 *p)
+{
+    ulonglong2 t;
+    asm volatile("ld.global.nc.v2.u64 {%0, %1}, [%2];" : "=l"(t.x), "=l"(t.y) : "l"(p));
+    return t;
+}
 
 // Bring the line holding p into L1 ahead of its load (no register cost).
 __device__ __forceinline__ void prefetch_l1(const void *p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
@@ -140,210 +146,175 @@ __device__ __forceinline__ u64 cta_sum4(const u64 *a, const u64 *b, const u64 *c
 }
 
 // ---- PROD -----------------------------------------------------------------------
+//
+// Every message sum and the fold of a product-weighted chunk are linear in
+// its entries, with weights that are products over the coordinates.  So a
+// chunk of 2^kr rows of 2^7 columns is read once, with two multiply-adds
+// per entry: U[x] = sum_row roww[row] V[row, x] holds all that the rounds of
+// the column coordinates need (their sums over the rows are weighted alike),
+// F[row] = sum_x colw[x] V[row, x] is the table folded by those rounds, on
+// which the row coordinates' rounds run.  The rounds of either vector are
+// then independent sums too (vec_rounds), one step instead of a chain of
+// folds.  Folding round by round took three products an entry, a reduction
+// and a fold per pair, and a chain of up to 13 dependent rounds.
 
-// Sum over the lanes l = 0 mod 2^(kk+1) of a warp (the lanes holding a
-// contribution in cross round kk; the others hold 0), written by lane 0.
-__device__ __forceinline__ void prod_round_sum(u64 c0, u64 c1, u32 kk, u64 *out)
+// The sums of every round of a vector of 2^kk entries in shared memory (kk <=
+// 7): thread 16 j + p takes round j's pairs p, p + 16, ..; w: its weights.
+// Afterwards lanes p = 0..7 hold the round's sum at 0 and lanes 8..15 that at 1.
+__device__ __forceinline__ u64 vec_rounds(const u64 *v, u32 kk, const u64 (&w)[4])
 {
+    const u32 j = threadIdx.x >> 4, p = threadIdx.x & 15;
+    acc128 a0, a1;
+    acc_zero(a0);
+    acc_zero(a1);
+    if (j < kk) {
+        const u32 half = 1u << (kk - 1), bit = 1u << j;
 #pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) {
-        if ((u32)o < (2u << kk)) break;
-        c0 = wred(c0 + __shfl_xor_sync(0xffffffffu, c0, o));
-        c1 = wred(c1 + __shfl_xor_sync(0xffffffffu, c1, o));
-    }
-    if ((threadIdx.x & 31) == 0) {
-        out[0] = c0;
-        out[1] = c1;
-    }
-}
-
-// Rounds off.. of a product-weighted chunk across threads.  Thread t holds
-// level value t (t < na); a round pairs values 2y and 2y+1, which sit in the
-// threads t = y 2^(kk+1) and t + 2^kk, and the first of them keeps the folded
-// value, so rounds stay inside a warp for kk < 5 (shuffles) and continue in
-// warp 0 after one exchange through shared memory.  The active thread of a
-// pair contributes E_k(y) u0 and E_k(y) u1; the per-warp sums of round k go
-// to sm.w[warp][2k..2k+1] (CTA-level rounds: warp 0's row, zeros elsewhere).
-__device__ __forceinline__ void prod_cross(u64 uv, u32 off, u32 tid, u32 na, u32 nr, ProdSmem &sm, u32 eoff0)
-{
-    const u32 lane = tid & 31, warp = tid >> 5;
-    // rolled: one copy of the round body keeps the kernel small
-#pragma unroll 1
-    for (u32 kk = 0; kk < 5; kk++) {
-        const u32 k = off + kk;
-        if (k < nr) {  // uniform
-            const u64 u1 = __shfl_down_sync(0xffffffffu, uv, 1u << kk);
-            u64 c0 = 0, c1 = 0;
-            if ((tid & ((2u << kk) - 1)) == 0 && tid < na) {
-                const u32 y = tid >> (kk + 1);
-                const u64 w = sm.E[eoff0 - (1u << (nr - k)) + y];
-                c0 = wmul(w, uv);
-                c1 = wmul(w, u1);
-                uv = wfold(uv, u1, sm.r[k][0], sm.r[k][1]);
-            }
-            prod_round_sum(c0, c1, kk, &sm.w[warp][2 * k]);
-        }
-    }
-    if (lane == 0) {
-        sm.lvl[warp] = uv;
-        for (u32 k = off + 5; k < nr && k < off + 7; k++)
-            if (warp) sm.w[warp][2 * k] = sm.w[warp][2 * k + 1] = 0;
-    }
-    __syncthreads();
-    if (off + 5 < nr && warp == 0) {
-        uv = (lane < WV_NT / 32) ? sm.lvl[lane] : 0;
-        for (u32 kk = 5; kk < 7; kk++) {
-            const u32 k = off + kk;
-            if (k < nr) {
-                const u64 u1 = __shfl_down_sync(0xffffffffu, uv, 1u << (kk - 5));
-                const u32 t = lane << 5;  // the thread index this lane stands for
-                u64 c0 = 0, c1 = 0;
-                if ((t & ((2u << kk) - 1)) == 0 && t < na) {
-                    const u32 y = t >> (kk + 1);
-                    const u64 w = sm.E[eoff0 - (1u << (nr - k)) + y];
-                    c0 = wmul(w, uv);
-                    c1 = wmul(w, u1);
-                    uv = wfold(uv, u1, sm.r[k][0], sm.r[k][1]);
-                }
-                prod_round_sum(c0, c1, kk - 5, &sm.w[0][2 * k]);
+        for (u32 i = 0; i < 4; i++) {
+            const u32 y = p + 16 * i;
+            if (y < half) {
+                const u32 x = ((y & ~(bit - 1)) << 1) | (y & (bit - 1));
+                mac(a0, w[i], v[x]);
+                mac(a1, w[i], v[x | bit]);
             }
         }
-        if (lane == 0) sm.lvl[0] = uv;
     }
+    // sixteen lanes' sums; the lanes' halves part after the first exchange
+    const bool up = (p & 8) != 0;
+    const u64 h0 = acc_red7(a0), h1 = acc_red7(a1);
+    u64 h = (up ? h1 : h0) + __shfl_xor_sync(0xffffffffu, up ? h0 : h1, 8);
+    h += __shfl_xor_sync(0xffffffffu, h, 4);
+    h = wred(h);
+    h += __shfl_xor_sync(0xffffffffu, h, 2);
+    h += __shfl_xor_sync(0xffffffffu, h, 1);
+    return wred(h);
 }
 
-// Rounds 0..3 of one run of 16 entries (run `sub` of the thread's 2^e):
-// pair weights Q_k(q), q = pair index + (sub << (3 - k)).
-__device__ __forceinline__ u64 prod_run16(u64 (&u)[16], u32 sub, u32 e, const ProdSmem &sm, u64 (&h)[12])
+// A thread's weights for vec_rounds.
+__device__ __forceinline__ void vec_weights(const u64 *T, u32 kk, bool use, u64 (&w)[4])
 {
 #pragma unroll
-    for (int k = 0; k < 4; k++) {
-        acc128 a0, a1, b0, b1;  // two chains per value for instruction-level parallelism
-        acc_zero(a0);
-        acc_zero(a1);
-        acc_zero(b0);
-        acc_zero(b1);
-        const u32 rr0 = sm.r[k][0], rr1 = sm.r[k][1];
-        const u32 qoff = (1u << e) - (1u << (e - k)) + (sub << (3 - k));
-#pragma unroll
-        for (int q = 0; q < (8 >> k); q++) {
-            const u64 w = sm.Q[qoff + q];
-            const u64 u0 = u[2 * q], u1 = u[2 * q + 1];
-            if (q & 1) {
-                mac(b0, w, u0);
-                mac(b1, w, u1);
-            } else {
-                mac(a0, w, u0);
-                mac(a1, w, u1);
-            }
-            u[q] = wfold(u0, u1, rr0, rr1);
-        }
-        h[2 * k] = wred(h[2 * k] + acc_red(a0) + acc_red(b0));
-        h[2 * k + 1] = wred(h[2 * k + 1] + acc_red(a1) + acc_red(b1));
-    }
-    return u[0];
+    for (u32 i = 0; i < 4; i++)
+        w[i] = (use && threadIdx.x < 16 * kk && i < vec_slots(kk)) ? __ldg(T + i * 16 * kk + threadIdx.x) : 0;
 }
 
-// In-register rounds for e in 4..6: runs of 16, then rounds 4 and 5 on the
-// runs' folded values.
-__device__ __forceinline__ u64 prod_regs_runs(const u64 *src, u32 e, bool ext, const ProdSmem &sm, u64 (&h)[12])
+// One chunk of a PROD wave (each kind is a function of its own: its registers
+// are allocated without those of the others, and there is one copy of its code).
+__device__ __noinline__ void prod_chunk(const ProdWave &W, u32 chunk)
 {
-    const u32 nruns = 1u << (e - 4);
-    const u32 q4 = (1u << e) - (1u << (e - 4)), q5 = (1u << e) - 2;
-    u64 f0 = 0, g0 = 0, uv = 0;
-    // a rolled loop keeps the kernel small (instruction-cache bound when unrolled)
-#pragma unroll 1
-    for (u32 sub = 0; sub < nruns; sub++) {
-        if (sub + 1 < nruns) prefetch_l1(src + (sub + 1) * PR_SUB);
-        u64 u[16];
-        const ulonglong2 *sv = reinterpret_cast<const ulonglong2 *>(src + sub * PR_SUB);
-#pragma unroll
-        for (int q = 0; q < 8; q++) {
-            const ulonglong2 t = ld_in(sv + q, ext);
-            u[2 * q] = t.x;
-            u[2 * q + 1] = t.y;
-        }
-        const u64 fs = prod_run16(u, sub, e, sm, h);
-        if (nruns == 1) {
-            uv = fs;
-        } else if (sub & 1) {
-            const u64 w = sm.Q[q4 + (sub >> 1)];
-            h[8] = wred(h[8] + wmul(w, f0));
-            h[9] = wred(h[9] + wmul(w, fs));
-            const u64 g = wfold(f0, fs, sm.r[4][0], sm.r[4][1]);
-            if (nruns == 2) {
-                uv = g;
-            } else if (sub == 1) {
-                g0 = g;
-            } else {
-                const u64 w5 = sm.Q[q5];
-                h[10] = wmul(w5, g0);
-                h[11] = wmul(w5, g);
-                uv = wfold(g0, g, sm.r[5][0], sm.r[5][1]);
-            }
-        } else {
-            f0 = fs;
-        }
-    }
-    return uv;
-}
-
-// One chunk of a PROD wave.
-__device__ void prod_chunk(const Globals &G, const ProdWave &W, u32 chunk, ProdSmem &sm)
-{
-    const u32 tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const u32 nr = W.nr, e = W.e;
-    const u32 na = 1u << (nr - e);
-    const u64 base = (u64)chunk << nr;
-    if (tid < nr) limbs31(G.chal[W.chal_off + tid], sm.r[tid][0], sm.r[tid][1]);
+    ProdSmem &sm = reinterpret_cast<WaveSmem *>(wv_dyn)->prod;
+    const u32 tid = threadIdx.x;
+    const u32 nr = W.nr, kc = W.kc, kr = W.kr, nchunks = W.nchunks;
+    const bool ext = W.r0 == 0, odd = (W.flags & WF_ODD) != 0;
     const u64 *blk = W.wblk;
-    const u32 qsize = (1u << e) - 1;
-    const u32 kb = e ? e - 1 : 0;
-    const u32 esize = (1u << (nr - kb)) - 1;
-    if (tid < qsize) sm.Q[tid] = blk[tid];
-    for (u32 k = tid; k < esize; k += WV_NT) sm.E[k] = blk[qsize + k];
-    if (tid == 0) {
-        const u64 *olo = blk + qsize + esize;
-        const u64 *ohi = olo + (1u << W.ho);
-        sm.echunk = f_mul(olo[chunk & ((1u << W.ho) - 1)], ohi[chunk >> W.ho]);
-    }
-    __syncthreads();
-    const u32 eoff0 = 1u << (nr - kb);
-    u64 uv = 0;
-    if (e > 0) {
-        u64 h[12];
+    const u64 *in = W.in + ((u64)chunk << (odd ? nr + 1 : nr));
+    u64 wc[4], wr[4], ea, eb, el;
+    auto weights = [&]() {
+        vec_weights(blk + pw_tcol(kr), kc, true, wc);
+        vec_weights(blk + pw_trow(kc, kr), kr, kr != 0, wr);
+        const u64 *olo = blk + pw_outer(kc, kr);  // weight of the coordinates beyond the chunk
+        ea = __ldg(olo + (chunk & ((1u << W.ho) - 1)));
+        eb = __ldg(olo + (1u << W.ho) + (chunk >> W.ho));
+        el = __ldg(blk + pw_last(kc, kr) + (kr ? 2 : 0) + ((tid >> 3) & 1));  // fold factor of the last coordinate
+    };
+    if (kr == 0) {
+        weights();
+        if (tid < (1u << kc)) sm.U[tid] = ld_in(in + (odd ? 2 * tid + 1 : tid), ext);
+        __syncthreads();
+    } else {
+        // columns 2c + 32 q, + 1 of rows rg, rg + 8, ..
+        const u32 c = tid & 15, rg = tid >> 4, nrow = 1u << kr;
+        const u64 *roww = blk + pw_roww(kr);
+        const ulonglong2 *src = reinterpret_cast<const ulonglong2 *>(in);
+        auto load = [&](u32 row, ulonglong2 (&t)[4]) {
 #pragma unroll
-        for (int i = 0; i < 12; i++) h[i] = 0;
-        if (tid < na) {
-            const u64 *src = W.in + base + ((u64)tid << e);
-            uv = prod_regs_runs(src, e, W.r0 == 0, sm, h);
-            const u64 T = sm.E[tid];  // E_{e-1}(tid): weight of the chunk bits above the thread's run
+            for (int q = 0; q < 4; q++) {
+                if (odd) {
+                    const ulonglong2 *s2 = src + 2 * (row * 64 + 16 * q + c);
+                    t[q] = make_ulonglong2(ld_in(s2, ext).y, ld_in(s2 + 1, ext).y);
+                } else {
+                    t[q] = ld_in(src + row * 64 + 16 * q + c, ext);
+                }
+            }
+        };
+        acc128 u[8];
 #pragma unroll
-            for (int i = 0; i < 12; i++) h[i] = wmul(T, h[i]);
+        for (int q = 0; q < 8; q++) acc_zero(u[q]);
+        ulonglong2 v[4];
+        u64 rw = 0;
+        if (rg < nrow) {
+            rw = __ldg(roww + rg);
+            load(rg, v);
         }
-        u64 h16[16];
+#pragma unroll 1
+        for (u32 row = rg; row < nrow; row += 8) {
+            ulonglong2 n[4];  // the next row's entries on their way during this row's products
+            u64 rn = 0;
+            const bool more = row + 8 < nrow;
+            if (more) {
+                rn = __ldg(roww + row + 8);
+                load(row + 8, n);
+            }
+            acc128 f0, f1;
+            acc_zero(f0);
+            acc_zero(f1);
 #pragma unroll
-        for (int i = 0; i < 16; i++) h16[i] = (i < 12) ? h[i] : 0;
-        const u64 s = warp_sum16(h16);
-        if ((lane & 1) == 0 && (lane >> 1) < 2 * e) sm.w[warp][lane >> 1] = s;
-    } else if (tid < na) {
-        uv = ld_in(W.in + base + tid, W.r0 == 0);
+            for (int q = 0; q < 4; q++) {
+                const ulonglong2 cw = ld_again(reinterpret_cast<const ulonglong2 *>(blk) + c + 16 * q);
+                mac(f0, cw.x, v[q].x);
+                mac(f1, cw.y, v[q].y);
+                mac(u[2 * q], rw, v[q].x);
+                mac(u[2 * q + 1], rw, v[q].y);
+            }
+            sm.f[c][row] = wred(acc_red7(f0) + acc_red7(f1));
+            if (more) {
+                rw = rn;
+#pragma unroll
+                for (int q = 0; q < 4; q++) v[q] = n[q];
+            }
+        }
+#pragma unroll
+        for (int q = 0; q < 4; q++)
+            *reinterpret_cast<ulonglong2 *>(&sm.u[rg][2 * c + 32 * q]) =
+                make_ulonglong2(acc_red(u[2 * q]), acc_red(u[2 * q + 1]));
+        weights();
+        __syncthreads();
+        {
+            const u64 a = wred(sm.u[0][tid] + sm.u[1][tid] + sm.u[2][tid] + sm.u[3][tid]);
+            const u64 b = wred(sm.u[4][tid] + sm.u[5][tid] + sm.u[6][tid] + sm.u[7][tid]);
+            sm.U[tid] = wred(a + b);
+            const u32 row = tid >> 1, g = (tid & 1) * 8;  // a row's sixteen column groups, eight a thread
+            u64 f = 0;
+            if (row < nrow) {
+                const u64 x = wred(sm.f[g][row] + sm.f[g + 1][row] + sm.f[g + 2][row] + sm.f[g + 3][row]);
+                f = wred(x + wred(sm.f[g + 4][row] + sm.f[g + 5][row] + sm.f[g + 6][row] + sm.f[g + 7][row]));
+            }
+            f = wred(f + __shfl_xor_sync(0xffffffffu, f, 1));
+            if ((tid & 1) == 0 && row < nrow) sm.F[row] = f;
+        }
+        __syncthreads();
     }
-    prod_cross(uv, e, tid, na, nr, sm, eoff0);
-    __syncthreads();
-    if (tid < 2 * nr) {
-        const u64 sum = wred(sm.w[0][tid] + sm.w[1][tid] + sm.w[2][tid] + sm.w[3][tid]);
-        const u32 k = tid >> 1, t = tid & 1;
-        W.part[((u64)k * W.nchunks + chunk) * 2 + t] = wmul(sum, sm.echunk);
+    const u32 j = tid >> 4, t = (tid >> 3) & 1;
+    const bool writer = (tid & 7) == 0;
+    const u64 ech = f_mul(ea, eb);
+    u64 h = vec_rounds(sm.U, kc, wc);
+    if (writer && j < kc) W.part[((u64)j * nchunks + chunk) * 2 + t] = wmul(h, ech);
+    if (kr) {
+        h = vec_rounds(sm.F, kr, wr);
+        if (writer && j < kr) W.part[((u64)(kc + j) * nchunks + chunk) * 2 + t] = wmul(h, ech);
     }
-    if (!(W.flags & WF_LAST) && tid == 0) W.out[chunk] = sm.lvl[0];
+    if (!(W.flags & WF_LAST)) {
+        // the chunk's value for the next wave: the last round's sums, folded
+        const u64 x = wmul(h, el), y = wred(x + __shfl_xor_sync(0xffffffffu, x, 8));
+        if (tid == 16 * ((kr ? kr : kc) - 1)) W.out[chunk] = y;
+    }
 }
 
 // ---- GEN ------------------------------------------------------------------------
 
 // N consecutive entries of a GEN wave's P, V, B tables at x0 (tables built
-// by k_build23, or the previous wave's outputs; the first waves of SQUARE and
-// TREE phase 2 form P and B themselves: sq2_run, tree2_run).
+// by k_build23, or the previous wave's outputs; first waves whose tables follow
+// from the wiring form P and B themselves: gen_source, bil_run).
 template <int N>
 __device__ __forceinline__ void gen_load(const GenWave &W, u64 x0, bool hasB, u64 (&p)[N], u64 (&v)[N], u64 (&b)[N])
 {
@@ -379,196 +350,220 @@ __device__ __forceinline__ void gen_load(const GenWave &W, u64 x0, bool hasB, u6
 // One general pair: the message's values at t = 0, 1 (c0, c1) and its
 // leading coefficient c2 = (P1 - P0)(V1 - V0), from which the value at 2 is
 // 2 c1 - c0 + 2 c2 (B is linear in t); then the folds, which share the
-// differences P1 - P0, V1 - V0, B1 - B0 (lazy, below 2^62.6).
-__device__ __forceinline__ void gen_pair(u64 p0, u64 p1, u64 v0, u64 v1, u64 b0, u64 b1, u32 rr0, u32 rr1,
-                                         u64 &c0, u64 &c1, u64 &c2, u64 &pn, u64 &vn, u64 &bn)
+// differences P1 - P0, V1 - V0 (lazy, below 1.5 2^62).  B is zero without hasB
+// (uniform).
+__device__ __forceinline__ void gen_pair(bool hasB, u64 p0, u64 p1, u64 v0, u64 v1, u64 b0, u64 b1, u64 r, u64 &c0, u64 &c1,
+                                         u64 &c2, u64 &pn, u64 &vn, u64 &bn)
 {
-    const u64 dp = p1 + (2 * FP_P) - p0, dv = v1 + (2 * FP_P) - v0, db = b1 + (2 * FP_P) - b0;
-    c0 = wred(wmul(p0, v0) + b0);
-    c1 = wred(wmul(p1, v1) + b1);
+    const u64 dp = p1 + (2 * FP_P) - p0, dv = v1 + (2 * FP_P) - v0;
+    c0 = wmul(p0, v0);
+    c1 = wmul(p1, v1);
     c2 = wmul(wred(dp), wred(dv));
-    pn = wlin1(p0, dp, rr0, rr1);
-    vn = wlin1(v0, dv, rr0, rr1);
-    bn = wlin1(b0, db, rr0, rr1);
+    pn = wlin1(p0, dp, r);
+    vn = wlin1(v0, dv, r);
+    if (hasB) {
+        c0 = wred(c0 + b0);
+        c1 = wred(c1 + b1);
+        bn = wfold(b0, b1, r);
+    }
 }
 
 // Round k on two folded triples held by one thread, summed into the
 // thread's shared-memory slots hs[3j..3j+2].
-__device__ __forceinline__ void gen_pair_acc(u64 p0, u64 p1, u64 v0, u64 v1, u64 b0, u64 b1, u32 rr0, u32 rr1,
-                                             GenSmem &sm, u32 j, u64 &pn, u64 &vn, u64 &bn)
+__device__ __forceinline__ void gen_pair_acc(bool hasB, u64 p0, u64 p1, u64 v0, u64 v1, u64 b0, u64 b1, u64 r, GenSmem &sm,
+                                             u32 j, u64 &pn, u64 &vn, u64 &bn)
 {
     u64 c0, c1, c2;
-    gen_pair(p0, p1, v0, v1, b0, b1, rr0, rr1, c0, c1, c2, pn, vn, bn);
+    gen_pair(hasB, p0, p1, v0, v1, b0, b1, r, c0, c1, c2, pn, vn, bn);
     const u32 t = threadIdx.x;
     sm.hs[3 * j][t] = wred(sm.hs[3 * j][t] + c0);
     sm.hs[3 * j + 1][t] = wred(sm.hs[3 * j + 1][t] + c1);
     sm.hs[3 * j + 2][t] = wred(sm.hs[3 * j + 2][t] + c2);
 }
 
-// Rounds 0..R-1 of N = 2^R entries held by one thread; adds to h[0..3R) and
-// leaves the folded values in p[0], v[0], b[0].
-template <int R>
-__device__ __forceinline__ void gen_regs(u64 (&p)[1 << R], u64 (&v)[1 << R], u64 (&b)[1 << R], const GenSmem &sm,
-                                         u64 (&h)[15])
+// A pair of a run, its message sums into the exact accumulators a[0..2] (a
+// thread's runs add at most 16 products to each, so they are reduced once at
+// the end and not in every run); the folds to p, v.
+__device__ __forceinline__ void gen_pair_run(u64 p0, u64 p1, u64 v0, u64 v1, u64 r, acc128 *a, u64 &p, u64 &v)
 {
-#pragma unroll
-    for (int k = 0; k < R; k++) {
-        acc128 a0, a1, a2;
-        acc_zero(a0);
-        acc_zero(a1);
-        acc_zero(a2);
-        const u32 rr0 = sm.r[k][0], rr1 = sm.r[k][1];
-#pragma unroll
-        for (int q = 0; q < (1 << (R - k - 1)); q++) {
-            const u64 p0 = p[2 * q], p1 = p[2 * q + 1], v0 = v[2 * q], v1 = v[2 * q + 1];
-            const u64 b0 = b[2 * q], b1 = b[2 * q + 1];
-            const u64 dp = p1 + (2 * FP_P) - p0, dv = v1 + (2 * FP_P) - v0, db = b1 + (2 * FP_P) - b0;
-            mac(a0, p0, v0);
-            mac(a1, p1, v1);
-            mac(a2, wred(dp), wred(dv));  // leading coefficient (see gen_pair)
-            acc_add(a0, b0);
-            acc_add(a1, b1);
-            p[q] = wlin1(p0, dp, rr0, rr1);
-            v[q] = wlin1(v0, dv, rr0, rr1);
-            b[q] = wlin1(b0, db, rr0, rr1);
-        }
-        h[3 * k] = wred(h[3 * k] + acc_red(a0));
-        h[3 * k + 1] = wred(h[3 * k + 1] + acc_red(a1));
-        h[3 * k + 2] = wred(h[3 * k + 2] + acc_red(a2));
+    const u64 dp = p1 + (2 * FP_P) - p0, dv = v1 + (2 * FP_P) - v0;
+    mac(a[0], p0, v0);
+    mac(a[1], p1, v1);
+    mac(a[2], wred(dp), wred(dv));  // leading coefficient (see gen_pair)
+    p = wlin1(p0, dp, r);
+    v = wlin1(v0, dv, r);
+}
+
+// Rounds 0 and 1 of 4 entries held by one thread: sums into a[0..2], a[3..5],
+// the folded values to pn, vn, bn (HASB: with B's terms).
+template <bool HASB>
+__device__ __forceinline__ void gen_run(const u64 (&p)[4], const u64 (&v)[4], const u64 (&b)[4], const GenSmem &sm,
+                                        acc128 (&a)[6], u64 &pn, u64 &vn, u64 &bn)
+{
+    const u64 r0 = sm.r[0], r1 = sm.r[1];
+    u64 q0, q1, u0, u1;
+    gen_pair_run(p[0], p[1], v[0], v[1], r0, a, q0, u0);
+    gen_pair_run(p[2], p[3], v[2], v[3], r0, a, q1, u1);
+    gen_pair_run(q0, q1, u0, u1, r1, a + 3, pn, vn);
+    if (HASB) {
+        acc_add(a[0], b[0] + b[2]);
+        acc_add(a[1], b[1] + b[3]);
+        const u64 c0 = wfold(b[0], b[1], r0), c1 = wfold(b[2], b[3], r0);
+        acc_add(a[3], c0);
+        acc_add(a[4], c1);
+        bn = wfold(c0, c1, r1);
     }
 }
 
-// Rounds 0 and 1 of the first wave of a TREE phase-2 instance on the 4
-// entries at x0 (gates g = x0/2 and x0/2 + 1 of layer i).  P and B vanish at
-// odd entries and P[2g] = eq(r_P, g) = w, B[2g] = w V[2g+1], so round 0 needs
-// per gate only w: its message is c0 = sum w (v0 + v1), c1 = 0 and leading
-// coefficient c2 = -sum w (v1 - v0), and the folds are P' = (1 - r_0) w,
-// V' = V folded, B' = (1 - r_0) w v1.  The common factor 1 - r_0 of P' and B'
-// is left out here: it multiplies the message of every later round of the
-// instance and is applied in the final reduction.  h[2] collects the c2 sum
-// with its sign flipped (restored by the caller).
-__device__ __forceinline__ void tree2_run(const Globals &G, const GenWave &W, u64 x0, const GenSmem &sm,
-                                          u64 (&h)[15], u64 &pn, u64 &vn, u64 &bn)
+// P (and B, for FIRST2) of one entry x of a first wave whose tables follow
+// from the wiring (GS_*); v = V[x], ve = V[x with bit 0 cleared]// (.x: P, .y: B).
+__device__ __noinline__ ulonglong2 gen_source(const Globals &G, const GenWave &W, u64 x, u64 v, u64 ve)
 {
-    const ulonglong2 *sv = reinterpret_cast<const ulonglong2 *>(W.inV + x0);
-    const ulonglong2 va = __ldg(sv), vb = __ldg(sv + 1);
-    const EqTab &T = G.layers[W.layer].trp;
-    const u64 wa = eq_at(T, x0 >> 1), wb = eq_at(T, (x0 >> 1) + 1);
-    const u64 da = va.y + (2 * FP_P) - va.x, db = vb.y + (2 * FP_P) - vb.x;  // below 2^62.6
-    acc128 s, t;
-    acc_zero(s);
-    acc_zero(t);
-    mac(s, wa, va.x + va.y);  // operands below 2^62 + 16
-    mac(s, wb, vb.x + vb.y);
-    mac(t, wa, da);
-    mac(t, wb, db);
-    h[0] = wred(h[0] + acc_red(s));
-    h[2] = wred(h[2] + acc_red(t));
-    const u32 a0 = sm.r[0][0], a1 = sm.r[0][1];
-    const u64 v0 = wlin1(va.x, da, a0, a1), v1 = wlin1(vb.x, db, a0, a1);
-    const u64 b0 = wmul(wa, va.y), b1 = wmul(wb, vb.y);
-    u64 c0, c1, c2;
-    gen_pair(wa, wb, v0, v1, b0, b1, sm.r[1][0], sm.r[1][1], c0, c1, c2, pn, vn, bn);
-    h[3] = wred(h[3] + c0);
-    h[4] = wred(h[4] + c1);
-    h[5] = wred(h[5] + c2);
-}
-
-// Rounds 0 and 1 of the first wave of a SQUARE phase-2 instance on the 4
-// entries at x0: P[x] = eq(r_P, x) V[x] and B = 0, so the B terms drop out.
-__device__ __forceinline__ void sq2_run(const Globals &G, const GenWave &W, u64 x0, const GenSmem &sm, u64 (&h)[15],
-                                        u64 &pn, u64 &vn)
-{
-    const ulonglong2 *sv = reinterpret_cast<const ulonglong2 *>(W.inV + x0);
-    const ulonglong2 va = __ldg(sv), vb = __ldg(sv + 1);
-    const EqTab &T = G.layers[W.layer].trp;
-    u64 v[4] = {va.x, va.y, vb.x, vb.y}, p[4];
-#pragma unroll
-    for (int q = 0; q < 4; q++) p[q] = wmul(eq_at(T, x0 + q), v[q]);
-#pragma unroll
-    for (int k = 0; k < 2; k++) {
-        acc128 a0, a1, a2;
-        acc_zero(a0);
-        acc_zero(a1);
-        acc_zero(a2);
-        const u32 rr0 = sm.r[k][0], rr1 = sm.r[k][1];
-#pragma unroll
-        for (int q = 0; q < (2 >> k); q++) {
-            const u64 p0 = p[2 * q], p1 = p[2 * q + 1], v0 = v[2 * q], v1 = v[2 * q + 1];
-            const u64 dp = p1 + (2 * FP_P) - p0, dv = v1 + (2 * FP_P) - v0;
-            mac(a0, p0, v0);
-            mac(a1, p1, v1);
-            mac(a2, wred(dp), wred(dv));
-            p[q] = wlin1(p0, dp, rr0, rr1);
-            v[q] = wlin1(v0, dv, rr0, rr1);
-        }
-        h[3 * k] = wred(h[3 * k] + acc_red(a0));
-        h[3 * k + 1] = wred(h[3 * k + 1] + acc_red(a1));
-        h[3 * k + 2] = wred(h[3 * k + 2] + acc_red(a2));
+    u64 p, b = 0;
+    if (W.src == GS_MM2) {
+        const u32 Lb = G.layers[W.layer].s / 3;
+        const u64 k = x & ((1ull << Lb) - 1), i = x >> Lb;
+        return make_ulonglong2((i >> Lb) ? 0 : wmul(__ldg(W.inP + k), __ldg(W.inB + i)), 0);
     }
-    pn = p[0];
-    vn = v[0];
+    const EqTab &T = G.layers[W.layer].trp;
+    switch (W.src) {
+    case GS_SQ2: p = wmul(eq_at(T, x), v); break;
+    case GS_PAIR2: p = wmul(eq_at(T, x), ve); break;
+    case GS_FINAL2: p = (x & 1) ? wmul(eq_at(T, x >> 1), v) : 0; break;
+    default: {  // GS_FIRST2
+        const u64 wa = eq_at(T, 2 * x + 1);
+        b = wmul(wa, v);
+        p = wred(wmul(eq_at(T, 2 * x), v) + wa);
+        break;
+    }
+    }
+    return make_ulonglong2(p, b);
 }
 
-// In-register rounds for e in 3..5: runs of 4 entries (rounds 0, 1), then
+// Rounds 0 and 1 of the first wave of a phase-2 instance of an F0_PAIR or
+// F0_FINAL layer on two pairs (va, vb) of entries.  With A = w V[2q] (PAIR; w =
+// eq(r_P, .) without its coordinate 0, whose value is a = (r_P)_0) or w V[2q+1]
+// (FINAL), P[2q + b] is A times a factor of b alone, so round 0's message
+// follows from sum A V[2q] and sum A V[2q+1] (a[0], a[1]), and its fold is A
+// times a constant, left out here and applied to the later rounds by k_final:
+// three products a pair besides w instead of seven.
+__device__ __forceinline__ void bil_run(u64 Aa, u64 Ab, ulonglong2 va, ulonglong2 vb, const GenSmem &sm,
+                                        acc128 (&a)[6], u64 &pn, u64 &vn)
+{
+    mac(a[0], Aa, va.x);
+    mac(a[0], Ab, vb.x);
+    mac(a[1], Aa, va.y);
+    mac(a[1], Ab, vb.y);
+    const u64 r = sm.r[0];
+    gen_pair_run(Aa, Ab, wfold(va.x, va.y, r), wfold(vb.x, vb.y, r), sm.r[1], a + 3, pn, vn);
+}
+
+// In-register rounds for e in 2..5: runs of 4 entries (rounds 0, 1), then
 // rounds 2.. on the runs' folded triples, combined like a binary counter.
+// SQUARE's and F0's P carries eq(r_P, .) = lo hi of its split table, and the
+// thread's entries share one hi (2^e entries, e at most half the coordinates),
+// so P is formed with lo alone and hi multiplies the thread's sums and its
+// folded P once.
 __device__ __forceinline__ void gen_regs_runs(const Globals &G, const GenWave &W, u64 x0, u32 e, bool hasB,
                                               GenSmem &sm, u64 (&h)[15], u64 &pv, u64 &vv, u64 &bv)
 {
-    const u32 nruns = 1u << (e - 2);
+    const u32 nruns = 1u << (e - 2), src = W.src;
+    const bool b_run = hasB || src == GS_FIRST2;
 #pragma unroll
     for (int j = 0; j < 9; j++) sm.hs[j][threadIdx.x] = 0;
+    acc128 a[6];
+#pragma unroll
+    for (int j = 0; j < 6; j++) acc_zero(a[j]);
+    const bool lohi = src == GS_SQ2 || src == GS_PAIR2 || src == GS_FINAL2;
+    const u64 *lo = nullptr;
+    u64 hi = 1;
+    if (lohi) {
+        const EqTab &T = G.layers[W.layer].trp;
+        const u64 x = src == GS_FINAL2 ? x0 >> 1 : x0;
+        lo = T.lo + (x & ((1ull << T.h) - 1));
+        hi = T.hi[x >> T.h];
+    }
     u64 p0 = 0, v0 = 0, b0 = 0, p1 = 0, v1 = 0, b1 = 0, p2 = 0, v2 = 0, b2 = 0;  // pending: rounds 2, 3, 4
     u64 tp = 0, tv = 0, tb = 0;
-    const bool tree2 = W.src == GS_TREE2;
     // a rolled loop keeps the kernel small (instruction-cache bound when unrolled)
 #pragma unroll 1
     for (u32 sub = 0; sub < nruns; sub++) {
         if (sub + 1 < nruns) {
             const u64 xn = x0 + 4 * (sub + 1);
             prefetch_l1(W.inV + xn);
-            if (W.src == GS_NONE) {
+            if (src == GS_NONE) {
                 prefetch_l1(W.inP + xn);
                 if (hasB) prefetch_l1(W.inB + xn);
             }
         }
-        if (tree2) {
-            tree2_run(G, W, x0 + 4 * sub, sm, h, tp, tv, tb);
-        } else if (W.src == GS_SQ2) {
-            sq2_run(G, W, x0 + 4 * sub, sm, h, tp, tv);
-            tb = 0;
+        if (src == GS_PAIR2 || src == GS_FINAL2) {
+            const ulonglong2 *sv = reinterpret_cast<const ulonglong2 *>(W.inV + x0 + 4 * sub);
+            const ulonglong2 va = __ldg(sv), vb = __ldg(sv + 1);
+            const ulonglong2 *sl = reinterpret_cast<const ulonglong2 *>(lo) + (src == GS_PAIR2 ? 2 * sub : sub);
+            ulonglong2 l = __ldg(sl);
+            if (src == GS_PAIR2) {
+                const ulonglong2 l2 = __ldg(sl + 1);
+                l = make_ulonglong2(wmul(l.x + l.y, va.x), wmul(l2.x + l2.y, vb.x));
+            } else {
+                l = make_ulonglong2(wmul(l.x, va.y), wmul(l.y, vb.y));
+            }
+            bil_run(l.x, l.y, va, vb, sm, a, tp, tv);
         } else {
             u64 p[4], v[4], b[4];
-            gen_load<4>(W, x0 + 4 * sub, hasB, p, v, b);
-            gen_regs<2>(p, v, b, sm, h);
-            tp = p[0];
-            tv = v[0];
-            tb = b[0];
+            if (src == GS_NONE) {
+                gen_load<4>(W, x0 + 4 * sub, hasB, p, v, b);
+            } else {
+                const ulonglong2 *sv = reinterpret_cast<const ulonglong2 *>(W.inV + x0 + 4 * sub);
+                const ulonglong2 va = __ldg(sv), vb = __ldg(sv + 1);
+                v[0] = va.x, v[1] = va.y, v[2] = vb.x, v[3] = vb.y;
+                if (src == GS_SQ2) {
+                    const ulonglong2 *sl = reinterpret_cast<const ulonglong2 *>(lo) + 2 * sub;
+                    const ulonglong2 l = __ldg(sl), l2 = __ldg(sl + 1);
+                    p[0] = wmul(l.x, v[0]), p[1] = wmul(l.y, v[1]), p[2] = wmul(l2.x, v[2]), p[3] = wmul(l2.y, v[3]);
+                } else {
+#pragma unroll
+                    for (int q = 0; q < 4; q++) {
+                        const ulonglong2 t = gen_source(G, W, x0 + 4 * sub + q, v[q], v[q & 2]);
+                        p[q] = t.x;
+                        b[q] = t.y;
+                    }
+                }
+            }
+            if (b_run)
+                gen_run<true>(p, v, b, sm, a, tp, tv, tb);
+            else
+                gen_run<false>(p, v, b, sm, a, tp, tv, tb);
         }
         if (!(sub & 1)) {  // wait for the partner run
             p0 = tp, v0 = tv, b0 = tb;
             continue;
         }
-        gen_pair_acc(p0, tp, v0, tv, b0, tb, sm.r[2][0], sm.r[2][1], sm, 0, tp, tv, tb);
+        gen_pair_acc(b_run, p0, tp, v0, tv, b0, tb, sm.r[2], sm, 0, tp, tv, tb);
         if (nruns == 2) continue;
         if (!(sub & 2)) {
             p1 = tp, v1 = tv, b1 = tb;
             continue;
         }
-        gen_pair_acc(p1, tp, v1, tv, b1, tb, sm.r[3][0], sm.r[3][1], sm, 1, tp, tv, tb);
+        gen_pair_acc(b_run, p1, tp, v1, tv, b1, tb, sm.r[3], sm, 1, tp, tv, tb);
         if (nruns == 4) continue;
         if (!(sub & 4)) {
             p2 = tp, v2 = tv, b2 = tb;
             continue;
         }
-        gen_pair_acc(p2, tp, v2, tv, b2, tb, sm.r[4][0], sm.r[4][1], sm, 2, tp, tv, tb);
+        gen_pair_acc(b_run, p2, tp, v2, tv, b2, tb, sm.r[4], sm, 2, tp, tv, tb);
+    }
+#pragma unroll
+    for (int j = 0; j < 6; j++) h[j] = acc_red(a[j]);
+#pragma unroll
+    for (int j = 0; j < 9; j++) h[6 + j] = sm.hs[j][threadIdx.x];
+    if (lohi) {  // every sum and P are linear in it (B = 0)
+#pragma unroll
+        for (int j = 0; j < 15; j++) h[j] = wmul(hi, h[j]);
+        tp = wmul(hi, tp);
     }
     pv = tp;
     vv = tv;
     bv = tb;
-    if (tree2) h[2] = wred((2 * FP_P) - h[2]);
-#pragma unroll
-    for (int j = 0; j < 9; j++) h[6 + j] = sm.hs[j][threadIdx.x];
 }
 
 // Sum over the lanes l = 0 mod 2^(kk+1) of a warp (the only lanes holding a
@@ -594,7 +589,7 @@ __device__ __forceinline__ void gen_round_sum(u64 c0, u64 c1, u64 c2, u32 kk, u6
 // prod_cross: the first thread of each pair keeps the folded values).  The
 // per-warp sums of round k go to sm.w[warp][3k..3k+2] (CTA-level rounds: warp
 // 0's row, zeros in the other rows).
-__device__ __forceinline__ void gen_cross(u64 &p, u64 &v, u64 &b, u32 off, u32 tid, u32 na, u32 nr, GenSmem &sm)
+__device__ __forceinline__ void gen_cross(bool hasB, u64 &p, u64 &v, u64 &b, u32 off, u32 tid, u32 na, u32 nr, GenSmem &sm)
 {
     const u32 lane = tid & 31, warp = tid >> 5;
     // rolled: one copy of the round body keeps the kernel small
@@ -605,10 +600,10 @@ __device__ __forceinline__ void gen_cross(u64 &p, u64 &v, u64 &b, u32 off, u32 t
             const u32 d = 1u << kk;
             const u64 p1 = __shfl_down_sync(0xffffffffu, p, d);
             const u64 v1 = __shfl_down_sync(0xffffffffu, v, d);
-            const u64 b1 = __shfl_down_sync(0xffffffffu, b, d);
+            const u64 b1 = hasB ? __shfl_down_sync(0xffffffffu, b, d) : 0;
             u64 c0 = 0, c1 = 0, c2 = 0;
             if ((tid & ((2u << kk) - 1)) == 0 && tid < na)
-                gen_pair(p, p1, v, v1, b, b1, sm.r[k][0], sm.r[k][1], c0, c1, c2, p, v, b);
+                gen_pair(hasB, p, p1, v, v1, b, b1, sm.r[k], c0, c1, c2, p, v, b);
             gen_round_sum(c0, c1, c2, kk, &sm.w[warp][3 * k]);
         }
     }
@@ -632,11 +627,11 @@ __device__ __forceinline__ void gen_cross(u64 &p, u64 &v, u64 &b, u32 off, u32 t
                 const u32 d = 1u << (kk - 5);
                 const u64 p1 = __shfl_down_sync(0xffffffffu, p, d);
                 const u64 v1 = __shfl_down_sync(0xffffffffu, v, d);
-                const u64 b1 = __shfl_down_sync(0xffffffffu, b, d);
+                const u64 b1 = hasB ? __shfl_down_sync(0xffffffffu, b, d) : 0;
                 const u32 t = lane << 5;
                 u64 c0 = 0, c1 = 0, c2 = 0;
                 if ((t & ((2u << kk) - 1)) == 0 && t < na)
-                    gen_pair(p, p1, v, v1, b, b1, sm.r[k][0], sm.r[k][1], c0, c1, c2, p, v, b);
+                    gen_pair(hasB, p, p1, v, v1, b, b1, sm.r[k], c0, c1, c2, p, v, b);
                 gen_round_sum(c0, c1, c2, kk - 5, &sm.w[0][3 * k]);
             }
         }
@@ -649,14 +644,15 @@ __device__ __forceinline__ void gen_cross(u64 &p, u64 &v, u64 &b, u32 off, u32 t
 }
 
 // One chunk of a GEN wave.
-__device__ void gen_chunk(const Globals &G, const GenWave &W, u32 chunk, GenSmem &sm)
+__device__ __noinline__ void gen_chunk(const Globals &G, const GenWave &W, u32 chunk)
 {
+    GenSmem &sm = reinterpret_cast<WaveSmem *>(wv_dyn)->gen;
     const u32 tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const u32 nr = W.nr, e = W.e;
     const u32 na = 1u << (nr - e);
     const u64 base = (u64)chunk << nr;
     const bool hasB = (W.flags & WF_HASB) != 0;
-    if (tid < nr) limbs31(G.chal[W.chal_off + tid], sm.r[tid][0], sm.r[tid][1]);
+    if (tid < nr) sm.r[tid] = G.chal[W.chal_off + tid];
     __syncthreads();
     u64 pv = 0, vv = 0, bv = 0;
     if (e > 0) {
@@ -676,18 +672,16 @@ __device__ void gen_chunk(const Globals &G, const GenWave &W, u32 chunk, GenSmem
         const u64 x = base + tid;
         const bool ext = W.r0 == 0;
         vv = ld_in(W.inV + x, ext);
-        if (W.src == GS_SQ2) {
-            pv = wmul(eq_at(G.layers[W.layer].trp, x), vv);
-        } else if (W.src == GS_TREE2) {
-            const u64 w = (x & 1) ? 0 : eq_at(G.layers[W.layer].trp, x >> 1);
-            pv = w;
-            bv = (x & 1) ? 0 : wmul(w, ld_in(W.inV + x + 1, ext));
-        } else {
+        if (W.src == GS_NONE) {
             pv = ld_in(W.inP + x, ext);
             bv = hasB ? ld_in(W.inB + x, ext) : 0;
+        } else {
+            const ulonglong2 t = gen_source(G, W, x, vv, W.src == GS_PAIR2 ? ld_in(W.inV + (x & ~1ull), ext) : vv);
+            pv = t.x;
+            bv = t.y;
         }
     }
-    gen_cross(pv, vv, bv, e, tid, na, nr, sm);
+    gen_cross(hasB || W.src == GS_FIRST2, pv, vv, bv, e, tid, na, nr, sm);
     __syncthreads();
     if (tid < 3 * nr) {
         const u64 sum = wred(sm.w[0][tid] + sm.w[1][tid] + sm.w[2][tid] + sm.w[3][tid]);
@@ -711,52 +705,53 @@ __device__ void gen_chunk(const Globals &G, const GenWave &W, u32 chunk, GenSmem
 
 // One level of coefficient folding in registers: D+1 -> D+2 coefficients.
 template <int D>
-__device__ __forceinline__ void line_fold(const u64 (&A)[D + 1], const u64 (&B)[D + 1], u32 a0, u32 a1, u32 b0,
-                                          u32 b1, u64 (&out)[D + 2])
+__device__ __forceinline__ void line_fold(const u64 (&A)[D + 1], const u64 (&B)[D + 1], u64 a, u64 b,
+                                          u64 (&out)[D + 2])
 {
     u64 d[D + 1];
 #pragma unroll
     for (int c = 0; c <= D; c++) d[c] = B[c] + (2 * FP_P) - A[c];
-    out[0] = wlin1(A[0], d[0], a0, a1);
+    out[0] = wlin1(A[0], d[0], a);
 #pragma unroll
-    for (int c = 1; c <= D; c++) out[c] = wlin2(A[c], d[c], d[c - 1], a0, a1, b0, b1);
-    out[D + 1] = wlin1(0, d[D], b0, b1);
+    for (int c = 1; c <= D; c++) out[c] = wlin2(A[c], d[c], d[c - 1], a, b);
+    out[D + 1] = wlin1(0, d[D], b);
 }
 
 // 8 consecutive entries -> one cubic (coordinates 0, 1, 2 of the run).
-__device__ __forceinline__ void line_run8(const u64 *v, const u32 *la, const u32 *lb, u64 (&out)[4])
+__device__ __forceinline__ void line_run8(const u64 *v, const u64 *la, const u64 *lb, u64 (&out)[4])
 {
     u64 l1[4][2];
 #pragma unroll
     for (int q = 0; q < 4; q++) {
         const u64 dd = v[2 * q + 1] + (2 * FP_P) - v[2 * q];
-        l1[q][0] = wlin1(v[2 * q], dd, la[0], la[1]);
-        l1[q][1] = wlin1(0, dd, lb[0], lb[1]);
+        l1[q][0] = wlin1(v[2 * q], dd, la[0]);
+        l1[q][1] = wlin1(0, dd, lb[0]);
     }
     u64 l2[2][3];
-    line_fold<1>(l1[0], l1[1], la[2], la[3], lb[2], lb[3], l2[0]);
-    line_fold<1>(l1[2], l1[3], la[2], la[3], lb[2], lb[3], l2[1]);
-    line_fold<2>(l2[0], l2[1], la[4], la[5], lb[4], lb[5], out);
+    line_fold<1>(l1[0], l1[1], la[1], lb[1], l2[0]);
+    line_fold<1>(l1[2], l1[3], la[1], lb[1], l2[1]);
+    line_fold<2>(l2[0], l2[1], la[2], lb[2], out);
 }
 
 // Coefficient `c` of the fold of polynomials A, B (degree deg, W values).
-__device__ __forceinline__ u64 line_coef(const u64 *A, const u64 *B, u32 deg, u32 c, const u32 *la, const u32 *lb)
+__device__ __forceinline__ u64 line_coef(const u64 *A, const u64 *B, u32 deg, u32 c, u64 la, u64 lb)
 {
     const u64 dc = (c <= deg) ? B[c] + (2 * FP_P) - A[c] : 0;
     const u64 dm = (c >= 1) ? B[c - 1] + (2 * FP_P) - A[c - 1] : 0;
     const u64 ac = (c <= deg) ? A[c] : 0;
-    return wlin2(ac, dc, dm, la[0], la[1], lb[0], lb[1]);
+    return wlin2(ac, dc, dm, la, lb);
 }
 
 // One chunk of one line wave, by the whole CTA.
-__device__ void line_chunk(const Globals &G, const LineWaveDev &W, u32 chunk, LineSmem &sm)
+__device__ __noinline__ void line_chunk(const Globals &G, const LineWaveDev &W, u32 chunk)
 {
+    LineSmem &sm = reinterpret_cast<WaveSmem *>(wv_dyn)->line;
     const u32 tid = threadIdx.x;
     if (tid < W.nl) {
         const u64 a = G.chal[W.a_off + W.l0 + tid];
         const u64 b = f_sub(G.chal[W.b_off + W.l0 + tid], a);
-        limbs31(a, sm.la[tid][0], sm.la[tid][1]);
-        limbs31(b, sm.lb[tid][0], sm.lb[tid][1]);
+        sm.la[tid] = a;
+        sm.lb[tid] = b;
     }
     __syncthreads();
     u32 m, deg, k0;  // polynomials in bufA, their degree, coordinates already folded
@@ -767,13 +762,11 @@ __device__ void line_chunk(const Globals &G, const LineWaveDev &W, u32 chunk, Li
         if (tid < na) {
             if (e == LN_E) {
                 const ulonglong2 *src = reinterpret_cast<const ulonglong2 *>(W.in + base + ((u64)tid << LN_E));
-                u32 la[12], lb[12];
+                u64 la[6], lb[6];
 #pragma unroll
                 for (int k = 0; k < 6; k++) {
-                    la[2 * k] = sm.la[k][0];
-                    la[2 * k + 1] = sm.la[k][1];
-                    lb[2 * k] = sm.lb[k][0];
-                    lb[2 * k + 1] = sm.lb[k][1];
+                    la[k] = sm.la[k];
+                    lb[k] = sm.lb[k];
                 }
                 // eight runs of 8 entries (cubics over coordinates 0..2), combined
                 // like a binary counter over coordinates 3, 4, 5; a rolled loop
@@ -798,14 +791,14 @@ __device__ void line_chunk(const Globals &G, const LineWaveDev &W, u32 chunk, Li
                         continue;
                     }
                     u64 q[5];
-                    line_fold<3>(c0, c, la[6], la[7], lb[6], lb[7], q);
+                    line_fold<3>(c0, c, la[3], lb[3], q);
                     if (!(run & 2)) {
 #pragma unroll
                         for (int i = 0; i < 5; i++) q0[i] = q[i];
                         continue;
                     }
                     u64 t5[6];
-                    line_fold<4>(q0, q, la[8], la[9], lb[8], lb[9], t5);
+                    line_fold<4>(q0, q, la[4], lb[4], t5);
 #pragma unroll
                     for (int i = 0; i < 6; i++) {
                         if (run & 4) s1[i] = t5[i];
@@ -813,7 +806,7 @@ __device__ void line_chunk(const Globals &G, const LineWaveDev &W, u32 chunk, Li
                     }
                 }
                 u64 p[7];
-                line_fold<5>(s0, s1, la[10], la[11], lb[10], lb[11], p);
+                line_fold<5>(s0, s1, la[5], lb[5], p);
 #pragma unroll
                 for (int c = 0; c < 7; c++) sm.bufA[tid * 7 + c] = p[c];
             } else {
@@ -834,7 +827,7 @@ __device__ void line_chunk(const Globals &G, const LineWaveDev &W, u32 chunk, Li
             const u64 dc = (c <= din) ? __ldcg(B + c) + (2 * FP_P) - __ldcg(A + c) : 0;
             const u64 dm = (c >= 1) ? __ldcg(B + c - 1) + (2 * FP_P) - __ldcg(A + c - 1) : 0;
             const u64 ac = (c <= din) ? __ldcg(A + c) : 0;
-            sm.bufA[j * C + c] = wlin2(ac, dc, dm, sm.la[0][0], sm.la[0][1], sm.lb[0][0], sm.lb[0][1]);
+            sm.bufA[j * C + c] = wlin2(ac, dc, dm, sm.la[0], sm.lb[0]);
         }
         m = half;
         deg = din + 1;
@@ -919,8 +912,6 @@ __device__ __forceinline__ bool wave_done(u32 *counter, u32 nchunks, u32 &s_flag
     return last;
 }
 
-extern __shared__ __align__(16) unsigned char wv_dyn[];
-
 #ifndef WV_MINB
 #define WV_MINB 4  // resident CTAs per SM the register allocation is sized for (4: 128 registers)
 #endif
@@ -928,41 +919,44 @@ extern __shared__ __align__(16) unsigned char wv_dyn[];
 __global__ void __launch_bounds__(WV_NT, WV_MINB) k_waves(const Globals *Gs, const LineWaveDev *lw, const ProdWave *pw,
                                                    const GenWave *gw, const Task *tasks, int ntasks, u32 *ctr)
 {
-    WaveSmem &sm = *reinterpret_cast<WaveSmem *>(wv_dyn);
     __shared__ int s_task;
     __shared__ u32 s_flag;
     // the final reduction may begin its launch on SMs this launch frees as it
     // drains (it waits for the whole launch before it reads what it wrote)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    // a CTA's first task is its own index (the grid has at most ntasks CTAs);
+    // the counter hands out the rest, each fetched while the task before it runs
+    int ti = blockIdx.x;
     for (;;) {
-        __syncthreads();  // the previous task is done with shared memory
-        if (threadIdx.x == 0) s_task = (int)atomicAdd(&ctr[0], 1u);
-        __syncthreads();
-        const int ti = s_task;
-        if (ti >= ntasks) break;
         const Task tk = tasks[ti];
+        int next = 0;
+        if (threadIdx.x == 0) next = (int)(gridDim.x + atomicAdd(&ctr[0], 1u));
         if (tk.type == TK_LINE) {
             const LineWaveDev &W = lw[tk.wave];
             const Globals &G = Gs[W.circ];
-            line_chunk(G, W, tk.chunk, sm.line);
-            if (W.tail && wave_done(W.counter, W.nchunks, s_flag)) line_chunk(G, lw[tk.wave + 1], 0, sm.line);
+            line_chunk(G, W, tk.chunk);
+            if (W.tail && wave_done(W.counter, W.nchunks, s_flag)) line_chunk(G, lw[tk.wave + 1], 0);
         } else if (tk.type == TK_PROD) {
             const ProdWave &W = pw[tk.wave];
-            const Globals &G = Gs[W.circ];
-            prod_chunk(G, W, tk.chunk, sm.prod);
+            prod_chunk(W, tk.chunk);
             if ((W.flags & WF_TAIL) && wave_done(W.counter, W.nchunks, s_flag)) {
                 __syncthreads();
-                prod_chunk(G, pw[tk.wave + 1], 0, sm.prod);
+                prod_chunk(pw[tk.wave + 1], 0);
             }
         } else {
             const GenWave &W = gw[tk.wave];
             const Globals &G = Gs[W.circ];
-            gen_chunk(G, W, tk.chunk, sm.gen);
+            gen_chunk(G, W, tk.chunk);
             if ((W.flags & WF_TAIL) && wave_done(W.counter, W.nchunks, s_flag)) {
                 __syncthreads();
-                gen_chunk(G, gw[tk.wave + 1], 0, sm.gen);
+                gen_chunk(G, gw[tk.wave + 1], 0);
             }
         }
+        if (threadIdx.x == 0) s_task = next;
+        __syncthreads();  // the task is done with shared memory
+        ti = s_task;
+        if (ti >= ntasks) break;
+        __syncthreads();  // s_task is read
     }
     // the CTA that exits last resets the task counter for the next launch
     if (threadIdx.x == 0) {
@@ -1001,7 +995,7 @@ void launch_waves(const Globals *Gs, const LineWaveDev *lw, const ProdWave *pw, 
 // The scalars a round's message needs besides its partial sums (loaded
 // before the sums, so that both sets of loads are in flight together).
 struct RoundScalars {
-    u64 ez, ch, v1, es, kap, c0, c1;
+    u64 ez, ch, rp0, v1, es, kap, c0, c1;
 };
 
 // Everything but v1 (the coin launch wrote it all before the wave launch).
@@ -1009,7 +1003,8 @@ __device__ __forceinline__ RoundScalars round_scalars_pre(const RoundRef &R)
 {
     RoundScalars S{};
     S.ez = *R.ez;
-    if (R.defer || R.kind < PK_GEN_FIRST) S.ch = *R.ch;
+    S.ch = *R.ch;
+    if (R.rp0) S.rp0 = *R.rp0;
     if (R.kind < PK_GEN_FIRST) {
         S.es = *R.esum;
         S.kap = *R.kap;
@@ -1019,31 +1014,63 @@ __device__ __forceinline__ RoundScalars round_scalars_pre(const RoundRef &R)
     return S;
 }
 
-// g(0), g(1), g(2) of round R from its canonical partial sums h, written to
-// the circuit's transcript.
+// g(0), g(1), g(2) of round R from its canonical partial sums h (and h2:
+// TREE phase 2's second instance), written to the circuit's transcript.
 __device__ __forceinline__ void final_round(const Globals *Gs, const RoundRef &R, const RoundScalars &S,
-                                            const u64 (&h)[3])
+                                            const u64 (&h)[3], const u64 (&h2)[2])
 {
-    const bool gen = R.kind >= PK_GEN_FIRST;
     const u64 ez = S.ez;
     u64 g0, g1, g2;
-    if (gen) {
-        u64 sg = (R.kind == PK_GEN_TAB) ? 1 : ez;
-        if (R.defer) sg = f_mul(sg, f_sub(1, S.ch));  // TREE phase 2: 1 - r_0 left out of P, B
-        g0 = f_mul(sg, h[0]);
-        g1 = f_mul(sg, h[1]);
-        // h[2] is the leading coefficient: value at 2 = 2 h1 - h0 + 2 h2
-        g2 = f_mul(sg, f_add(f_sub(f_add(h[1], h[1]), h[0]), f_add(h[2], h[2])));
+    if (R.kind >= PK_GEN_FIRST) {
+        // h[2] is the leading coefficient: value at 2 = 2 g(1) - g(0) + 2 h2
+        u64 s0 = (R.kind == PK_GEN_TAB) ? 1 : ez, s1 = s0, s2 = s0, lead = h[2];
+        if (R.kind == PK_GEN_PAIR2 || R.kind == PK_GEN_FINAL2) {
+            // round 0: P[2q + b] = A f_b, f = (1 - a, a) (PAIR) or (0, 1) (FINAL);
+            // later rounds carry the fold f_0 + r_0 (f_1 - f_0) left out of P
+            const u64 a = R.kind == PK_GEN_PAIR2 ? S.rp0 : 1, f0 = f_sub(1, a);
+            if (R.j == 0) {
+                s0 = f_mul(ez, f0);
+                s1 = f_mul(ez, a);
+                s2 = f_sub(s1, s0);
+                lead = f_sub(h[1], h[0]);
+            } else {
+                s0 = s1 = s2 = f_mul(ez, f_add(f0, f_mul(S.ch, f_sub(a, f0))));
+            }
+        }
+        g0 = f_mul(s0, h[0]);
+        g1 = f_mul(s1, h[1]);
+        lead = f_mul(s2, lead);
+        g2 = f_add(f_sub(f_add(g1, g1), g0), f_add(lead, lead));
+    } else if (R.kind == PK_TREE2) {
+        const u64 kj = f_mul(ez, S.kap), c0 = S.c0, c1 = S.c1;
+        const u64 d = f_sub(f_add(h[1], h[1]), h[0]);  // h(2)
+        if (R.j == 0) {  // L_0(t) (h(t) + h(1)), L_0 = 1 - t
+            g0 = f_mul(ez, f_add(h[0], h[1]));
+            g1 = 0;
+            g2 = f_neg(f_mul(ez, f_add(d, h[1])));
+        } else {
+            const u64 sb = f_mul(ez, f_sub(1, S.ch));
+            const u64 b0 = f_mul(sb, f_mul(c0, h2[0])), b1 = f_mul(sb, f_mul(c1, h2[1]));
+            g0 = f_add(f_mul(kj, f_mul(c0, h[0])), b0);
+            g1 = f_add(f_mul(kj, f_mul(c1, h[1])), b1);
+            g2 = f_add(f_mul(kj, f_mul(f_sub(f_add(c1, c1), c0), d)), f_sub(f_add(b1, b1), b0));
+        }
     } else {
-        const u64 v1 = S.v1, ch = S.ch, es = S.es, kap = S.kap, c0 = S.c0, c1 = S.c1;
-        u64 sigma = 1, c2u = 0;
+        const u64 v1 = S.v1, es = S.es, kap = S.kap, c0 = S.c0, c1 = S.c1;
+        // the instance sums sigma P (sv V + add)
+        u64 sigma = 1, sv = 1, add = 0;
         if (R.kind == PK_TREE3) {
-            sigma = f_mul(ez, f_sub(1, ch));
-            c2u = v1;
-        } else if (R.kind == PK_SQ3) {
+            sigma = f_mul(ez, f_sub(1, S.ch));
+            add = v1;
+        } else if (R.kind == PK_FIRST3) {
+            sigma = ez;
+            add = f_mul(S.rp0, v1);
+            sv = f_add(S.rp0, f_sub(v1, add));  // rp0 + v1 (1 - rp0)
+        } else if (R.kind != PK_PH1) {
             sigma = f_mul(ez, v1);
         }
-        const u64 h0 = f_add(h[0], f_mul(c2u, es)), h1 = f_add(h[1], f_mul(c2u, es));
+        const u64 ce = f_mul(add, es);
+        const u64 h0 = f_add(f_mul(sv, h[0]), ce), h1 = f_add(f_mul(sv, h[1]), ce);
         const u64 kj = f_mul(sigma, kap);
         g0 = f_mul(kj, f_mul(c0, h0));
         g1 = f_mul(kj, f_mul(c1, h1));
@@ -1078,12 +1105,14 @@ __global__ void __launch_bounds__(256) k_final(Globals *Gs, const RoundRef *roun
             S = (gw == gw0) ? S0 : round_scalars_pre(R);
             if (R.kind < PK_GEN_FIRST) S.v1 = *R.v1;  // written by the layer's line reduction
         }
-        u64 h[3] = {0, 0, 0};
-        if (R.kind >= PK_GEN_FIRST)
+        u64 h[3] = {0, 0, 0}, h2[2] = {0, 0};
+        if (R.kind >= PK_GEN_FIRST) {
             warp_record_sums<3>(R.part_pos, R.nchunks, lane, h);
-        else
+        } else {
             warp_record_sums<2>(R.part_pos, R.nchunks, lane, h);
-        if (lane == 0) final_round(Gs, R, S, h);
+            if (R.nchunks2) warp_record_sums<2>(R.part2_pos, R.nchunks2, lane, h2);
+        }
+        if (lane == 0) final_round(Gs, R, S, h, h2);
     }
     for (u64 t = gt; t < (u64)(nrounds - nbig); t += nthreads) {
         const RoundRef R = rounds[nbig + t];
@@ -1094,7 +1123,11 @@ __global__ void __launch_bounds__(256) k_final(Globals *Gs, const RoundRef *roun
         for (u32 q = 0; q < R.nchunks; q++)
             for (u32 v = 0; v < nv; v++) h[v] = wred(h[v] + R.part_pos[(u64)q * nv + v]);
         for (u32 v = 0; v < 3; v++) h[v] = wcanon(h[v]);
-        final_round(Gs, R, S, h);
+        u64 h2[2] = {0, 0};
+        for (u32 q = 0; q < R.nchunks2; q++)
+            for (u32 v = 0; v < 2; v++) h2[v] = wred(h2[v] + R.part2_pos[(u64)q * 2 + v]);
+        for (u32 v = 0; v < 2; v++) h2[v] = wcanon(h2[v]);
+        final_round(Gs, R, S, h, h2);
     }
     // the outputs open each transcript: a CTA per circuit (grid-stride over
     // the circuits), its threads over the outputs; the proof's in-place input

@@ -43,8 +43,9 @@ struct LayerDev {
     u64 *Vn;          // layer i+1 values
     u64 tr_msg;       // transcript offset of the layer's round values
     u64 tr_q;         // transcript offset of q(0..s_{i+1})
-    EqTab tz, trp, tr1, tr2;  // eq tables of z_i, r_P, r1, r2
-    u64 *P2, *B2, *P3, *B3;   // phase-2/3 tables over layer i+1 (B* NULL if !has_add)
+    EqTab trp, tr1, tr2;  // eq tables of r_P, r1, r2 (r1, r2: table-built layers, verifier)
+    u64 *P2, *B2, *P3, *B3;   // EXPLICIT: phase-2/3 tables over layer i+1 (B* NULL if !has_add)
+    u64 *mu, *mei;            // MATMULT: tables of k_mm_tables (n entries each)
     const unsigned char *type;  // EXPLICIT only
     const u32 *in1, *in2;
     const u32 *by1_off, *by1_g;  // gates grouped by in1: offsets [S_{i+1}+1], gate ids [S_i]
@@ -82,24 +83,60 @@ __device__ __forceinline__ void gate_wiring(const LayerDev &L, u64 g, u64 &a, u6
 
 // Flags of a sum-check wave.  WF_TAIL: the next descriptor (a single chunk)
 // is run by the CTA that finishes this wave's last chunk.
-enum : u32 { WF_HASB = 2, WF_LAST = 4, WF_TAIL = 8 };
+// WF_ODD: a PROD wave over the odd entries of its input table.
+enum : u32 { WF_HASB = 2, WF_LAST = 4, WF_TAIL = 8, WF_ODD = 16 };
 
 // Kinds of sum-check instance (SCI).  Product-weighted ones (< PK_GEN_FIRST)
 // keep P = sigma prod_m L_m(x_m) implicit; general ones fold P, V, B tables.
+// Phase 3's gates with in2 = x have a product-form weight over x in every
+// structured kind, so it needs no table: with w, e the factors eq(r_P, .),
+// eq(r1, .) of the gates and their first in-neighbours,
+//   SQUARE    L_m = w_m e_m;
+//   TREE      L_0 = (0, 1), L_m = w_{m-1} e_m, summed with V + v1;
+//   F0_PAIR   in2 = 2q of gates 2q, 2q+1: L_0 = (w_0(0) e_0(0) + w_0(1) e_0(1), 0), L_m = w_m e_m;
+//   F0_FINAL  in2 = 2q+1: L_0 = (0, e_0(1)), L_m = w_{m-1} e_m;
+//   F0_FIRST  gates 2x (MUL), 2x+1 (ADD): L_m = w_{m+1} e_m, and per entry
+//             (w_0(0) v1 + w_0(1)) V + w_0(1) v1;
+//   MATMULT   x = (j, k, 1): L = w over j, w e over k, and on the top bit (0,
+//             the sum over i of w e, times e's own top factor).
 enum : u32 {
     PK_PH1 = 0,        // phase 1 of any layer: P = eq(z_i, .), V = V_i
-    PK_TREE3 = 1,      // TREE phase 3: L_0 = (0,1), L_m = eq(rP_{m-1},.) eq(r1_m,.), U = V + v1
-    PK_SQ3 = 2,        // SQUARE phase 3: L_m = eq(rP_m,.) eq(r1_m,.), sigma = eq(z,rP) v1
-    PK_GEN_FIRST = 8,
-    PK_GEN_SQ2 = 8,    // SQUARE phase 2: P[x] = eq(rP, x) V[x] (times eq(z, rP))
-    PK_GEN_TREE2 = 9,  // TREE phase 2: P[2g] = eq(rP, g), B[2g] = P[2g] V[2g+1] (times eq(z, rP))
-    PK_GEN_TAB = 10    // tables built by k_build23
+    PK_TREE3 = 1,
+    PK_SQ3 = 2,        // sigma = eq(z,rP) v1, as for the next three
+    PK_PAIR3 = 3,
+    PK_FINAL3 = 4,
+    PK_MM3 = 5,
+    PK_FIRST3 = 6,
+    // TREE phase 2: P[2g] = eq(rP, g), B[2g] = P[2g] V[2g+1] (times eq(z, rP)).
+    // P is a product over the coordinates, L_0 = (1, 0).  Folding B by r_0
+    // leaves (1 - r_0) eq(rP, g) V[2g+1], whose sums and folds are again linear
+    // in V with product weights, those of a folded coordinate e_m L_m instead
+    // of e_m: an instance of its own over the odd entries (PK_TREE2B), whose
+    // sums join round j >= 1 of PK_TREE2 in the final reduction.
+    PK_TREE2 = 7,
+    PK_TREE2B = 8,
+    PK_GEN_FIRST = 16,
+    PK_GEN_EZ = 16,    // phase 2 of SQUARE and F0 layers, P and B formed from the wiring (times eq(z, rP))
+    PK_GEN_PAIR2 = 17,   // phase 2 of F0_PAIR and
+    PK_GEN_FINAL2 = 18,  // F0_FINAL layers with a first wave in registers (bil_run)
+    PK_GEN_TAB = 19    // tables built by k_build23 (EXPLICIT) or k_mm_tables (MATMULT)
 };
 
 // Source of the first GEN wave's P and B.
-enum : u32 { GS_NONE = 0, GS_SQ2 = 1, GS_TREE2 = 2 };
+//   SQ2     P[x] = eq(rP, x) V[x]
+//   PAIR2   P[2q] = eq(rP, 2q) V[2q], P[2q+1] = eq(rP, 2q+1) V[2q]
+//   FINAL2  P[2q+1] = eq(rP, q) V[2q+1], P[2q] = 0
+//   FIRST2  P[x] = eq(rP, 2x) V[x] + eq(rP, 2x+1), B[x] = eq(rP, 2x+1) V[x]
+//   MM2     P[(k, i, 0)] = u[k] ei[i] (inP, inB: the tables of k_mm_tables), P[(., ., 1)] = 0
+enum : u32 { GS_NONE = 0, GS_SQ2 = 1, GS_PAIR2 = 2, GS_FINAL2 = 3, GS_FIRST2 = 4, GS_MM2 = 5 };
 
-#define PR_M 6  // PROD: at most 2^6 entries per thread, folded in registers (128 threads per CTA)
+// PROD: a chunk of more than 2^PR_C entries is a matrix of 2^kr rows of 2^PR_C
+// columns, kr <= PR_R (128 threads per CTA)
+#define PR_C 7
+#define PR_R 6
+// Words of the message-weight table of kk coordinates (see ProdWave::wblk).
+__host__ __device__ __forceinline__ u32 vec_slots(u32 kk) { return kk > 5 ? 1u << (kk - 5) : 1u; }
+__host__ __device__ __forceinline__ u32 vec_words(u32 kk) { return vec_slots(kk) * kk * 16; }
 #define GN_M 5  // GEN: at most 2^5 entries per thread (128 threads per CTA)
 // Evaluation runs holding F0_PAIR layers take chunks of at most 2^8 input
 // entries: one pair per thread of a 256-thread evaluation CTA.
@@ -117,23 +154,37 @@ struct SciDev {
     u64 *esum;     // PROD: prod_{m>j} (c0_m + c1_m)
 };
 
-// One wave of a PROD SCI: each CTA folds 2^nr entries (the first e rounds in
-// registers, 2^e entries per thread; the rest across the CTA).
+// One wave of a PROD SCI: each CTA takes a chunk of 2^nr entries, nr = kc + kr
+// (kc low coordinates: columns, kr high ones: rows; kr > 0 only with kc = PR_C).
+// wblk, the wave's weights (k_coins; e_m(b) the fold's factor of local
+// coordinate m, L_m the instance's):
+//   kr > 0: colw[x] = prod_{m<kc} e_m(x_m) (2^kc words, the fold of the columns),
+//           roww[y] = prod_{m>=kc} L_m(y_m) (2^kr words, the rows' weight)
+//   message weights of the columns, and of the rows if kr > 0: over the kk
+//           coordinates from a, entry y of round j (y: the other kk - 1 bits)
+//           prod_{m<j} e_{a+m}(y_m) prod_{m>j} L_{a+m}(y_{m-1}), at
+//           word (y / 16) 16 kk + 16 j + y mod 16
+//   e(0), e(1) of the last column coordinate, then of the last row coordinate
+//   outer lo / hi: split table of prod_{m >= r0+nr} L_m over the chunk index
 struct ProdWave {
     u32 circ;
     u32 sci;
-    u32 r0, nr, e;
+    u32 r0, nr, kc, kr;
     u32 nchunks;
     u32 flags;
     u32 no, ho;        // coordinates beyond the chunk (r0+nr..n-1) and their split
-    u32 chal_off;      // challenge of local round k: chal[chal_off + k]
-    u32 pad;
     const u64 *in;     // entries of this wave's table
     u64 *out;          // one folded value per chunk (unused on the last wave)
-    u64 *wblk;         // weight block: Q, E, outer lo, outer hi
+    u64 *wblk;
     u64 *part;         // partials: part[(k * nchunks + chunk) * 2 + t]
     u32 *counter;      // chunks finished (WF_TAIL only; reset by the last)
 };
+// Offsets in wblk.
+__host__ __device__ __forceinline__ u32 pw_roww(u32 kr) { return kr ? 1u << PR_C : 0u; }
+__host__ __device__ __forceinline__ u32 pw_tcol(u32 kr) { return kr ? (1u << PR_C) + (1u << kr) : 0u; }
+__host__ __device__ __forceinline__ u32 pw_trow(u32 kc, u32 kr) { return pw_tcol(kr) + vec_words(kc); }
+__host__ __device__ __forceinline__ u32 pw_last(u32 kc, u32 kr) { return pw_trow(kc, kr) + (kr ? vec_words(kr) : 0u); }
+__host__ __device__ __forceinline__ u32 pw_outer(u32 kc, u32 kr) { return pw_last(kc, kr) + 4; }
 
 // One wave of a GEN SCI.
 struct GenWave {
@@ -199,11 +250,12 @@ struct RoundRef {
     u32 circ;
     u32 sci;
     u32 j;            // round index within the SCI
-    u32 defer;        // TREE phase 2, j >= 1: the message carries the factor 1 - (first challenge of the
-                      // phase), left out of P and B by the first wave's round 0
+    u32 nchunks2;     // TREE phase 2, j >= 1: the PK_TREE2B instance's partials of the round
+    const u64 *part2_pos;
     const u64 *ez;    // eq(z_i, r_P) of the layer
     const u64 *v1;    // V~_{i+1}(r1) of the layer
-    const u64 *ch;    // TREE phases 2 and 3: the first challenge of phase 2
+    const u64 *ch;    // the first challenge of phase 2
+    const u64 *rp0;   // the first challenge of phase 1 (NULL without one)
     const u64 *lc;    // PROD: c0, c1 of round j
     const u64 *kap;   // PROD: kappa_j
     const u64 *esum;  // PROD: esum_j
@@ -292,15 +344,11 @@ struct GatherChunk {
 #define VC_RESULT_WORDS 8  // verifier result words (device)
 
 // ---- launch entry points (implemented in the .cu files) -------------------------
-// An eq table to build and where its point comes from: challenges
-// chal[off ..] (EQ_SRC_CHAL) or the point z_layer (EQ_SRC_Z).
-enum : u32 { EQ_SRC_CHAL = 0, EQ_SRC_Z = 1 };
+// An eq table to build, its point the challenges chal[off ..].
 struct EqJob {
     EqTab t;
     u32 circ;
-    u32 src;
     u32 off;
-    u32 layer;
 };
 
 void launch_params(Globals *G, u64 seed, u64 *tr, const u64 *in, cudaStream_t st);
@@ -309,10 +357,12 @@ const void *vparams_kernel();  // k_vparams, likewise
 void launch_params_batch(Globals *Gs, const CallParams *cp, int n, cudaStream_t st);
 // Every member's inputs into its input layer, one launch (all inputs device memory).
 void launch_gather_inputs(const CallParams *cp, const GatherChunk *chunks, int nchunks, cudaStream_t st);
-// One launch: setup of every circuit (challenges, points, eq(z_i, r_P)),
-// the eq tables and the product weights of the PROD waves.
-void launch_coins(const Globals *Gs, int ncirc, const EqJob *eqjobs, int neq, const SciDev *scis,
-                  const ProdWave *pw, int npw, cudaStream_t st);
+// One launch: setup of every circuit (challenges, points, eq(z_i, r_P), by
+// coin_setups(d) CTAs listed as {circuit, slice}), the eq tables and the
+// product weights of the PROD waves.
+__host__ __device__ __forceinline__ u32 coin_setups(u32 d) { return (d + 7) / 8; }
+void launch_coins(const Globals *Gs, const Item *setups, int nsetup, const EqJob *eqjobs, int neq,
+                  const SciDev *scis, const ProdWave *pw, int npw, cudaStream_t st);
 void launch_eval_layers(const Globals *Gs, const LayerEval *le, const Item *items, int nitems, cudaStream_t st);
 // maxblock: the largest block (entries) of any run layer or tail output in
 // the launch (<= 2048); it sizes the two shared-memory buffers.
@@ -322,6 +372,9 @@ void launch_eval_segs(const Globals *Gs, const EvalSeg *segs, const Item *items,
 void launch_check_canonical(const u64 *x, u64 n, u32 *status, cudaStream_t st);
 void launch_check_inputs(const Globals *Gs, const Item *items, int nitems, cudaStream_t st);
 void launch_build23(const Globals *Gs, const BuildItem *items, int nitems, cudaStream_t st);
+// MATMULT layers' phase-2 factors (BuildItem: MM_ROWS rows of the second matrix).
+#define MM_ROWS 8u
+void launch_mm_tables(const Globals *Gs, const BuildItem *items, int nitems, cudaStream_t st);
 // Explicit layers: an entry w of layer i+1 read by more than BUILD_HEAVY
 // gates is summed after launch_build23 by npieces CTAs of up to
 // BUILD_PIECE gates each (kind 1: its in1 list, 2: its in2 list); each writes

@@ -380,8 +380,8 @@ static void staged_partition(vc_circuit *c, Arena &A)
     };
     split(P.groupsA, c->stA);
     split(P.groupsB, c->stB);
-    c->stBuild.assign(ng + 1, {});
-    for (const BuildItem &b : P.builds) c->stBuild[list_of(b.layer)].push_back(b);
+    c->stMm.assign(ng + 1, {});
+    for (const BuildItem &b : P.mms) c->stMm[list_of(b.layer)].push_back(b);
     c->stEval.assign(d, {});
     for (u32 i = 0; i < d; i++) {
         const u64 blocks = ((u64(1) << c->s[i]) + 255) / 256;
@@ -403,9 +403,9 @@ static void staged_partition(vc_circuit *c, Arena &A)
     };
     take_lists(c->stA, c->d_stA);
     take_lists(c->stB, c->d_stB);
-    c->d_stBuild.assign(ng + 1, nullptr);
+    c->d_stMm.assign(ng + 1, nullptr);
     c->d_stEval.assign(d, nullptr);
-    for (u32 l = 0; l <= ng; l++) c->d_stBuild[l] = A.take<BuildItem>(c->stBuild[l].size() + 1);
+    for (u32 l = 0; l <= ng; l++) c->d_stMm[l] = A.take<BuildItem>(c->stMm[l].size() + 1);
     for (u32 i = 0; i < d; i++) c->d_stEval[i] = A.take<Item>(c->stEval[i].size() + 1);
     c->stctr_off.assign(ng + 1, 0);
     u32 nctr = 0;
@@ -432,7 +432,7 @@ static cudaError_t staged_upload(vc_circuit *c)
         for (size_t g = 0; e == cudaSuccess && g < c->stA[i].size(); g++) e = upload(c->d_stA[i][g], c->stA[i][g]);
     for (size_t i = 0; e == cudaSuccess && i < c->stB.size(); i++)
         for (size_t g = 0; e == cudaSuccess && g < c->stB[i].size(); g++) e = upload(c->d_stB[i][g], c->stB[i][g]);
-    for (size_t l = 0; e == cudaSuccess && l < c->stBuild.size(); l++) e = upload(c->d_stBuild[l], c->stBuild[l]);
+    for (size_t l = 0; e == cudaSuccess && l < c->stMm.size(); l++) e = upload(c->d_stMm[l], c->stMm[l]);
     for (u32 i = 0; e == cudaSuccess && i < c->d; i++) e = upload(c->d_stEval[i], c->stEval[i]);
     u32 nctr = 0;
     for (size_t l = 0; l < c->stA.size(); l++) nctr += 2 * (u32)(c->stA[l].size() + c->stB[l].size());
@@ -515,6 +515,8 @@ static size_t layout(vc_circuit *c, uintptr_t base, uintptr_t hbase)
     // layers and their eq tables
     c->L.assign(d, LayerDev{});
     P.eqjobs.clear();
+    P.setups.clear();
+    for (u32 k = 0; k < coin_setups(d); k++) P.setups.push_back({0u, k});
     c->eq_verify.clear();
     c->explicit_layers.clear();
     for (u32 i = 0; i < d; i++) {
@@ -530,14 +532,20 @@ static size_t layout(vc_circuit *c, uintptr_t base, uintptr_t hbase)
         L.tr_msg = c->tr_msg[i];
         L.tr_q = c->tr_q[i];
         const u64 *r = G.chal + L.chal_off;
-        L.tz = take_eq(A, G.pts + L.z_off, L.s);
-        L.trp = take_eq(A, r, L.s);
-        L.tr1 = take_eq(A, r + L.s, L.sn);
-        L.tr2 = take_eq(A, r + L.s + L.sn, L.sn);
-        P.eqjobs.push_back({L.tz, 0u, EQ_SRC_Z, 0u, i});
-        P.eqjobs.push_back({L.trp, 0u, EQ_SRC_CHAL, L.chal_off, 0u});
-        P.eqjobs.push_back({L.tr1, 0u, EQ_SRC_CHAL, L.chal_off + L.s, 0u});
+        if (needs_eq_rp(L.kind)) {
+            L.trp = take_eq(A, r, L.s);
+            P.eqjobs.push_back({L.trp, 0u, L.chal_off});
+        }
         const bool tabs = needs_tables(L.kind);
+        if (tabs) {
+            L.tr1 = take_eq(A, r + L.s, L.sn);
+            L.tr2 = take_eq(A, r + L.s + L.sn, L.sn);
+            P.eqjobs.push_back({L.tr1, 0u, L.chal_off + L.s});
+        }
+        if (L.kind == W_MATMULT) {
+            L.mu = A.take<u64>(u64(1) << (L.s / 3));
+            L.mei = A.take<u64>(u64(1) << (L.s / 3));
+        }
         L.P2 = tabs ? A.take<u64>(S(i + 1)) : nullptr;
         L.P3 = tabs ? A.take<u64>(S(i + 1)) : nullptr;
         L.B2 = (tabs && L.has_add) ? A.take<u64>(S(i + 1)) : nullptr;
@@ -551,9 +559,9 @@ static size_t layout(vc_circuit *c, uintptr_t base, uintptr_t hbase)
             L.by2_off = A.take<u32>(S(i + 1) + 1);
             L.by2_g = A.take<u32>(S(i));
             c->explicit_layers.push_back(i);
-            c->eq_verify.push_back({L.trp, 0u, EQ_SRC_CHAL, L.chal_off, 0u});
-            c->eq_verify.push_back({L.tr1, 0u, EQ_SRC_CHAL, L.chal_off + L.s, 0u});
-            c->eq_verify.push_back({L.tr2, 0u, EQ_SRC_CHAL, L.chal_off + L.s + L.sn, 0u});
+            c->eq_verify.push_back({L.trp, 0u, L.chal_off});
+            c->eq_verify.push_back({L.tr1, 0u, L.chal_off + L.s});
+            c->eq_verify.push_back({L.tr2, 0u, L.chal_off + L.s + L.sn});
         }
     }
 
@@ -606,17 +614,18 @@ static size_t layout(vc_circuit *c, uintptr_t base, uintptr_t hbase)
         }
     }
 
-    // phase-2/3 table builds: one thread per entry of layer i+1, and a CTA
-    // per entry of an explicit layer that more than BUILD_HEAVY gates read
+    // phase-2/3 table builds of explicit layers: one thread per entry of layer
+    // i+1, and a CTA per entry that more than BUILD_HEAVY gates read; and the
+    // phase-2 factors of MATMULT layers, a warp per row
     P.builds.clear();
     P.heavy.clear();
+    P.mms.clear();
     for (u32 i = 0; i < d; i++) {
+        if (c->kind[i] == W_MATMULT)
+            for (u32 b = 0; b < ((1u << (c->s[i] / 3)) + MM_ROWS - 1) / MM_ROWS; b++) P.mms.push_back({0u, i, b, 0u});
         if (!needs_tables(c->kind[i])) continue;
-        // F0 pair and final layers: a thread per pair of entries of layer i+1
-        const bool pairs = c->kind[i] == W_F0_PAIR || c->kind[i] == W_F0_FINAL;
-        const u64 blocks = ((pairs ? S(i + 1) / 2 : S(i + 1)) + 255) / 256;
+        const u64 blocks = (S(i + 1) + 255) / 256;
         for (u64 b = 0; b < blocks; b++) P.builds.push_back({0u, i, (u32)b, 0u});
-        if (c->kind[i] != W_EXPLICIT) continue;
         for (u64 w = 0; w < S(i + 1); w++)
             for (u32 kind = 1; kind <= 2; kind++) {
                 const auto &off = (kind == 1) ? c->by1_off[i] : c->by2_off[i];
@@ -635,28 +644,85 @@ static size_t layout(vc_circuit *c, uintptr_t base, uintptr_t hbase)
     P.gw.clear();
     P.rounds.clear();
     std::vector<u64> pw_off, gw_off, round_off;
+    struct Tree2Part {
+        u64 round, off;
+        u32 nchunks;
+    };
+    std::vector<Tree2Part> tree2_part;  // PK_TREE2B partials by the round they join
     u64 part_total = 0;
     u32 smax = 0;
     for (u32 i = 0; i <= d; i++) smax = std::max(smax, c->s[i]);
     for (u32 i = 0; i < d; i++) {
         const LayerDev &L = c->L[i];
-        for (u32 ph = 1; ph <= 3; ph++) {
-            const u32 n = (ph == 1) ? c->s[i] : c->s[i + 1];
+        u64 tree2_rounds = 0;  // index of phase 2's first round
+        for (u32 ph = 1; ph <= 4; ph++) {
+            // ph 4: the second instance of a TREE layer's phase 2 (PK_TREE2B),
+            // over the odd entries of layer i+1; its round j belongs to round
+            // j + 1 of phase 2
+            if (ph == 4 && L.kind != W_TREE) continue;
+            const u32 n = (ph == 1) ? c->s[i] : (ph == 4) ? c->s[i + 1] - 1 : c->s[i + 1];
             if (n == 0) continue;
-            const u32 roff = (ph == 1) ? 0 : (ph == 2) ? c->s[i] : c->s[i] + c->s[i + 1];
+            const u32 roff = (ph == 1) ? 0 : (ph == 2) ? c->s[i] : (ph == 4) ? c->s[i] + 1 : c->s[i] + c->s[i + 1];
+            if (ph == 2) tree2_rounds = P.rounds.size();
             SciDev Sc{};
             Sc.circ = 0;
             Sc.n = n;
             Sc.layer = i;
             Sc.chal_off = c->chal_off[i] + roff;
             Sc.tr_off = c->tr_msg[i] + 3ull * roff;
-            if (ph == 1) Sc.kind = PK_PH1;
-            else if (L.kind == W_SQUARE) Sc.kind = (ph == 2) ? PK_GEN_SQ2 : PK_SQ3;
-            else if (L.kind == W_TREE) Sc.kind = (ph == 2) ? PK_GEN_TREE2 : PK_TREE3;
-            else Sc.kind = PK_GEN_TAB;
+            u32 src = GS_NONE;  // the first GEN wave's source
+            const u64 *inP = nullptr, *inB = nullptr;
+            if (ph == 1) {
+                Sc.kind = PK_PH1;
+            } else if (ph == 4) {
+                Sc.kind = PK_TREE2B;
+            } else if (ph == 3) {
+                switch (L.kind) {
+                case W_SQUARE: Sc.kind = PK_SQ3; break;
+                case W_TREE: Sc.kind = PK_TREE3; break;
+                case W_F0_PAIR: Sc.kind = PK_PAIR3; break;
+                case W_F0_FINAL: Sc.kind = PK_FINAL3; break;
+                case W_F0_FIRST: Sc.kind = PK_FIRST3; break;
+                case W_MATMULT: Sc.kind = PK_MM3; break;
+                default:
+                    Sc.kind = PK_GEN_TAB;
+                    inP = L.P3;
+                    inB = L.B3;
+                    break;
+                }
+            } else {
+                // F0 pair and final layers: the first wave's round 0 leaves a
+                // factor out of P if it runs in registers (applied by k_final)
+                const bool regs = std::min(c->cfg.gn_chunk, n) > WV_LOG;
+                Sc.kind = PK_GEN_EZ;
+                switch (L.kind) {
+                case W_SQUARE: src = GS_SQ2; break;
+                case W_TREE: Sc.kind = PK_TREE2; break;
+                case W_F0_PAIR:
+                    src = GS_PAIR2;
+                    if (regs) Sc.kind = PK_GEN_PAIR2;
+                    break;
+                case W_F0_FINAL:
+                    src = GS_FINAL2;
+                    if (regs) Sc.kind = PK_GEN_FINAL2;
+                    break;
+                case W_F0_FIRST: src = GS_FIRST2; break;
+                case W_MATMULT:
+                    Sc.kind = PK_GEN_TAB;
+                    src = GS_MM2;
+                    inP = L.mu;
+                    inB = L.mei;
+                    break;
+                default:
+                    Sc.kind = PK_GEN_TAB;
+                    inP = L.P2;
+                    inB = L.B2;
+                    break;
+                }
+            }
             const u32 sci = (u32)P.scis.size();
             const bool prod = Sc.kind < PK_GEN_FIRST;
-            if (prod) {
+            if (prod && ph != 4) {
                 Sc.Lc = A.take<u64>(2 * n);
                 Sc.kap = A.take<u64>(n);
                 Sc.esum = A.take<u64>(n);
@@ -668,29 +734,25 @@ static size_t layout(vc_circuit *c, uintptr_t base, uintptr_t hbase)
             const u32 split = (c->cfg.pr_split == VC_SPLIT_WIDEST) ? smax : c->cfg.pr_split;
             const u32 C = prod ? ((n < split && c->cfg.pr_chunk > 1) ? c->cfg.pr_chunk - 1 : c->cfg.pr_chunk)
                                : c->cfg.gn_chunk;
-            const u32 M = prod ? (u32)PR_M : (u32)GN_M;
-            const bool tab = Sc.kind == PK_GEN_TAB;
-            const bool tabB = tab && L.has_add;
-            const bool anyB = tabB || Sc.kind == PK_GEN_TREE2;
-            const u64 *inP = tab ? (ph == 2 ? L.P2 : L.P3) : nullptr;
-            const u64 *inB = tabB ? (ph == 2 ? L.B2 : L.B3) : nullptr;
+            const bool tab = needs_tables(L.kind) && ph != 1;  // waits for k_build23
+            const bool anyB = (tab && L.has_add) || src == GS_FIRST2;
             const u64 *inV = (ph == 1) ? L.V : L.Vn;
-            // TREE phase 2 with a first wave in registers: its round 0 leaves
-            // the factor 1 - r_0 out of P and B (applied per round by k_final)
-            const bool defer = Sc.kind == PK_GEN_TREE2 && std::min(C, n) > WV_LOG;
             u32 r0 = 0, g = 0;
             bool tail = false;
             for (u32 w = 0;; w++) {
                 const u32 nr = std::min(C, n - r0);
                 const u32 nchunks = u32(1) << (n - r0 - nr);
                 const bool last = (r0 + nr == n);
-                // entries per thread: all WV threads busy, at most 2^M each; the
-                // register phase works on runs (16 entries PROD, 4 GEN), so a
-                // wave of more than WV threads' entries takes at least one run
-                const u32 run = prod ? 4u : 2u;
-                const u32 e = nr > WV_LOG ? std::min(M, std::max(run, nr - WV_LOG)) : 0u;
+                // GEN: entries per thread: all WV threads busy, at most 2^GN_M
+                // each; the register phase works on runs of 4, so a wave of
+                // more than WV threads' entries takes at least one run
+                const u32 e = nr > WV_LOG ? std::min((u32)GN_M, std::max(2u, nr - WV_LOG)) : 0u;
                 const bool has_tail = !last && (n - r0 - nr) <= C;  // the next wave is one chunk
                 for (u32 k = 0; k < nr; k++) {
+                    if (ph == 4) {  // joins a round of phase 2
+                        tree2_part.push_back({tree2_rounds + r0 + k + 1, part_total + u64(k) * nchunks * nv, nchunks});
+                        continue;
+                    }
                     RoundRef R{};
                     R.tr_pos = Sc.tr_off + 3ull * (r0 + k);
                     R.nchunks = nchunks;
@@ -698,10 +760,10 @@ static size_t layout(vc_circuit *c, uintptr_t base, uintptr_t hbase)
                     R.circ = 0;
                     R.sci = sci;
                     R.j = r0 + k;
-                    R.defer = (defer && R.j >= 1) ? 1u : 0u;
                     R.ez = G.scal + SCAL_EQZRP(i);
                     R.v1 = G.scal + SCAL_V1(i);
                     R.ch = G.chal + c->chal_off[i] + c->s[i];
+                    R.rp0 = c->s[i] ? G.chal + c->chal_off[i] : nullptr;
                     if (prod) {
                         R.lc = Sc.Lc + 2 * R.j;
                         R.kap = Sc.kap + R.j;
@@ -717,17 +779,15 @@ static size_t layout(vc_circuit *c, uintptr_t base, uintptr_t hbase)
                     W.sci = sci;
                     W.r0 = r0;
                     W.nr = nr;
-                    W.e = e;
+                    W.kc = std::min(nr, (u32)PR_C);
+                    W.kr = nr - W.kc;
                     W.nchunks = nchunks;
-                    W.flags = (last ? WF_LAST : 0) | (has_tail ? WF_TAIL : 0);
+                    W.flags = (last ? WF_LAST : 0) | (has_tail ? WF_TAIL : 0) | (ph == 4 && w == 0 ? WF_ODD : 0);
                     W.no = n - r0 - nr;
                     W.ho = (W.no + 1) / 2;
-                    W.chal_off = Sc.chal_off + r0;
                     W.in = inV;
                     W.out = last ? nullptr : A.take<u64>(nchunks);
-                    const u32 kb = W.e ? W.e - 1 : 0;
-                    W.wblk = A.take<u64>(((1u << W.e) - 1) + ((1u << (nr - kb)) - 1) + (1u << W.ho) +
-                                         (1u << (W.no - W.ho)));
+                    W.wblk = A.take<u64>(pw_outer(W.kc, W.kr) + (1u << W.ho) + (1u << (W.no - W.ho)));
                     W.counter = has_tail ? A.take<u32>(1) : nullptr;
                     pw_off.push_back(part_total);
                     idx = (u32)P.pw.size();
@@ -741,8 +801,8 @@ static size_t layout(vc_circuit *c, uintptr_t base, uintptr_t hbase)
                     W.nr = nr;
                     W.e = e;
                     W.nchunks = nchunks;
-                    W.src = (w > 0 || tab) ? GS_NONE : (Sc.kind == PK_GEN_SQ2 ? GS_SQ2 : GS_TREE2);
-                    W.flags = (last ? WF_LAST : 0) | (((w > 0 && anyB) || tabB) ? WF_HASB : 0) |
+                    W.src = w > 0 ? (u32)GS_NONE : src;
+                    W.flags = (last ? WF_LAST : 0) | ((anyB && W.src == GS_NONE) ? WF_HASB : 0) |
                               (has_tail ? WF_TAIL : 0);
                     W.layer = i;
                     W.chal_off = Sc.chal_off + r0;
@@ -774,6 +834,10 @@ static size_t layout(vc_circuit *c, uintptr_t base, uintptr_t hbase)
     for (size_t k = 0; k < P.pw.size(); k++) P.pw[k].part = c->partials + pw_off[k];
     for (size_t k = 0; k < P.gw.size(); k++) P.gw[k].part = c->partials + gw_off[k];
     for (size_t k = 0; k < P.rounds.size(); k++) P.rounds[k].part_pos = c->partials + round_off[k];
+    for (const Tree2Part &t : tree2_part) {
+        P.rounds[t.round].part2_pos = c->partials + t.off;
+        P.rounds[t.round].nchunks2 = t.nchunks;
+    }
     P.outs.assign(1, 0u);
     sort_tasks(P);
 
@@ -838,6 +902,7 @@ void plan_take(Plan &P, Arena &A, bool own_G)
 {
     if (own_G) P.d_G = A.take<Globals>(P.ncirc);
     P.d_checks = A.take<Item>(P.checks.size() + 1);
+    P.d_setups = A.take<Item>(P.setups.size() + 1);
     P.d_eqjobs = A.take<EqJob>(P.eqjobs.size() + 1);
     P.d_segs = A.take<EvalSeg>(P.segs.size() + 1);
     P.d_levs = A.take<LayerEval>(P.levs.size() + 1);
@@ -856,6 +921,7 @@ void plan_take(Plan &P, Arena &A, bool own_G)
     P.d_ctr = A.take<u32>(2 * (P.groupsA.size() + P.groupsB.size()) + 2);
     P.d_lw = A.take<LineWaveDev>(P.lw.size() + 1);
     P.d_builds = A.take<BuildItem>(P.builds.size() + 1);
+    P.d_mms = A.take<BuildItem>(P.mms.size() + 1);
     P.d_heavy = A.take<HeavyItem>(P.heavy.size() + 1);
     P.d_scis = A.take<SciDev>(P.scis.size() + 1);
     P.d_pw = A.take<ProdWave>(P.pw.size() + 1);
@@ -872,8 +938,10 @@ bool plan_valid(const Plan &P)
     const u32 nc = (u32)P.ncirc;
     for (const Item &it : P.checks)
         if (it.wave >= nc) return false;
+    for (const Item &it : P.setups)
+        if (it.wave >= nc) return false;
     for (const EqJob &J : P.eqjobs)
-        if (J.circ >= nc || J.t.n > 30 || (J.src != EQ_SRC_CHAL && J.src != EQ_SRC_Z)) return false;
+        if (J.circ >= nc || J.t.n > 30) return false;
     for (const EvalSeg &S : P.segs)
         if (S.circ >= nc) return false;
     for (const LayerEval &E : P.levs)
@@ -885,8 +953,9 @@ bool plan_valid(const Plan &P)
                        P.lw[k + 1].circ != W.circ || P.lw[k + 1].l0 != W.l0 + W.nl || !W.counter))
             return false;
     }
-    for (const BuildItem &b : P.builds)
-        if (b.circ >= nc) return false;
+    for (const auto *bs : {&P.builds, &P.mms})
+        for (const BuildItem &b : *bs)
+            if (b.circ >= nc) return false;
     for (const HeavyItem &b : P.heavy)
         if (b.circ >= nc || (b.kind != 1 && b.kind != 2) || b.piece >= b.npieces || !b.part || !b.ctr) return false;
     for (const SciDev &S : P.scis)
@@ -894,7 +963,8 @@ bool plan_valid(const Plan &P)
     for (size_t k = 0; k < P.pw.size(); k++) {
         const ProdWave &W = P.pw[k];
         if (W.circ >= nc || W.sci >= P.scis.size() || P.scis[W.sci].circ != W.circ) return false;
-        if (W.nr > PR_CHUNK_LOG || W.e > (u32)PR_M || W.e > W.nr || W.nr - W.e > WV_LOG || (W.e && W.e < 4))
+        if (W.nr < 1 || W.kc + W.kr != W.nr || W.kc > (u32)PR_C || W.kr > (u32)PR_R || (W.kr && W.kc != (u32)PR_C) ||
+            W.r0 + W.nr + W.no != P.scis[W.sci].n || W.ho > W.no)
             return false;
         if ((W.flags & WF_TAIL) && (k + 1 >= P.pw.size() || P.pw[k + 1].nchunks != 1 || P.pw[k + 1].sci != W.sci ||
                                     P.pw[k + 1].r0 != W.r0 + W.nr || !W.counter))
@@ -972,6 +1042,7 @@ cudaError_t plan_upload(Plan &P)
 {
     if (!plan_valid(P)) return cudaErrorInvalidValue;
     cudaError_t e = upload(P.d_checks, P.checks);
+    if (e == cudaSuccess) e = upload(P.d_setups, P.setups);
     if (e == cudaSuccess) e = upload(P.d_eqjobs, P.eqjobs);
     if (e == cudaSuccess) e = upload(P.d_segs, P.segs);
     if (e == cudaSuccess) e = upload(P.d_levs, P.levs);
@@ -985,6 +1056,7 @@ cudaError_t plan_upload(Plan &P)
     if (e == cudaSuccess) e = cudaMemset(P.d_ctr, 0, sizeof(u32) * (2 * (P.groupsA.size() + P.groupsB.size()) + 2));
     if (e == cudaSuccess) e = upload(P.d_lw, P.lw);
     if (e == cudaSuccess) e = upload(P.d_builds, P.builds);
+    if (e == cudaSuccess) e = upload(P.d_mms, P.mms);
     if (e == cudaSuccess) e = upload(P.d_heavy, P.heavy);
     if (e == cudaSuccess) e = upload(P.d_scis, P.scis);
     if (e == cudaSuccess) e = upload(P.d_pw, P.pw);
@@ -999,6 +1071,7 @@ cudaError_t plan_upload_async(Plan &P, cudaStream_t st)
     if (!plan_valid(P)) return cudaErrorInvalidValue;
     cudaError_t e = upload_async(P.d_G, P.h_G, st);
     if (e == cudaSuccess) e = upload_async(P.d_checks, P.checks, st);
+    if (e == cudaSuccess) e = upload_async(P.d_setups, P.setups, st);
     if (e == cudaSuccess) e = upload_async(P.d_eqjobs, P.eqjobs, st);
     if (e == cudaSuccess) e = upload_async(P.d_segs, P.segs, st);
     if (e == cudaSuccess) e = upload_async(P.d_levs, P.levs, st);
@@ -1015,6 +1088,7 @@ cudaError_t plan_upload_async(Plan &P, cudaStream_t st)
         e = cudaMemsetAsync(P.d_ctr, 0, sizeof(u32) * (2 * (P.groupsA.size() + P.groupsB.size()) + 2), st);
     if (e == cudaSuccess) e = upload_async(P.d_lw, P.lw, st);
     if (e == cudaSuccess) e = upload_async(P.d_builds, P.builds, st);
+    if (e == cudaSuccess) e = upload_async(P.d_mms, P.mms, st);
     if (e == cudaSuccess) e = upload_async(P.d_heavy, P.heavy, st);
     if (e == cudaSuccess) e = upload_async(P.d_scis, P.scis, st);
     if (e == cudaSuccess) e = upload_async(P.d_pw, P.pw, st);
@@ -1086,6 +1160,7 @@ void plan_merge(Plan &B, const std::vector<vc_circuit *> &cs)
         const u32 oseg = (u32)B.segs.size(), olev = (u32)B.levs.size(), olw = (u32)B.lw.size();
         const u32 osci = (u32)B.scis.size(), opw = (u32)B.pw.size(), ogw = (u32)B.gw.size();
         for (Item it : P.checks) B.checks.push_back({cj, it.chunk});
+        for (Item it : P.setups) B.setups.push_back({cj, it.chunk});
         for (EqJob J : P.eqjobs) {
             J.circ = cj;
             B.eqjobs.push_back(J);
@@ -1122,6 +1197,10 @@ void plan_merge(Plan &B, const std::vector<vc_circuit *> &cs)
         for (BuildItem b : P.builds) {
             b.circ = cj;
             B.builds.push_back(b);
+        }
+        for (BuildItem b : P.mms) {
+            b.circ = cj;
+            B.mms.push_back(b);
         }
         for (HeavyItem b : P.heavy) {
             b.circ = cj;
@@ -1210,10 +1289,12 @@ void enqueue_plan(Plan &P, cudaStream_t st)
     mark(VC_STAGE_EVAL, 1, st);
     cudaStreamWaitEvent(sa, P.ev_fork, 0);
     mark(VC_STAGE_TABLES, 0, sa);
-    launch_coins(Gs, P.ncirc, P.d_eqjobs, (int)P.eqjobs.size(), P.d_scis, P.d_pw, (int)P.pw.size(), sa);
+    launch_coins(Gs, P.d_setups, (int)P.setups.size(), P.d_eqjobs, (int)P.eqjobs.size(), P.d_scis, P.d_pw, (int)P.pw.size(), sa);
     mark(VC_STAGE_TABLES, 1, sa);
     cudaEventRecord(P.ev_tables, sa);
     cudaStreamWaitEvent(st, P.ev_tables, 0);
+    // MATMULT layers' phase-2 factors (they need the coins and the layer's inputs)
+    launch_mm_tables(Gs, P.d_mms, (int)P.mms.size(), st);
     // line reductions, product-weighted and on-the-fly general waves
     mark(VC_STAGE_WAVES, 0, st);
     if (nA) waves(P.groupsA[0], P.d_groupsA[0], 0);
@@ -1339,10 +1420,10 @@ static void enqueue_staged(vc_circuit &c, cudaStream_t st)
     auto bytes = [&](u32 i) { return (u64(1) << c.s[i]) * sizeof(u64); };
     auto wide = [&](u32 i) { return c.st_slot[i] >= 0; };
     auto run_list = [&](u32 l) {  // the launches of list l (a group of iterations, or the narrow ones)
+        launch_mm_tables(Gs, c.d_stMm[l], (int)c.stMm[l].size(), st);
         for (size_t g = 0; g < c.stA[l].size(); g++)
             launch_waves(Gs, P.d_lw, P.d_pw, P.d_gw, c.d_stA[l][g], (int)c.stA[l][g].size(),
                          c.d_stctr + c.stctr_off[l] + 2 * g, st);
-        if (!c.stBuild[l].empty()) launch_build23(Gs, c.d_stBuild[l], (int)c.stBuild[l].size(), st);
         for (size_t g = 0; g < c.stB[l].size(); g++)
             launch_waves(Gs, P.d_lw, P.d_pw, P.d_gw, c.d_stB[l][g], (int)c.stB[l][g].size(),
                          c.d_stctr + c.stctr_off[l] + 2 * (c.stA[l].size() + g), st);
@@ -1350,7 +1431,7 @@ static void enqueue_staged(vc_circuit &c, cudaStream_t st)
     launch_params(P.d_G, 0, nullptr, nullptr, st);  // arguments set per launch
     cudaEventRecord(P.ev_fork, st);
     cudaStreamWaitEvent(sa, P.ev_fork, 0);
-    launch_coins(Gs, P.ncirc, P.d_eqjobs, (int)P.eqjobs.size(), P.d_scis, P.d_pw, (int)P.pw.size(), sa);
+    launch_coins(Gs, P.d_setups, (int)P.setups.size(), P.d_eqjobs, (int)P.eqjobs.size(), P.d_scis, P.d_pw, (int)P.pw.size(), sa);
     cudaEventRecord(P.ev_tables, sa);
     // evaluation; holder[s] = the wide layer in slot s (-1: none yet)
     std::vector<int> holder(c.st_nslots, -1);
@@ -1415,10 +1496,10 @@ static void enqueue_windowed(vc_circuit &c, cudaStream_t st)
     const Globals *Gs = P.d_G;
     cudaStream_t sa = P.aux;
     auto run_list = [&](u32 l) {
+        launch_mm_tables(Gs, c.d_stMm[l], (int)c.stMm[l].size(), st);
         for (size_t g = 0; g < c.stA[l].size(); g++)
             launch_waves(Gs, P.d_lw, P.d_pw, P.d_gw, c.d_stA[l][g], (int)c.stA[l][g].size(),
                          c.d_stctr + c.stctr_off[l] + 2 * g, st);
-        if (!c.stBuild[l].empty()) launch_build23(Gs, c.d_stBuild[l], (int)c.stBuild[l].size(), st);
         for (size_t g = 0; g < c.stB[l].size(); g++)
             launch_waves(Gs, P.d_lw, P.d_pw, P.d_gw, c.d_stB[l][g], (int)c.stB[l][g].size(),
                          c.d_stctr + c.stctr_off[l] + 2 * (c.stA[l].size() + g), st);
@@ -1426,7 +1507,7 @@ static void enqueue_windowed(vc_circuit &c, cudaStream_t st)
     launch_params(P.d_G, 0, nullptr, nullptr, st);  // arguments set per launch
     cudaEventRecord(P.ev_fork, st);
     cudaStreamWaitEvent(sa, P.ev_fork, 0);
-    launch_coins(Gs, P.ncirc, P.d_eqjobs, (int)P.eqjobs.size(), P.d_scis, P.d_pw, (int)P.pw.size(), sa);
+    launch_coins(Gs, P.d_setups, (int)P.setups.size(), P.d_eqjobs, (int)P.eqjobs.size(), P.d_scis, P.d_pw, (int)P.pw.size(), sa);
     cudaEventRecord(P.ev_tables, sa);
     launch_check_inputs(Gs, P.d_checks, (int)P.checks.size(), st);  // the inputs are in layer d
     bool coins = false;
@@ -1486,6 +1567,7 @@ int count_launches(const Plan &P)
     for (size_t k = 0; k < P.seg_items.size(); k++) n += (!P.seg_items[k].empty()) + (!P.lev_items[k].empty());
     for (const auto &v : P.groupsA) n += !v.empty();
     n += !P.builds.empty();
+    n += !P.mms.empty();
     n += !P.heavy.empty();
     for (const auto &v : P.groupsB) n += !v.empty();
     return n + 1;  // final
@@ -1941,7 +2023,7 @@ static cudaError_t pergate_launch(vc_circuit *c, cudaStream_t st)
             launch_eval_segs(P.d_G, P.d_segs, P.d_seg_items[k], (int)P.seg_items[k].size(), P.seg_maxblock[k], P.cap);
             launch_eval_layers(P.d_G, P.d_levs, P.d_lev_items[k], (int)P.lev_items[k].size(), P.cap);
         }
-        launch_coins(P.d_G, 1, nullptr, 0, nullptr, nullptr, 0, P.cap);
+        launch_coins(P.d_G, P.d_setups, (int)P.setups.size(), nullptr, 0, nullptr, nullptr, 0, P.cap);
         launch_pergate(P.d_G, c->d_pg, (int)c->d, c->d_pg_blk, c->pg_nblk, c->d_pg_lblk, c->pg_nlblk, c->pg_rounds,
                        P.cap);
         cudaGraph_t g = nullptr;
@@ -2079,7 +2161,7 @@ extern "C" vc_status vc_verify(vc_circuit *c, const uint64_t *inputs, uint64_t s
             launch_vparams(c->d_Gv, c->d_vp, 0, nullptr, nullptr, nullptr, c->d_result, cs);
             cudaEventRecord(c->P.ev_fork, cs);
             cudaStreamWaitEvent(c->P.aux, c->P.ev_fork, 0);
-            launch_coins(c->d_Gv, 1, c->d_eq_verify, (int)c->eq_verify.size(), nullptr, nullptr, 0, cs);
+            launch_coins(c->d_Gv, c->P.d_setups, (int)c->P.setups.size(), c->d_eq_verify, (int)c->eq_verify.size(), nullptr, nullptr, 0, cs);
             launch_verify(c->d_Gv, c->Gv, c->Vd, c->s[c->d], c->s[0], c->d_vwire, (int)c->vwire.size(),
                           c->P.aux, c->P.ev_tables, cs);
         };
@@ -2123,7 +2205,7 @@ extern "C" vc_status vc_verify_input(vc_circuit *c, const uint64_t *inputs, uint
             cudaStreamWaitEvent(c->P.aux, c->P.ev_fork, 0);
             launch_verify_input(c->d_Gv, c->Gv, c->Vd, c->s[c->d], c->s[0], c->P.aux);
             cudaEventRecord(c->P.ev_tables, c->P.aux);
-            launch_coins(c->d_Gv, 1, nullptr, 0, nullptr, nullptr, 0, cs);
+            launch_coins(c->d_Gv, c->P.d_setups, (int)c->P.setups.size(), nullptr, 0, nullptr, nullptr, 0, cs);
             cudaStreamWaitEvent(cs, c->P.ev_tables, 0);
         };
         e = capture_graph(c->P.cap, enqueue, &c->vin_exec, vparams_in_kernel(), &c->vin_graph, &c->vin_node,
@@ -2159,7 +2241,7 @@ extern "C" vc_status vc_verify_transcript(vc_circuit *c, uint64_t seed, const ui
     if (e != cudaSuccess) return VC_ECUDA;
     // plain launches with the per-call pointers as arguments (one launch for
     // structured circuits): nothing to capture, nothing to write first
-    launch_coins(c->d_Gv, 0, c->d_eq_verify, (int)c->eq_verify.size(), nullptr, nullptr, 0, st);
+    launch_coins(c->d_Gv, nullptr, 0, c->d_eq_verify, (int)c->eq_verify.size(), nullptr, nullptr, 0, st);
     launch_verify_transcript(c->d_Gv, c->Gv, c->Vd, c->s[c->d], c->s[0], c->d_vwire, (int)c->vwire.size(), dtr,
                              ka ? accept : nullptr, st);
     return verifier_finish(c, ka && kt && !c->vin_sync, ka, accept, st);
@@ -2187,7 +2269,7 @@ static cudaError_t pv_capture(vc_circuit *c)
     enqueue_plan(c->P, cs);
     cudaStreamWaitEvent(c->pv_vs, c->pv_fork, 0);
     launch_vparams(c->d_Gv, c->d_vp, 0, nullptr, nullptr, nullptr, c->d_result, c->pv_vs);
-    launch_coins(c->d_Gv, 1, c->d_eq_verify, (int)c->eq_verify.size(), nullptr, nullptr, 0, c->pv_vs);
+    launch_coins(c->d_Gv, c->P.d_setups, (int)c->P.setups.size(), c->d_eq_verify, (int)c->eq_verify.size(), nullptr, nullptr, 0, c->pv_vs);
     launch_verify_input(c->d_Gv, c->Gv, c->Vd, c->s[c->d], c->s[0], c->pv_vs);
     cudaEventRecord(c->pv_join, c->pv_vs);
     cudaStreamWaitEvent(cs, c->pv_join, 0);
