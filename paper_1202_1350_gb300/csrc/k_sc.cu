@@ -89,9 +89,15 @@ __device__ __forceinline__ u64 warp_sum32(u64 (&v)[32])
 
 #define WV_NT 128
 
+#define PR_RING 4  // rows per thread in flight
+
 struct ProdSmem {
-    u64 u[8][1 << PR_C];       // row groups' column sums
+    union {
+        ulonglong2 ring[PR_RING][4][WV_NT];  // each thread's entries of its next rows (its own copies)
+        u64 u[8][1 << PR_C];                 // row groups' column sums
+    };
     u64 f[16][(1 << PR_R) + 1];  // column groups' row sums
+    u64 rw[1 << PR_R];
     u64 U[1 << PR_C], F[1 << PR_R];
 };
 
@@ -127,13 +133,21 @@ extern __shared__ __align__(16) unsigned char wv_dyn[];  // a WaveSmem
 __device__ __forceinline__ ulonglong2 ld_in(const ulonglong2 *p, bool ext) { return ext ? __ldg(p) : __ldcg(p); }
 __device__ __forceinline__ u64 ld_in(const u64 *p, bool ext) { return ext ? __ldg(p) : __ldcg(p); }
 
-// A load that stays where it is written: weights that a loop needs in every
-// pass and that cost more as registers kept through it than as L1 hits.
-__device__ __forceinline__ ulonglong2 ld_again(const ulonglong2 *p)
+// Asynchronous copies to shared memory: 16 bytes through L2 (also what other
+// CTAs of this launch wrote), or 8 bytes through L1 (a first wave's input).
+__device__ __forceinline__ void cp16(void *dst, const void *src)
 {
-    ulonglong2 t;
-    asm volatile("ld.global.nc.v2.u64 {%0, %1}, [%2];" : "=l"(t.x), "=l"(t.y) : "l"(p));
-    return t;
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((u32)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp8(void *dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((u32)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_wait()
+{
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
 // Bring the line holding p into L1 ahead of its load (no register cost).
@@ -143,6 +157,12 @@ __device__ __forceinline__ void prefetch_l1(const void *p) { asm volatile("prefe
 __device__ __forceinline__ u64 cta_sum4(const u64 *a, const u64 *b, const u64 *c, const u64 *d)
 {
     return wred(*a + *b + *c + *d);
+}
+
+// The next task of the CTA (thread 0; ctr NULL: the CTA keeps the one it has).
+__device__ __forceinline__ int claim_task(u32 *ctr)
+{
+    return (ctr && threadIdx.x == 0) ? (int)(gridDim.x + atomicAdd(ctr, 1u)) : 0;
 }
 
 // ---- PROD -----------------------------------------------------------------------
@@ -200,7 +220,7 @@ __device__ __forceinline__ void vec_weights(const u64 *T, u32 kk, bool use, u64 
 
 // One chunk of a PROD wave (each kind is a function of its own: its registers
 // are allocated without those of the others, and there is one copy of its code).
-__device__ __noinline__ void prod_chunk(const ProdWave &W, u32 chunk)
+__device__ __noinline__ int prod_chunk(const ProdWave &W, u32 chunk, u32 *ctr)
 {
     ProdSmem &sm = reinterpret_cast<WaveSmem *>(wv_dyn)->prod;
     const u32 tid = threadIdx.x;
@@ -208,76 +228,79 @@ __device__ __noinline__ void prod_chunk(const ProdWave &W, u32 chunk)
     const bool ext = W.r0 == 0, odd = (W.flags & WF_ODD) != 0;
     const u64 *blk = W.wblk;
     const u64 *in = W.in + ((u64)chunk << (odd ? nr + 1 : nr));
-    u64 wc[4], wr[4], ea, eb, el;
-    auto weights = [&]() {
-        vec_weights(blk + pw_tcol(kr), kc, true, wc);
-        vec_weights(blk + pw_trow(kc, kr), kr, kr != 0, wr);
-        const u64 *olo = blk + pw_outer(kc, kr);  // weight of the coordinates beyond the chunk
-        ea = __ldg(olo + (chunk & ((1u << W.ho) - 1)));
-        eb = __ldg(olo + (1u << W.ho) + (chunk >> W.ho));
-        el = __ldg(blk + pw_last(kc, kr) + (kr ? 2 : 0) + ((tid >> 3) & 1));  // fold factor of the last coordinate
+    // columns 2c + 32 q, + 1 of rows rg, rg + 8, .., each thread's next
+    // PR_RING rows on their way into shared memory while it works: an L2 load
+    // takes about two rows' products
+    const u32 c = tid & 15, rg = tid >> 4, nrow = kr ? 1u << kr : 0u;
+    auto fetch = [&](u32 row) {
+        if (row < nrow) {
+            ulonglong2 *dst = &sm.ring[(row >> 3) & (PR_RING - 1)][0][tid];
+            const ulonglong2 *src = reinterpret_cast<const ulonglong2 *>(in);
+            if (odd) {
+                src += 2 * (row * 64 + c);
+#pragma unroll
+                for (int q = 0; q < 4; q++) {
+                    cp8(&dst[q * WV_NT].x, &src[32 * q].y);
+                    cp8(&dst[q * WV_NT].y, &src[32 * q + 1].y);
+                }
+            } else {
+                src += row * 64 + c;
+#pragma unroll
+                for (int q = 0; q < 4; q++) cp16(&dst[q * WV_NT], &src[16 * q]);
+            }
+        }
+        cp_commit();
     };
+    if (kr) {
+#pragma unroll
+        for (u32 i = 0; i < PR_RING; i++) fetch(rg + 8 * i);
+        if (tid < nrow) sm.rw[tid] = __ldg(blk + pw_roww(kr) + tid);
+    }
+    u64 wc[4], wr[4];
+    vec_weights(blk + pw_tcol(kr), kc, true, wc);
+    vec_weights(blk + pw_trow(kc, kr), kr, kr != 0, wr);
+    const u64 *olo = blk + pw_outer(kc, kr);  // weight of the coordinates beyond the chunk
+    const u64 ea = __ldg(olo + (chunk & ((1u << W.ho) - 1))), eb = __ldg(olo + (1u << W.ho) + (chunk >> W.ho));
+    // fold factor of the last coordinate
+    const u64 el = __ldg(blk + pw_last(kc, kr) + (kr ? 2 : 0) + ((tid >> 3) & 1));
     if (kr == 0) {
-        weights();
         if (tid < (1u << kc)) sm.U[tid] = ld_in(in + (odd ? 2 * tid + 1 : tid), ext);
         __syncthreads();
     } else {
-        // columns 2c + 32 q, + 1 of rows rg, rg + 8, ..
-        const u32 c = tid & 15, rg = tid >> 4, nrow = 1u << kr;
-        const u64 *roww = blk + pw_roww(kr);
-        const ulonglong2 *src = reinterpret_cast<const ulonglong2 *>(in);
-        auto load = [&](u32 row, ulonglong2 (&t)[4]) {
+        ulonglong2 cw[4];
 #pragma unroll
-            for (int q = 0; q < 4; q++) {
-                if (odd) {
-                    const ulonglong2 *s2 = src + 2 * (row * 64 + 16 * q + c);
-                    t[q] = make_ulonglong2(ld_in(s2, ext).y, ld_in(s2 + 1, ext).y);
-                } else {
-                    t[q] = ld_in(src + row * 64 + 16 * q + c, ext);
-                }
-            }
-        };
+        for (int q = 0; q < 4; q++) cw[q] = __ldg(reinterpret_cast<const ulonglong2 *>(blk) + c + 16 * q);
         acc128 u[8];
 #pragma unroll
         for (int q = 0; q < 8; q++) acc_zero(u[q]);
-        ulonglong2 v[4];
-        u64 rw = 0;
-        if (rg < nrow) {
-            rw = __ldg(roww + rg);
-            load(rg, v);
-        }
+        __syncthreads();  // sm.rw
 #pragma unroll 1
         for (u32 row = rg; row < nrow; row += 8) {
-            ulonglong2 n[4];  // the next row's entries on their way during this row's products
-            u64 rn = 0;
-            const bool more = row + 8 < nrow;
-            if (more) {
-                rn = __ldg(roww + row + 8);
-                load(row + 8, n);
-            }
+            cp_wait<PR_RING - 1>();
+            const ulonglong2 *src = &sm.ring[(row >> 3) & (PR_RING - 1)][0][tid];
+            ulonglong2 v[4];
+#pragma unroll
+            for (int q = 0; q < 4; q++) v[q] = src[q * WV_NT];
+            const u64 rw = sm.rw[row];
+            fetch(row + 8 * PR_RING);
             acc128 f0, f1;
             acc_zero(f0);
             acc_zero(f1);
 #pragma unroll
             for (int q = 0; q < 4; q++) {
-                const ulonglong2 cw = ld_again(reinterpret_cast<const ulonglong2 *>(blk) + c + 16 * q);
-                mac(f0, cw.x, v[q].x);
-                mac(f1, cw.y, v[q].y);
+                mac(f0, cw[q].x, v[q].x);
+                mac(f1, cw[q].y, v[q].y);
                 mac(u[2 * q], rw, v[q].x);
                 mac(u[2 * q + 1], rw, v[q].y);
             }
             sm.f[c][row] = wred(acc_red7(f0) + acc_red7(f1));
-            if (more) {
-                rw = rn;
-#pragma unroll
-                for (int q = 0; q < 4; q++) v[q] = n[q];
-            }
         }
+        cp_wait<0>();
+        __syncthreads();  // the ring's memory becomes sm.u
 #pragma unroll
         for (int q = 0; q < 4; q++)
             *reinterpret_cast<ulonglong2 *>(&sm.u[rg][2 * c + 32 * q]) =
                 make_ulonglong2(acc_red(u[2 * q]), acc_red(u[2 * q + 1]));
-        weights();
         __syncthreads();
         {
             const u64 a = wred(sm.u[0][tid] + sm.u[1][tid] + sm.u[2][tid] + sm.u[3][tid]);
@@ -294,6 +317,7 @@ __device__ __noinline__ void prod_chunk(const ProdWave &W, u32 chunk)
         }
         __syncthreads();
     }
+    const int next = claim_task(ctr);
     const u32 j = tid >> 4, t = (tid >> 3) & 1;
     const bool writer = (tid & 7) == 0;
     const u64 ech = f_mul(ea, eb);
@@ -308,6 +332,7 @@ __device__ __noinline__ void prod_chunk(const ProdWave &W, u32 chunk)
         const u64 x = wmul(h, el), y = wred(x + __shfl_xor_sync(0xffffffffu, x, 8));
         if (tid == 16 * ((kr ? kr : kc) - 1)) W.out[chunk] = y;
     }
+    return next;
 }
 
 // ---- GEN ------------------------------------------------------------------------
@@ -483,19 +508,21 @@ __device__ __forceinline__ void gen_regs_runs(const Globals &G, const GenWave &W
         lo = T.lo + (x & ((1ull << T.h) - 1));
         hi = T.hi[x >> T.h];
     }
+    // the second line of each of the thread's tables (32 entries are two)
+    // comes while the first is used
+    if (nruns > 4) {
+        prefetch_l1(W.inV + x0 + 16);
+        if (lohi) prefetch_l1(lo + (src == GS_FINAL2 ? 8 : 16));
+        if (src == GS_NONE) {
+            prefetch_l1(W.inP + x0 + 16);
+            if (hasB) prefetch_l1(W.inB + x0 + 16);
+        }
+    }
     u64 p0 = 0, v0 = 0, b0 = 0, p1 = 0, v1 = 0, b1 = 0, p2 = 0, v2 = 0, b2 = 0;  // pending: rounds 2, 3, 4
     u64 tp = 0, tv = 0, tb = 0;
     // a rolled loop keeps the kernel small (instruction-cache bound when unrolled)
 #pragma unroll 1
     for (u32 sub = 0; sub < nruns; sub++) {
-        if (sub + 1 < nruns) {
-            const u64 xn = x0 + 4 * (sub + 1);
-            prefetch_l1(W.inV + xn);
-            if (src == GS_NONE) {
-                prefetch_l1(W.inP + xn);
-                if (hasB) prefetch_l1(W.inB + xn);
-            }
-        }
         if (src == GS_PAIR2 || src == GS_FINAL2) {
             const ulonglong2 *sv = reinterpret_cast<const ulonglong2 *>(W.inV + x0 + 4 * sub);
             const ulonglong2 va = __ldg(sv), vb = __ldg(sv + 1);
@@ -644,7 +671,7 @@ __device__ __forceinline__ void gen_cross(bool hasB, u64 &p, u64 &v, u64 &b, u32
 }
 
 // One chunk of a GEN wave.
-__device__ __noinline__ void gen_chunk(const Globals &G, const GenWave &W, u32 chunk)
+__device__ __noinline__ int gen_chunk(const Globals &G, const GenWave &W, u32 chunk, u32 *ctr)
 {
     GenSmem &sm = reinterpret_cast<WaveSmem *>(wv_dyn)->gen;
     const u32 tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -681,6 +708,7 @@ __device__ __noinline__ void gen_chunk(const Globals &G, const GenWave &W, u32 c
             bv = t.y;
         }
     }
+    const int next = claim_task(ctr);
     gen_cross(hasB || W.src == GS_FIRST2, pv, vv, bv, e, tid, na, nr, sm);
     __syncthreads();
     if (tid < 3 * nr) {
@@ -693,6 +721,7 @@ __device__ __noinline__ void gen_chunk(const Globals &G, const GenWave &W, u32 c
         W.outV[chunk] = sm.lvl[1][0];
         if (W.outB) W.outB[chunk] = sm.lvl[2][0];
     }
+    return next;
 }
 
 // ---- line reduction -----------------------------------------------------------------
@@ -743,7 +772,7 @@ __device__ __forceinline__ u64 line_coef(const u64 *A, const u64 *B, u32 deg, u3
 }
 
 // One chunk of one line wave, by the whole CTA.
-__device__ __noinline__ void line_chunk(const Globals &G, const LineWaveDev &W, u32 chunk)
+__device__ __noinline__ int line_chunk(const Globals &G, const LineWaveDev &W, u32 chunk, u32 *ctr)
 {
     LineSmem &sm = reinterpret_cast<WaveSmem *>(wv_dyn)->line;
     const u32 tid = threadIdx.x;
@@ -775,7 +804,7 @@ __device__ __noinline__ void line_chunk(const Globals &G, const LineWaveDev &W, 
                 u64 s0[6] = {0, 0, 0, 0, 0, 0}, s1[6] = {0, 0, 0, 0, 0, 0};
 #pragma unroll 1
                 for (int run = 0; run < 8; run++) {
-                    if (run < 7) prefetch_l1(src + 4 * (run + 1));
+                    if (!(run & 1) && run < 6) prefetch_l1(src + 4 * (run + 2));  // the next line
                     u64 v[8];
 #pragma unroll
                     for (int t = 0; t < 4; t++) {
@@ -834,6 +863,7 @@ __device__ __noinline__ void line_chunk(const Globals &G, const LineWaveDev &W, 
         k0 = 1;
     }
     __syncthreads();
+    const int next = claim_task(ctr);
     u64 *cur = sm.bufA, *nxt = sm.bufB;
     u32 k = k0;
     if (m == WV_NT && deg == LN_E && k + 5 <= W.nl) {
@@ -892,6 +922,7 @@ __device__ __noinline__ void line_chunk(const Globals &G, const LineWaveDev &W, 
         }
         if (tid == 0) G.scal[SCAL_V1(W.layer)] = wcanon(cur[0]);
     }
+    return next;
 }
 
 // ---- the persistent launch ------------------------------------------------------------
@@ -925,31 +956,32 @@ __global__ void __launch_bounds__(WV_NT, WV_MINB) k_waves(const Globals *Gs, con
     // drains (it waits for the whole launch before it reads what it wrote)
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     // a CTA's first task is its own index (the grid has at most ntasks CTAs);
-    // the counter hands out the rest, each fetched while the task before it runs
+    // the counter hands out the rest, each claimed in the last part of the task
+    // before it: earlier, and a long task would hold back one that an idle CTA
+    // could run; later, and every task would wait for the counter
     int ti = blockIdx.x;
     for (;;) {
         const Task tk = tasks[ti];
         int next = 0;
-        if (threadIdx.x == 0) next = (int)(gridDim.x + atomicAdd(&ctr[0], 1u));
         if (tk.type == TK_LINE) {
             const LineWaveDev &W = lw[tk.wave];
             const Globals &G = Gs[W.circ];
-            line_chunk(G, W, tk.chunk);
-            if (W.tail && wave_done(W.counter, W.nchunks, s_flag)) line_chunk(G, lw[tk.wave + 1], 0);
+            next = line_chunk(G, W, tk.chunk, ctr);
+            if (W.tail && wave_done(W.counter, W.nchunks, s_flag)) line_chunk(G, lw[tk.wave + 1], 0, nullptr);
         } else if (tk.type == TK_PROD) {
             const ProdWave &W = pw[tk.wave];
-            prod_chunk(W, tk.chunk);
+            next = prod_chunk(W, tk.chunk, ctr);
             if ((W.flags & WF_TAIL) && wave_done(W.counter, W.nchunks, s_flag)) {
                 __syncthreads();
-                prod_chunk(pw[tk.wave + 1], 0);
+                prod_chunk(pw[tk.wave + 1], 0, nullptr);
             }
         } else {
             const GenWave &W = gw[tk.wave];
             const Globals &G = Gs[W.circ];
-            gen_chunk(G, W, tk.chunk);
+            next = gen_chunk(G, W, tk.chunk, ctr);
             if ((W.flags & WF_TAIL) && wave_done(W.counter, W.nchunks, s_flag)) {
                 __syncthreads();
-                gen_chunk(G, gw[tk.wave + 1], 0);
+                gen_chunk(G, gw[tk.wave + 1], 0, nullptr);
             }
         }
         if (threadIdx.x == 0) s_task = next;
