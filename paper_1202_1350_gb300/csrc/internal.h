@@ -10,9 +10,11 @@
 #include "vc.h"
 
 constexpr u32 WV_LOG = 7;                  // log2 of the threads of a wave CTA
-constexpr u32 PR_CHUNK_LOG = PR_C + PR_R;    // rounds of one PROD chunk
+constexpr u32 PR_CHUNK_LOG = 13;             // rounds of one PROD chunk, and
+constexpr u32 PR_CHUNK_WIDE = PR_C + PR_R;   // of one in a wide instance
 constexpr u32 GN_CHUNK_LOG = GN_M + WV_LOG;  // rounds of one GEN chunk (2^GN_M entries per thread)
 constexpr u32 LN_CHUNK0_LOG = 6 + WV_LOG;    // coordinates of a first line-wave chunk (64 entries per thread)
+constexpr u32 LN_XTRA = 2;                   // more coordinates of a first line-wave chunk (256 entries per thread)
 constexpr u32 LN_CHUNKW_LOG = WV_LOG;        // coordinates of a later line-wave chunk (one polynomial per thread)
 
 // Tile shapes of a circuit's plan (the autotuner's knobs): rounds folded

@@ -326,11 +326,53 @@ __device__ void coins_prep(const Globals &G, bool rej, const SciDev &S, const Pr
     }
 }
 
+// Line-weight role, one line wave: the weight polynomials over its kk
+// coordinates (LineWaveDev::wt), each a product of a polynomial over the lower
+// half of the coordinates and one over the upper half.
+__device__ void coins_line(const Globals &G, bool rej, const LineWaveDev &W)
+{
+    __shared__ u64 a[8], b[8];
+    __shared__ u64 part[24][5];  // 16 lower, 8 upper polynomials of degree <= 4
+    const u32 tid = threadIdx.x, kk = W.kk, h = (kk + 1) / 2, g = kk - h;
+    if (tid < kk) {
+        const u32 k = W.l0 + W.e + tid;
+        const u64 x = chal_of(G, rej, W.a_off + k);
+        a[tid] = x;
+        b[tid] = f_sub(chal_of(G, rej, W.b_off + k), x);
+    }
+    __syncthreads();
+    const bool up = tid >= 16;
+    const u32 m0 = up ? h : 0, nm = up ? g : h, y = up ? tid - 16 : tid;
+    if (tid < 24 && y < (1u << nm)) {
+        u64 *q = part[tid];
+        q[0] = 1;
+#pragma unroll 1
+        for (u32 m = 0; m < nm; m++) {
+            const bool one = (y >> m) & 1;  // l_m = a + b t, 1 - l_m
+            const u64 c0 = one ? a[m0 + m] : f_sub(1, a[m0 + m]), c1 = one ? b[m0 + m] : f_neg(b[m0 + m]);
+            q[m + 1] = f_mul(c1, q[m]);
+#pragma unroll 1
+            for (u32 j = m; j > 0; j--) q[j] = f_add(f_mul(c0, q[j]), f_mul(c1, q[j - 1]));
+            q[0] = f_mul(c0, q[0]);
+        }
+    }
+    __syncthreads();
+#pragma unroll 1
+    for (u32 idx = tid; idx < ((kk + 1) << kk); idx += CN_NT) {
+        const u32 y2 = idx & ((1u << kk) - 1), c = idx >> kk;
+        const u64 *lo = part[y2 & ((1u << h) - 1)], *hi = part[16 + (y2 >> h)];
+        u64 v = 0;
+#pragma unroll 1
+        for (u32 j = c > h ? c - h : 0; j <= c && j <= g; j++) v = f_add(v, f_mul(lo[c - j], hi[j]));
+        W.wt[idx] = v;
+    }
+}
+
 // CTAs [0, nsetup): setup, slice `chunk` of circuit `wave` of each item (8
-// layers a slice); then one per eq job; then one per PROD wave.
+// layers a slice); then one per eq job; one per PROD wave; one per line wave.
 __global__ void __launch_bounds__(CN_NT) k_coins(const Globals *Gs, const Item *setups, int nsetup,
                                                  const EqJob *eqjobs, int neq, const SciDev *scis,
-                                                 const ProdWave *pw)
+                                                 const ProdWave *pw, int npw, const LineWaveDev *lw)
 {
     int b = blockIdx.x;
     if (b < nsetup) {
@@ -347,14 +389,20 @@ __global__ void __launch_bounds__(CN_NT) k_coins(const Globals *Gs, const Item *
         return;
     }
     b -= neq;
-    const ProdWave &W = pw[b];
+    if (b < npw) {
+        const ProdWave &W = pw[b];
+        const Globals &G = Gs[W.circ];
+        coins_prep(G, draws_rejected(G), scis[W.sci], W);
+        return;
+    }
+    const LineWaveDev &W = lw[b - npw];
     const Globals &G = Gs[W.circ];
-    coins_prep(G, draws_rejected(G), scis[W.sci], W);
+    coins_line(G, draws_rejected(G), W);
 }
 
 void launch_coins(const Globals *Gs, const Item *setups, int nsetup, const EqJob *eqjobs, int neq,
-                  const SciDev *scis, const ProdWave *pw, int npw, cudaStream_t st)
+                  const SciDev *scis, const ProdWave *pw, int npw, const LineWaveDev *lw, int nlw, cudaStream_t st)
 {
-    const int grid = nsetup + neq + npw;
-    if (grid > 0) k_coins<<<grid, CN_NT, 0, st>>>(Gs, setups, nsetup, eqjobs, neq, scis, pw);
+    const int grid = nsetup + neq + npw + nlw;
+    if (grid > 0) k_coins<<<grid, CN_NT, 0, st>>>(Gs, setups, nsetup, eqjobs, neq, scis, pw, npw, lw);
 }

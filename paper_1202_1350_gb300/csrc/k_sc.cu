@@ -89,33 +89,35 @@ __device__ __forceinline__ u64 warp_sum32(u64 (&v)[32])
 
 #define WV_NT 128
 
+#ifndef PR_RING
 #define PR_RING 4  // rows per thread in flight
+#endif
 
 struct ProdSmem {
     union {
         ulonglong2 ring[PR_RING][4][WV_NT];  // each thread's entries of its next rows (its own copies)
         u64 u[8][1 << PR_C];                 // row groups' column sums
     };
-    u64 f[16][(1 << PR_R) + 1];  // column groups' row sums
+    u64 f[8][(1 << PR_R) + 1];   // column groups' row sums
     u64 rw[1 << PR_R];
     u64 U[1 << PR_C], F[1 << PR_R];
 };
 
 struct GenSmem {
     u64 r[32];
-    u64 lvl[3][WV_NT / 32];
-    u64 w[WV_NT / 32][40];
-    u64 hs[9][WV_NT];  // per-thread sums of in-register rounds 2..4 (kept out of registers)
+    u64 lvl[3];
+    u64 w[WV_NT / 32][16];  // per-warp sums of the in-register rounds
+    u64 hs[9][WV_NT];       // per-thread sums of in-register rounds 2..4 (kept out of registers)
+    u64 x[3][WV_NT];        // the threads' folded triples
+    u64 c[3][WV_NT + 4];    // cross rounds' pair terms: round kk's at 2 (64 - (64 >> kk)) ..
 };
 
-#define LN_E 6        // line: coordinates folded per thread in registers (first wave)
-#define LN_BUFA 2048  // line: shared-memory polynomial buffers (coefficients): a later
-#define LN_BUFB 1024  // wave's first level is 64 pairs x <= 32 coefficients
-
 struct LineSmem {
-    u64 la[32], lb[32];  // a_k and b_k for the wave's coordinates
-    u64 bufA[LN_BUFA];
-    u64 bufB[LN_BUFB];
+    u64 a[8], b[8];          // a_k and b_k of the coordinates folded in registers
+    // the threads' polynomials, coefficient c in row c, then their products'
+    // (a row length that spreads the sum's reads over the banks)
+    u64 part[32][WV_NT + 4];
+    u64 res[32];
 };
 
 union WaveSmem {
@@ -293,7 +295,9 @@ __device__ __noinline__ int prod_chunk(const ProdWave &W, u32 chunk, u32 *ctr)
                 mac(u[2 * q], rw, v[q].x);
                 mac(u[2 * q + 1], rw, v[q].y);
             }
-            sm.f[c][row] = wred(acc_red7(f0) + acc_red7(f1));
+            u64 f = wred(acc_red7(f0) + acc_red7(f1));
+            f = wred(f + __shfl_xor_sync(0xFFFFu << (tid & 16), f, 1));  // (half a warp has the same rows)
+            if (!(c & 1)) sm.f[c >> 1][row] = f;
         }
         cp_wait<0>();
         __syncthreads();  // the ring's memory becomes sm.u
@@ -306,14 +310,14 @@ __device__ __noinline__ int prod_chunk(const ProdWave &W, u32 chunk, u32 *ctr)
             const u64 a = wred(sm.u[0][tid] + sm.u[1][tid] + sm.u[2][tid] + sm.u[3][tid]);
             const u64 b = wred(sm.u[4][tid] + sm.u[5][tid] + sm.u[6][tid] + sm.u[7][tid]);
             sm.U[tid] = wred(a + b);
-            const u32 row = tid >> 1, g = (tid & 1) * 8;  // a row's sixteen column groups, eight a thread
-            u64 f = 0;
-            if (row < nrow) {
-                const u64 x = wred(sm.f[g][row] + sm.f[g + 1][row] + sm.f[g + 2][row] + sm.f[g + 3][row]);
-                f = wred(x + wred(sm.f[g + 4][row] + sm.f[g + 5][row] + sm.f[g + 6][row] + sm.f[g + 7][row]));
+            const u32 g = (tid & 1) * 4;  // a row's eight sums, four a thread
+#pragma unroll 1
+            for (u32 row = tid >> 1; row < ((nrow + 63) & ~63u); row += WV_NT / 2) {
+                u64 f = 0;
+                if (row < nrow) f = wred(sm.f[g][row] + sm.f[g + 1][row] + sm.f[g + 2][row] + sm.f[g + 3][row]);
+                f = wred(f + __shfl_xor_sync(0xffffffffu, f, 1));
+                if ((tid & 1) == 0 && row < nrow) sm.F[row] = f;
             }
-            f = wred(f + __shfl_xor_sync(0xffffffffu, f, 1));
-            if ((tid & 1) == 0 && row < nrow) sm.F[row] = f;
         }
         __syncthreads();
     }
@@ -593,80 +597,46 @@ __device__ __forceinline__ void gen_regs_runs(const Globals &G, const GenWave &W
     bv = tb;
 }
 
-// Sum over the lanes l = 0 mod 2^(kk+1) of a warp (the only lanes holding a
-// contribution in cross round kk; the others hold 0), written by lane 0 to
-// out[0..2].
-__device__ __forceinline__ void gen_round_sum(u64 c0, u64 c1, u64 c2, u32 kk, u64 *out)
+// Rounds off.. of a general chunk across threads: the threads' triples meet
+// in shared memory, round 0's pairs are taken by two warps, the later rounds
+// by one, each pair's terms kept in sm.c and summed once at the end (the four
+// warps working every round, and summing it, were a third of a chunk's
+// instructions).  The folded triple of the chunk goes to sm.lvl.
+__device__ __forceinline__ void gen_cross(bool hasB, u64 p, u64 v, u64 b, u32 off, u32 tid, u32 nr, GenSmem &sm)
 {
-#pragma unroll
-    for (int o = 16; o >= 1; o >>= 1) {
-        if ((u32)o < (2u << kk)) break;
-        c0 = wred(c0 + __shfl_xor_sync(0xffffffffu, c0, o));
-        c1 = wred(c1 + __shfl_xor_sync(0xffffffffu, c1, o));
-        c2 = wred(c2 + __shfl_xor_sync(0xffffffffu, c2, o));
-    }
-    if ((threadIdx.x & 31) == 0) {
-        out[0] = c0;
-        out[1] = c1;
-        out[2] = c2;
-    }
-}
-
-// Rounds off.. of a general chunk across threads (same placement as
-// prod_cross: the first thread of each pair keeps the folded values).  The
-// per-warp sums of round k go to sm.w[warp][3k..3k+2] (CTA-level rounds: warp
-// 0's row, zeros in the other rows).
-__device__ __forceinline__ void gen_cross(bool hasB, u64 &p, u64 &v, u64 &b, u32 off, u32 tid, u32 na, u32 nr, GenSmem &sm)
-{
-    const u32 lane = tid & 31, warp = tid >> 5;
-    // rolled: one copy of the round body keeps the kernel small
-#pragma unroll 1
-    for (int kk = 0; kk < 5; kk++) {
-        const u32 k = off + kk;
-        if (k < nr) {
-            const u32 d = 1u << kk;
-            const u64 p1 = __shfl_down_sync(0xffffffffu, p, d);
-            const u64 v1 = __shfl_down_sync(0xffffffffu, v, d);
-            const u64 b1 = hasB ? __shfl_down_sync(0xffffffffu, b, d) : 0;
-            u64 c0 = 0, c1 = 0, c2 = 0;
-            if ((tid & ((2u << kk) - 1)) == 0 && tid < na)
-                gen_pair(hasB, p, p1, v, v1, b, b1, sm.r[k], c0, c1, c2, p, v, b);
-            gen_round_sum(c0, c1, c2, kk, &sm.w[warp][3 * k]);
-        }
-    }
-    if (lane == 0) {
-        sm.lvl[0][warp] = p;
-        sm.lvl[1][warp] = v;
-        sm.lvl[2][warp] = b;
-        for (u32 k = off + 5; k < nr && k < off + 7; k++)
-            if (warp) sm.w[warp][3 * k] = sm.w[warp][3 * k + 1] = sm.w[warp][3 * k + 2] = 0;
-    }
+    const u32 ncross = nr - off;
+    sm.x[0][tid] = p;
+    sm.x[1][tid] = v;
+    if (hasB) sm.x[2][tid] = b;
     __syncthreads();
-    if (off + 5 < nr && warp == 0) {
-        const bool have = lane < WV_NT / 32;
-        p = have ? sm.lvl[0][lane] : 0;
-        v = have ? sm.lvl[1][lane] : 0;
-        b = have ? sm.lvl[2][lane] : 0;
-#pragma unroll
-        for (int kk = 5; kk < 7; kk++) {
-            const u32 k = off + kk;
-            if (k < nr) {
-                const u32 d = 1u << (kk - 5);
-                const u64 p1 = __shfl_down_sync(0xffffffffu, p, d);
-                const u64 v1 = __shfl_down_sync(0xffffffffu, v, d);
-                const u64 b1 = hasB ? __shfl_down_sync(0xffffffffu, b, d) : 0;
-                const u32 t = lane << 5;
-                u64 c0 = 0, c1 = 0, c2 = 0;
-                if ((t & ((2u << kk) - 1)) == 0 && t < na)
-                    gen_pair(hasB, p, p1, v, v1, b, b1, sm.r[k], c0, c1, c2, p, v, b);
-                gen_round_sum(c0, c1, c2, kk - 5, &sm.w[0][3 * k]);
-            }
+    u32 base = 0;  // round kk's terms start here
+#pragma unroll 1
+    for (u32 kk = 0; kk < ncross; kk++) {
+        const u32 np = 1u << (ncross - 1 - kk);  // pairs
+        if (tid < np) {
+            u64 c0, c1, c2;
+            b = 0;
+            gen_pair(hasB, sm.x[0][2 * tid], sm.x[0][2 * tid + 1], sm.x[1][2 * tid], sm.x[1][2 * tid + 1],
+                     hasB ? sm.x[2][2 * tid] : 0, hasB ? sm.x[2][2 * tid + 1] : 0, sm.r[off + kk], c0, c1, c2, p, v, b);
+            sm.c[0][base + tid] = c0;
+            sm.c[1][base + tid] = c1;
+            sm.c[2][base + tid] = c2;
         }
-        if (lane == 0) {
-            sm.lvl[0][0] = p;
-            sm.lvl[1][0] = v;
-            sm.lvl[2][0] = b;
+        if (np > 32) __syncthreads();  // two warps read what either wrote
+        else if (tid < 32) __syncwarp();
+        if (tid < np) {
+            sm.x[0][tid] = p;
+            sm.x[1][tid] = v;
+            if (hasB) sm.x[2][tid] = b;
         }
+        if (np > 32) __syncthreads();
+        else if (tid < 32) __syncwarp();
+        base += np;
+    }
+    if (tid == 0) {
+        sm.lvl[0] = p;
+        sm.lvl[1] = v;
+        sm.lvl[2] = hasB ? b : 0;
     }
 }
 
@@ -694,7 +664,7 @@ __device__ __noinline__ int gen_chunk(const Globals &G, const GenWave &W, u32 ch
 #pragma unroll
         for (int i = 0; i < 16; i++) h16[i] = (i < 15) ? h[i] : 0;
         const u64 s = warp_sum16(h16);
-        if ((lane & 1) == 0 && (lane >> 1) < 3 * e) sm.w[warp][lane >> 1] = s;
+        if ((lane & 1) == 0) sm.w[warp][lane >> 1] = s;
     } else if (tid < na) {
         const u64 x = base + tid;
         const bool ext = W.r0 == 0;
@@ -709,17 +679,28 @@ __device__ __noinline__ int gen_chunk(const Globals &G, const GenWave &W, u32 ch
         }
     }
     const int next = claim_task(ctr);
-    gen_cross(hasB || W.src == GS_FIRST2, pv, vv, bv, e, tid, na, nr, sm);
+    gen_cross(hasB || W.src == GS_FIRST2, pv, vv, bv, e, tid, nr, sm);
     __syncthreads();
-    if (tid < 3 * nr) {
-        const u64 sum = wred(sm.w[0][tid] + sm.w[1][tid] + sm.w[2][tid] + sm.w[3][tid]);
-        const u32 k = tid / 3, t = tid % 3;
-        W.part[((u64)k * W.nchunks + chunk) * 3 + t] = sum;
+    // four threads a value: in-register rounds from the warps' sums, cross
+    // rounds from their pairs' terms
+    for (u32 o = tid >> 2; o < 3 * nr; o += WV_NT / 4) {
+        const u32 k = o / 3, t = o - 3 * k, q = tid & 3;
+        u64 s = 0;
+        if (k < e) {
+            s = sm.w[q][o];
+        } else {
+            const u32 np = 1u << (nr - 1 - k), first = (1u << (nr - e)) - 2 * np;
+            for (u32 i = q; i < np; i += 4) s = wred(s + sm.c[t][first + i]);
+        }
+        const u32 m = 0xFu << (threadIdx.x & 28);
+        s = wred(s + __shfl_xor_sync(m, s, 1));
+        s = wred(s + __shfl_xor_sync(m, s, 2));
+        if (q == 0) W.part[((u64)k * W.nchunks + chunk) * 3 + t] = s;
     }
     if (!(W.flags & WF_LAST) && tid == 0) {
-        W.outP[chunk] = sm.lvl[0][0];
-        W.outV[chunk] = sm.lvl[1][0];
-        if (W.outB) W.outB[chunk] = sm.lvl[2][0];
+        W.outP[chunk] = sm.lvl[0];
+        W.outV[chunk] = sm.lvl[1];
+        if (W.outB) W.outB[chunk] = sm.lvl[2];
     }
     return next;
 }
@@ -728,9 +709,12 @@ __device__ __noinline__ int gen_chunk(const Globals &G, const GenWave &W, u32 ch
 // q(t) = V~_{i+1}(l(t)), folding V_{i+1} with coordinates a_k + b_k t in
 // coefficient form (degree grows by one per folded coordinate):
 //   out_c = A_c + a (B_c - A_c) + b (B_{c-1} - A_{c-1}),  c = 0 .. deg + 1.
-// A first-wave chunk folds LN_E coordinates per thread in registers (2^LN_E
-// consecutive entries) and the rest in shared memory; a later wave folds up
-// to 7 coordinates of one polynomial per thread.
+// A first-wave chunk folds e coordinates per thread in registers; the next kk
+// are folded in one step, since the result is the sum over the threads of
+// their polynomials times weight polynomials that the coins alone fix
+// (k_coins): 8 (e + 1) multiply-adds a thread and one sum over the CTA.
+// Folding those coordinates level by level through shared memory was half of
+// a chunk's time (10 us of 20) and most of a small circuit's.
 
 // One level of coefficient folding in registers: D+1 -> D+2 coefficients.
 template <int D>
@@ -762,165 +746,152 @@ __device__ __forceinline__ void line_run8(const u64 *v, const u64 *la, const u64
     line_fold<2>(l2[0], l2[1], la[2], lb[2], out);
 }
 
-// Coefficient `c` of the fold of polynomials A, B (degree deg, W values).
-__device__ __forceinline__ u64 line_coef(const u64 *A, const u64 *B, u32 deg, u32 c, u64 la, u64 lb)
+// e coordinates (3..8) of a thread's 2^e consecutive entries: runs of 8
+// (cubics over coordinates 0..2), combined like a binary counter over
+// coordinates 3, 4, .. (a rolled loop keeps one copy of the run code; from
+// coordinate 6 on the pending polynomials wait in sm.part); the polynomial to
+// sm.part[0..e][tid].
+__device__ __forceinline__ void line_regs(const u64 *entries, u32 e, LineSmem &sm)
 {
-    const u64 dc = (c <= deg) ? B[c] + (2 * FP_P) - A[c] : 0;
-    const u64 dm = (c >= 1) ? B[c - 1] + (2 * FP_P) - A[c - 1] : 0;
-    const u64 ac = (c <= deg) ? A[c] : 0;
-    return wlin2(ac, dc, dm, la, lb);
+    const ulonglong2 *src = reinterpret_cast<const ulonglong2 *>(entries);
+    const u32 tid = threadIdx.x, nruns = 1u << (e - 3);
+    u64 la[3], lb[3];
+#pragma unroll
+    for (int k = 0; k < 3; k++) {
+        la[k] = sm.a[k];
+        lb[k] = sm.b[k];
+    }
+    u64 c0[4] = {0, 0, 0, 0}, q0[5] = {0, 0, 0, 0, 0}, s0[6] = {0, 0, 0, 0, 0, 0};
+    u64 *const dst = &sm.part[0][tid];
+    auto store = [](u64 *to, const auto &v) {
+#pragma unroll
+        for (u32 i = 0; i < sizeof(v) / sizeof(u64); i++) to[i * (WV_NT + 4)] = v[i];
+    };
+#pragma unroll 1
+    for (u32 run = 0; run < nruns; run++) {
+        if (!(run & 1) && run + 2 < nruns) prefetch_l1(src + 4 * (run + 2));  // the next line
+        u64 v[8];
+#pragma unroll
+        for (int t = 0; t < 4; t++) {
+            const ulonglong2 w = __ldg(src + 4 * run + t);
+            v[2 * t] = w.x;
+            v[2 * t + 1] = w.y;
+        }
+        u64 c[4];
+        line_run8(v, la, lb, c);
+        if (nruns == 1) store(dst, c);
+        if (!(run & 1)) {
+#pragma unroll
+            for (int i = 0; i < 4; i++) c0[i] = c[i];
+            continue;
+        }
+        u64 q[5];
+        line_fold<3>(c0, c, sm.a[3], sm.b[3], q);
+        if (nruns == 2) store(dst, q);
+        if (!(run & 2)) {
+#pragma unroll
+            for (int i = 0; i < 5; i++) q0[i] = q[i];
+            continue;
+        }
+        u64 t5[6];
+        line_fold<4>(q0, q, sm.a[4], sm.b[4], t5);
+        if (nruns == 4) store(dst, t5);
+        if (!(run & 4)) {
+#pragma unroll
+            for (int i = 0; i < 6; i++) s0[i] = t5[i];
+            continue;
+        }
+        u64 p[7];
+        line_fold<5>(s0, t5, sm.a[5], sm.b[5], p);
+        if (nruns == 8) store(dst, p);
+        if (!(run & 8)) {
+            store(dst, p);
+            continue;
+        }
+        u64 p0[7], p6[8];
+#pragma unroll
+        for (int i = 0; i < 7; i++) p0[i] = sm.part[i][tid];
+        line_fold<6>(p0, p, sm.a[6], sm.b[6], p6);
+        if (nruns == 16) store(dst, p6);
+        if (!(run & 16)) {
+            store(&sm.part[8][tid], p6);
+            continue;
+        }
+        u64 r0[8], p7[9];
+#pragma unroll
+        for (int i = 0; i < 8; i++) r0[i] = sm.part[8 + i][tid];
+        line_fold<7>(r0, p6, sm.a[7], sm.b[7], p7);
+        store(dst, p7);
+    }
 }
 
 // One chunk of one line wave, by the whole CTA.
 __device__ __noinline__ int line_chunk(const Globals &G, const LineWaveDev &W, u32 chunk, u32 *ctr)
 {
     LineSmem &sm = reinterpret_cast<WaveSmem *>(wv_dyn)->line;
-    const u32 tid = threadIdx.x;
-    if (tid < W.nl) {
-        const u64 a = G.chal[W.a_off + W.l0 + tid];
-        const u64 b = f_sub(G.chal[W.b_off + W.l0 + tid], a);
-        sm.la[tid] = a;
-        sm.lb[tid] = b;
+    const u32 tid = threadIdx.x, e = W.e, kk = W.kk, l0 = W.l0;
+    const u32 deg0 = l0 + e, C = deg0 + kk + 1;  // a thread's degree; the result's coefficients
+    if (tid < e) {
+        const u64 a = G.chal[W.a_off + l0 + tid];
+        sm.a[tid] = a;
+        sm.b[tid] = f_sub(G.chal[W.b_off + l0 + tid], a);
     }
+    const bool on = tid < (1u << kk);
+    const u64 npoly = (u64)W.nchunks << W.nl;
+    const u64 y = ((u64)chunk << kk) + tid;  // the thread's polynomial in the wave's input
     __syncthreads();
-    u32 m, deg, k0;  // polynomials in bufA, their degree, coordinates already folded
-    if (W.l0 == 0) {
-        const u32 e = (W.nl >= LN_E) ? LN_E : 0;
-        const u32 na = 1u << (W.nl - e);
-        const u64 base = (u64)chunk << W.nl;
-        if (tid < na) {
-            if (e == LN_E) {
-                const ulonglong2 *src = reinterpret_cast<const ulonglong2 *>(W.in + base + ((u64)tid << LN_E));
-                u64 la[6], lb[6];
+    if (e && on) line_regs(W.in + (y << e), e, sm);
+    u64 w[8];
 #pragma unroll
-                for (int k = 0; k < 6; k++) {
-                    la[k] = sm.la[k];
-                    lb[k] = sm.lb[k];
-                }
-                // eight runs of 8 entries (cubics over coordinates 0..2), combined
-                // like a binary counter over coordinates 3, 4, 5; a rolled loop
-                // keeps one copy of the run code
-                u64 c0[4] = {0, 0, 0, 0}, q0[5] = {0, 0, 0, 0, 0};
-                u64 s0[6] = {0, 0, 0, 0, 0, 0}, s1[6] = {0, 0, 0, 0, 0, 0};
+    for (u32 b = 0; b < 8; b++) w[b] = (on && b <= kk) ? __ldg(W.wt + (b << kk) + tid) : 0;
+    // coefficient c of the product is complete once p_c is in: eight
+    // accumulators in turn
+    acc128 a[8];
+#pragma unroll
+    for (int i = 0; i < 8; i++) acc_zero(a[i]);
 #pragma unroll 1
-                for (int run = 0; run < 8; run++) {
-                    if (!(run & 1) && run < 6) prefetch_l1(src + 4 * (run + 2));  // the next line
-                    u64 v[8];
+    for (u32 c0 = 0; c0 < C; c0 += 8) {
 #pragma unroll
-                    for (int t = 0; t < 4; t++) {
-                        const ulonglong2 w = __ldg(src + 4 * run + t);
-                        v[2 * t] = w.x;
-                        v[2 * t + 1] = w.y;
-                    }
-                    u64 c[4];
-                    line_run8(v, la, lb, c);
-                    if (!(run & 1)) {
+        for (u32 i = 0; i < 8; i++) {
+            const u32 c = c0 + i;
+            if (c < C) {
+                if (c <= deg0 && on) {
+                    const u64 p = e ? sm.part[c][tid] : l0 ? __ldcg(W.in + c * npoly + y) : __ldg(W.in + y);
 #pragma unroll
-                        for (int i = 0; i < 4; i++) c0[i] = c[i];
-                        continue;
-                    }
-                    u64 q[5];
-                    line_fold<3>(c0, c, la[3], lb[3], q);
-                    if (!(run & 2)) {
-#pragma unroll
-                        for (int i = 0; i < 5; i++) q0[i] = q[i];
-                        continue;
-                    }
-                    u64 t5[6];
-                    line_fold<4>(q0, q, la[4], lb[4], t5);
-#pragma unroll
-                    for (int i = 0; i < 6; i++) {
-                        if (run & 4) s1[i] = t5[i];
-                        else s0[i] = t5[i];
-                    }
+                    for (u32 b = 0; b < 8; b++) mac(a[(i + b) & 7], p, w[b]);
                 }
-                u64 p[7];
-                line_fold<5>(s0, s1, la[5], lb[5], p);
-#pragma unroll
-                for (int c = 0; c < 7; c++) sm.bufA[tid * 7 + c] = p[c];
-            } else {
-                sm.bufA[tid] = __ldg(W.in + base + tid);
+                sm.part[c][tid] = acc_red(a[i]);
+                acc_zero(a[i]);
             }
         }
-        m = na;
-        deg = e;
-        k0 = e;
-    } else {
-        // polynomials of degree l0 from the previous wave (written by other
-        // CTAs of this launch when run as a tail: read through L2)
-        const u32 din = W.l0, npoly = 1u << W.nl, half = npoly >> 1, C = din + 2;
-        const u64 *in = W.in + ((u64)chunk << W.nl) * (din + 1);
-        for (u32 idx = tid; idx < half * C; idx += WV_NT) {
-            const u32 j = idx / C, c = idx - j * C;
-            const u64 *A = in + (u64)(2 * j) * (din + 1), *B = A + (din + 1);
-            const u64 dc = (c <= din) ? __ldcg(B + c) + (2 * FP_P) - __ldcg(A + c) : 0;
-            const u64 dm = (c >= 1) ? __ldcg(B + c - 1) + (2 * FP_P) - __ldcg(A + c - 1) : 0;
-            const u64 ac = (c <= din) ? __ldcg(A + c) : 0;
-            sm.bufA[j * C + c] = wlin2(ac, dc, dm, sm.la[0], sm.lb[0]);
+    }
+    const int next = claim_task(ctr);
+    __syncthreads();
+    {
+        const u32 c = tid >> 2, q = tid & 3;
+        u64 s = 0;
+        if (c < C) {
+#pragma unroll 1
+            for (u32 i = q; i < (1u << kk); i += 8)
+                s = wred(s + sm.part[c][i] + (i + 4 < (1u << kk) ? sm.part[c][i + 4] : 0));
         }
-        m = half;
-        deg = din + 1;
-        k0 = 1;
+        s = wred(s + __shfl_xor_sync(0xffffffffu, s, 1));
+        s = wred(s + __shfl_xor_sync(0xffffffffu, s, 2));
+        if (q == 0 && c < C) sm.res[c] = s;
     }
     __syncthreads();
-    const int next = claim_task(ctr);
-    u64 *cur = sm.bufA, *nxt = sm.bufB;
-    u32 k = k0;
-    if (m == WV_NT && deg == LN_E && k + 5 <= W.nl) {
-        // One polynomial per thread: the first five levels stay inside each
-        // warp (its 32 polynomials -> 1) with no CTA barrier.  A warp works
-        // in its own parts of the buffers: its level-0 inputs in bufA, then
-        // alternately 256 entries of bufB and its bufA part; its result goes
-        // past every warp's inputs, to bufA[1024 + warp (LN_E + 6)].
-        const u32 warp = tid >> 5, lane = tid & 31;
-        u64 *ownA = sm.bufA + warp * 32 * (LN_E + 1), *ownB = sm.bufB + warp * 256;
-        const u64 *in = ownA;
-        u32 cnt = 32, d = deg;
-        for (u32 lv = 0; lv < 5; lv++, k++) {
-            u64 *out = (lv == 4) ? sm.bufA + 1024 + warp * (LN_E + 6) : ((lv & 1) ? ownA : ownB);
-            const u32 half = cnt >> 1, C = d + 2;
-            for (u32 idx = lane; idx < half * C; idx += 32) {
-                const u32 j = idx / C, c = idx - j * C;
-                out[j * C + c] = line_coef(in + (2 * j) * (d + 1), in + (2 * j + 1) * (d + 1), d, c, sm.la[k], sm.lb[k]);
-            }
-            __syncwarp();
-            in = out;
-            cnt = half;
-            d += 1;
-        }
-        __syncthreads();
-        cur = sm.bufA + 1024;
-        m = WV_NT / 32;
-        deg = d;
-    }
-    for (; k < W.nl; k++) {
-        const u32 half = m >> 1, C = deg + 2;
-        for (u32 idx = tid; idx < half * C; idx += WV_NT) {
-            const u32 j = idx / C, c = idx - j * C;
-            nxt[j * C + c] =
-                line_coef(cur + (2 * j) * (deg + 1), cur + (2 * j + 1) * (deg + 1), deg, c, sm.la[k], sm.lb[k]);
-        }
-        __syncthreads();
-        u64 *t = cur;
-        cur = nxt;
-        nxt = t;
-        m = half;
-        deg += 1;
-    }
-    // cur[0..deg] is this chunk's polynomial
+    const u64 *q = sm.res;  // q[0..deg] is this chunk's polynomial
+    const u32 deg = C - 1;
     if (!W.last) {
-        u64 *out = W.out + (u64)chunk * (deg + 1);
-        for (u32 c = tid; c <= deg; c += WV_NT) out[c] = cur[c];
+        if (tid <= deg) W.out[(u64)tid * W.nchunks + chunk] = q[tid];
     } else {
         // q(t) for t = 0..n by Horner; q(0) = V~_{i+1}(r1) feeds phase 3
-        const u32 n = W.n;
-        u64 *tr = G.tr + W.tr_q;
-        for (u32 t = tid; t <= n; t += WV_NT) {
-            u64 acc = cur[deg];
-            for (int c = (int)deg - 1; c >= 0; c--) acc = wred(wmul(acc, (u64)t) + cur[c]);
-            tr[t] = wcanon(acc);
+        if (tid <= W.n) {
+            u64 acc = q[deg];
+            for (int c = (int)deg - 1; c >= 0; c--) acc = wred(wmul(acc, (u64)tid) + q[c]);
+            G.tr[W.tr_q + tid] = wcanon(acc);
         }
-        if (tid == 0) G.scal[SCAL_V1(W.layer)] = wcanon(cur[0]);
+        if (tid == 0) G.scal[SCAL_V1(W.layer)] = wcanon(q[0]);
     }
     return next;
 }

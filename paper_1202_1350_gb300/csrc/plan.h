@@ -133,7 +133,7 @@ enum : u32 { GS_NONE = 0, GS_SQ2 = 1, GS_PAIR2 = 2, GS_FINAL2 = 3, GS_FIRST2 = 4
 // PROD: a chunk of more than 2^PR_C entries is a matrix of 2^kr rows of 2^PR_C
 // columns, kr <= PR_R (128 threads per CTA)
 #define PR_C 7
-#define PR_R 6
+#define PR_R 7
 // Words of the message-weight table of kk coordinates (see ProdWave::wblk).
 __host__ __device__ __forceinline__ u32 vec_slots(u32 kk) { return kk > 5 ? 1u << (kk - 5) : 1u; }
 __host__ __device__ __forceinline__ u32 vec_words(u32 kk) { return vec_slots(kk) * kk * 16; }
@@ -206,15 +206,21 @@ struct GenWave {
 // Line reduction of layer i (q(t) = V~_{i+1}(l(t)), l(t) = r1 + t (r2 - r1)),
 // computed by folding V_{i+1} with the coordinates a_k + b_k t in coefficient
 // form: after folding j coordinates each entry is a polynomial of degree j.
+// A wave folds nl = e + kk coordinates of each chunk: e in registers (2^e
+// consecutive entries a thread; 0 or 3..8), kk in one step, as the sum over
+// the 2^kk threads of their polynomials times the weight polynomials
+// prod_m (l_m or 1 - l_m) (wt: coefficient b of thread y at b 2^kk + y).
 struct LineWaveDev {
     u32 circ;
     u32 layer;
     u32 n;        // s_{i+1}
     u32 l0, nl;   // coordinates [l0, l0 + nl) folded by this wave
+    u32 e, kk;
     u32 nchunks;
     u32 last;
-    const u64 *in;  // l0 == 0: V_{i+1}; else polys [chunk][l0 + 1]
-    u64 *out;       // polys [nchunks][l0 + nl + 1] (unused on the last wave)
+    const u64 *in;  // l0 == 0: V_{i+1}; else coefficient c of poly q at c (nchunks << nl) + q
+    u64 *out;       // coefficient c of chunk's poly at c nchunks + chunk (unused on the last wave)
+    u64 *wt;        // (kk + 1) 2^kk words
     u32 a_off;      // a_k = chal[a_off + k] (= r1), b_k = chal[b_off + k] - a_k
     u32 b_off;
     u64 tr_q;
@@ -359,10 +365,10 @@ void launch_params_batch(Globals *Gs, const CallParams *cp, int n, cudaStream_t 
 void launch_gather_inputs(const CallParams *cp, const GatherChunk *chunks, int nchunks, cudaStream_t st);
 // One launch: setup of every circuit (challenges, points, eq(z_i, r_P), by
 // coin_setups(d) CTAs listed as {circuit, slice}), the eq tables and the
-// product weights of the PROD waves.
+// weights of the PROD waves and of the line waves.
 __host__ __device__ __forceinline__ u32 coin_setups(u32 d) { return (d + 7) / 8; }
 void launch_coins(const Globals *Gs, const Item *setups, int nsetup, const EqJob *eqjobs, int neq,
-                  const SciDev *scis, const ProdWave *pw, int npw, cudaStream_t st);
+                  const SciDev *scis, const ProdWave *pw, int npw, const LineWaveDev *lw, int nlw, cudaStream_t st);
 void launch_eval_layers(const Globals *Gs, const LayerEval *le, const Item *items, int nitems, cudaStream_t st);
 // maxblock: the largest block (entries) of any run layer or tail output in
 // the launch (<= 2048); it sizes the two shared-memory buffers.

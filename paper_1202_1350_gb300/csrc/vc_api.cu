@@ -585,7 +585,11 @@ static size_t layout(vc_circuit *c, uintptr_t base, uintptr_t hbase)
         const u64 *in = c->V[i + 1];
         bool tail = false;
         for (u32 w = 0;; w++) {
-            const u32 cap = (w == 0) ? c->cfg.ln_chunk0 : LN_CHUNKW_LOG;
+            // first chunks of more than 20 coordinates take up to two more, so
+            // that the next wave is their last (a third was a launch of its own)
+            u32 cap = (w == 0) ? c->cfg.ln_chunk0 : LN_CHUNKW_LOG;
+            if (w == 0 && cap == LN_CHUNK0_LOG && n > cap + LN_CHUNKW_LOG)
+                cap = std::min(LN_CHUNK0_LOG + LN_XTRA, n - LN_CHUNKW_LOG);
             const u32 nl = std::min(cap, n - l0);
             LineWaveDev W{};
             W.circ = 0;
@@ -593,6 +597,9 @@ static size_t layout(vc_circuit *c, uintptr_t base, uintptr_t hbase)
             W.n = n;
             W.l0 = l0;
             W.nl = nl;
+            W.e = (w > 0 || nl <= WV_LOG) ? 0u : std::max(3u, nl - WV_LOG);
+            W.kk = nl - W.e;
+            W.wt = A.take<u64>((W.kk + 1) << W.kk);
             W.nchunks = u32(1) << (n - l0 - nl);
             W.last = (l0 + nl == n);
             W.in = in;
@@ -732,8 +739,15 @@ static size_t layout(vc_circuit *c, uintptr_t base, uintptr_t hbase)
             // smaller PROD instances (dispatched after the larger ones) use
             // half-size chunks, which evens out the end of the launch
             const u32 split = (c->cfg.pr_split == VC_SPLIT_WIDEST) ? smax : c->cfg.pr_split;
-            const u32 C = prod ? ((n < split && c->cfg.pr_chunk > 1) ? c->cfg.pr_chunk - 1 : c->cfg.pr_chunk)
-                               : c->cfg.gn_chunk;
+            u32 C = prod ? ((n < split && c->cfg.pr_chunk > 1) ? c->cfg.pr_chunk - 1 : c->cfg.pr_chunk)
+                         : c->cfg.gn_chunk;
+            // with the default shapes wide PROD instances take larger chunks
+            // (about 7,000 cycles of a chunk do not depend on its size): 2^13
+            // from 14 coordinates, 2^14 from 19.  F2 2^22 waves 206 us with 2^12
+            // and 2^13, 194 with 2^13, 182 with these (2^14 from 17: 182, but
+            // MATMULT 128 71 against 67).
+            if (prod && c->cfg.pr_chunk == PR_CHUNK_LOG && c->cfg.pr_split == VC_SPLIT_WIDEST && n >= 14)
+                C = n >= 19 ? PR_CHUNK_WIDE : PR_CHUNK_LOG;
             const bool tab = needs_tables(L.kind) && ph != 1;  // waits for k_build23
             const bool anyB = (tab && L.has_add) || src == GS_FIRST2;
             const u64 *inV = (ph == 1) ? L.V : L.Vn;
@@ -980,7 +994,9 @@ bool plan_valid(const Plan &P)
             return false;
     }
     for (const LineWaveDev &W : P.lw)
-        if (W.nl > (W.l0 ? LN_CHUNKW_LOG : LN_CHUNK0_LOG) || W.n > 30) return false;
+        if (W.n > 30 || W.e + W.kk != W.nl || W.kk > WV_LOG || W.l0 + W.nl > W.n ||
+            (W.l0 ? W.e != 0 : W.e > 8 || (W.e && W.e < 3)))
+            return false;
     for (const RoundRef &R : P.rounds)
         if (R.sci >= P.scis.size() || R.j >= P.scis[R.sci].n || R.circ >= nc || P.scis[R.sci].circ != R.circ ||
             !R.ez || !R.v1 || !R.ch || (R.kind < PK_GEN_FIRST && (!R.lc || !R.kap || !R.esum)))
@@ -1289,7 +1305,8 @@ void enqueue_plan(Plan &P, cudaStream_t st)
     mark(VC_STAGE_EVAL, 1, st);
     cudaStreamWaitEvent(sa, P.ev_fork, 0);
     mark(VC_STAGE_TABLES, 0, sa);
-    launch_coins(Gs, P.d_setups, (int)P.setups.size(), P.d_eqjobs, (int)P.eqjobs.size(), P.d_scis, P.d_pw, (int)P.pw.size(), sa);
+    launch_coins(Gs, P.d_setups, (int)P.setups.size(), P.d_eqjobs, (int)P.eqjobs.size(), P.d_scis, P.d_pw, (int)P.pw.size(),
+                 P.d_lw, (int)P.lw.size(), sa);
     mark(VC_STAGE_TABLES, 1, sa);
     cudaEventRecord(P.ev_tables, sa);
     cudaStreamWaitEvent(st, P.ev_tables, 0);
@@ -1431,7 +1448,8 @@ static void enqueue_staged(vc_circuit &c, cudaStream_t st)
     launch_params(P.d_G, 0, nullptr, nullptr, st);  // arguments set per launch
     cudaEventRecord(P.ev_fork, st);
     cudaStreamWaitEvent(sa, P.ev_fork, 0);
-    launch_coins(Gs, P.d_setups, (int)P.setups.size(), P.d_eqjobs, (int)P.eqjobs.size(), P.d_scis, P.d_pw, (int)P.pw.size(), sa);
+    launch_coins(Gs, P.d_setups, (int)P.setups.size(), P.d_eqjobs, (int)P.eqjobs.size(), P.d_scis, P.d_pw, (int)P.pw.size(),
+                 P.d_lw, (int)P.lw.size(), sa);
     cudaEventRecord(P.ev_tables, sa);
     // evaluation; holder[s] = the wide layer in slot s (-1: none yet)
     std::vector<int> holder(c.st_nslots, -1);
@@ -1507,7 +1525,8 @@ static void enqueue_windowed(vc_circuit &c, cudaStream_t st)
     launch_params(P.d_G, 0, nullptr, nullptr, st);  // arguments set per launch
     cudaEventRecord(P.ev_fork, st);
     cudaStreamWaitEvent(sa, P.ev_fork, 0);
-    launch_coins(Gs, P.d_setups, (int)P.setups.size(), P.d_eqjobs, (int)P.eqjobs.size(), P.d_scis, P.d_pw, (int)P.pw.size(), sa);
+    launch_coins(Gs, P.d_setups, (int)P.setups.size(), P.d_eqjobs, (int)P.eqjobs.size(), P.d_scis, P.d_pw, (int)P.pw.size(),
+                 P.d_lw, (int)P.lw.size(), sa);
     cudaEventRecord(P.ev_tables, sa);
     launch_check_inputs(Gs, P.d_checks, (int)P.checks.size(), st);  // the inputs are in layer d
     bool coins = false;
@@ -2023,7 +2042,8 @@ static cudaError_t pergate_launch(vc_circuit *c, cudaStream_t st)
             launch_eval_segs(P.d_G, P.d_segs, P.d_seg_items[k], (int)P.seg_items[k].size(), P.seg_maxblock[k], P.cap);
             launch_eval_layers(P.d_G, P.d_levs, P.d_lev_items[k], (int)P.lev_items[k].size(), P.cap);
         }
-        launch_coins(P.d_G, P.d_setups, (int)P.setups.size(), nullptr, 0, nullptr, nullptr, 0, P.cap);
+        launch_coins(P.d_G, P.d_setups, (int)P.setups.size(), nullptr, 0, nullptr, nullptr, 0, nullptr, 0,
+                     P.cap);
         launch_pergate(P.d_G, c->d_pg, (int)c->d, c->d_pg_blk, c->pg_nblk, c->d_pg_lblk, c->pg_nlblk, c->pg_rounds,
                        P.cap);
         cudaGraph_t g = nullptr;
@@ -2161,7 +2181,8 @@ extern "C" vc_status vc_verify(vc_circuit *c, const uint64_t *inputs, uint64_t s
             launch_vparams(c->d_Gv, c->d_vp, 0, nullptr, nullptr, nullptr, c->d_result, cs);
             cudaEventRecord(c->P.ev_fork, cs);
             cudaStreamWaitEvent(c->P.aux, c->P.ev_fork, 0);
-            launch_coins(c->d_Gv, c->P.d_setups, (int)c->P.setups.size(), c->d_eq_verify, (int)c->eq_verify.size(), nullptr, nullptr, 0, cs);
+            launch_coins(c->d_Gv, c->P.d_setups, (int)c->P.setups.size(), c->d_eq_verify, (int)c->eq_verify.size(), nullptr, nullptr, 0,
+                         nullptr, 0, cs);
             launch_verify(c->d_Gv, c->Gv, c->Vd, c->s[c->d], c->s[0], c->d_vwire, (int)c->vwire.size(),
                           c->P.aux, c->P.ev_tables, cs);
         };
@@ -2205,7 +2226,8 @@ extern "C" vc_status vc_verify_input(vc_circuit *c, const uint64_t *inputs, uint
             cudaStreamWaitEvent(c->P.aux, c->P.ev_fork, 0);
             launch_verify_input(c->d_Gv, c->Gv, c->Vd, c->s[c->d], c->s[0], c->P.aux);
             cudaEventRecord(c->P.ev_tables, c->P.aux);
-            launch_coins(c->d_Gv, c->P.d_setups, (int)c->P.setups.size(), nullptr, 0, nullptr, nullptr, 0, cs);
+            launch_coins(c->d_Gv, c->P.d_setups, (int)c->P.setups.size(), nullptr, 0, nullptr, nullptr, 0, nullptr, 0,
+                         cs);
             cudaStreamWaitEvent(cs, c->P.ev_tables, 0);
         };
         e = capture_graph(c->P.cap, enqueue, &c->vin_exec, vparams_in_kernel(), &c->vin_graph, &c->vin_node,
@@ -2241,7 +2263,8 @@ extern "C" vc_status vc_verify_transcript(vc_circuit *c, uint64_t seed, const ui
     if (e != cudaSuccess) return VC_ECUDA;
     // plain launches with the per-call pointers as arguments (one launch for
     // structured circuits): nothing to capture, nothing to write first
-    launch_coins(c->d_Gv, nullptr, 0, c->d_eq_verify, (int)c->eq_verify.size(), nullptr, nullptr, 0, st);
+    launch_coins(c->d_Gv, nullptr, 0, c->d_eq_verify, (int)c->eq_verify.size(), nullptr, nullptr, 0, nullptr, 0,
+                 st);
     launch_verify_transcript(c->d_Gv, c->Gv, c->Vd, c->s[c->d], c->s[0], c->d_vwire, (int)c->vwire.size(), dtr,
                              ka ? accept : nullptr, st);
     return verifier_finish(c, ka && kt && !c->vin_sync, ka, accept, st);
@@ -2269,7 +2292,8 @@ static cudaError_t pv_capture(vc_circuit *c)
     enqueue_plan(c->P, cs);
     cudaStreamWaitEvent(c->pv_vs, c->pv_fork, 0);
     launch_vparams(c->d_Gv, c->d_vp, 0, nullptr, nullptr, nullptr, c->d_result, c->pv_vs);
-    launch_coins(c->d_Gv, c->P.d_setups, (int)c->P.setups.size(), c->d_eq_verify, (int)c->eq_verify.size(), nullptr, nullptr, 0, c->pv_vs);
+    launch_coins(c->d_Gv, c->P.d_setups, (int)c->P.setups.size(), c->d_eq_verify, (int)c->eq_verify.size(), nullptr, nullptr, 0,
+                 nullptr, 0, c->pv_vs);
     launch_verify_input(c->d_Gv, c->Gv, c->Vd, c->s[c->d], c->s[0], c->pv_vs);
     cudaEventRecord(c->pv_join, c->pv_vs);
     cudaStreamWaitEvent(cs, c->pv_join, 0);
