@@ -486,14 +486,17 @@ __global__ void __launch_bounds__(256) k_build23(const Globals *Gs, const BuildI
     const Globals &G = Gs[bi.circ];
     const u32 i = bi.layer;
     const LayerDev &L = G.layers[i];
-    const u64 w = (u64)bi.block * blockDim.x + threadIdx.x;
-    if (w >= (1ull << L.sn)) return;
+    // the gates of an entry are chains of dependent loads: eight threads walk
+    // them together (one alone: up to 32 chains one after another, 28 us)
+    const u32 lane = threadIdx.x % BUILD_LANES;
+    const u64 w = (u64)bi.block * BUILD_ENTRIES + threadIdx.x / BUILD_LANES;
+    const bool in = w < (1ull << L.sn);
     const u64 ez = G.scal[SCAL_EQZRP(i)];
     const u64 v1 = G.scal[SCAL_V1(i)];
     const u64 *V = L.Vn;
     u64 P2 = 0, B2 = 0, A2 = 0, M2 = 0;
-    const u32 a0 = L.by1_off[w], a1 = L.by1_off[w + 1];
-    for (u32 q = a0; q < a1 && a1 - a0 <= BUILD_HEAVY; q++) {
+    const u32 a0 = in ? L.by1_off[w] : 0, a1 = in ? L.by1_off[w + 1] : 0;
+    for (u32 q = a0 + lane; q < a1 && a1 - a0 <= BUILD_HEAVY; q += BUILD_LANES) {
         const u32 g = L.by1_g[q];
         const u64 wg = f_mul(ez, eq_at(L.trp, g));
         if (L.type[g]) {
@@ -503,13 +506,21 @@ __global__ void __launch_bounds__(256) k_build23(const Globals *Gs, const BuildI
             B2 = f_add(B2, f_mul(wg, V[L.in2[g]]));
         }
     }
-    const u32 b0 = L.by2_off[w], b1 = L.by2_off[w + 1];
-    for (u32 q = b0; q < b1 && b1 - b0 <= BUILD_HEAVY; q++) {
+    const u32 b0 = in ? L.by2_off[w] : 0, b1 = in ? L.by2_off[w + 1] : 0;
+    for (u32 q = b0 + lane; q < b1 && b1 - b0 <= BUILD_HEAVY; q += BUILD_LANES) {
         const u32 g = L.by2_g[q];
         const u64 ug = f_mul(f_mul(ez, eq_at(L.trp, g)), eq_at(L.tr1, L.in1[g]));
         if (L.type[g]) M2 = f_add(M2, ug);
         else A2 = f_add(A2, ug);
     }
+#pragma unroll
+    for (u32 o = BUILD_LANES / 2; o > 0; o >>= 1) {
+        P2 = f_add(P2, __shfl_xor_sync(0xffffffffu, P2, o));
+        B2 = f_add(B2, __shfl_xor_sync(0xffffffffu, B2, o));
+        A2 = f_add(A2, __shfl_xor_sync(0xffffffffu, A2, o));
+        M2 = f_add(M2, __shfl_xor_sync(0xffffffffu, M2, o));
+    }
+    if (!in || lane) return;
     L.P2[w] = P2;
     L.P3[w] = f_add(A2, f_mul(v1, M2));
     if (L.has_add) {

@@ -1090,6 +1090,20 @@ __global__ void __launch_bounds__(256) k_final(Globals *Gs, const RoundRef *roun
 {
     const u32 lane = threadIdx.x & 31;
     const u64 gt = blockIdx.x * (u64)blockDim.x + threadIdx.x, nthreads = (u64)gridDim.x * blockDim.x;
+    // the outputs open each transcript (the evaluation wrote them before the
+    // wave launch began): gridDim / nouts CTAs a circuit (one CTA copying
+    // MATMULT's 2^14 outputs took 14 us); the proof's in-place input pointer is
+    // cleared (later evaluations read the input layer)
+    const u32 slices = gridDim.x > (u32)nouts ? gridDim.x / nouts : 1u;
+    for (u32 k = blockIdx.x; k < (u32)nouts * slices; k += gridDim.x) {
+        Globals &G = Gs[outs[k % nouts]];
+        const u32 sl = k / nouts;
+        if (sl == 0 && threadIdx.x == 0) G.in = nullptr;
+        const u64 n = G.S0;
+        const u64 *__restrict__ src = G.out_src;
+        u64 *__restrict__ dst = G.tr;
+        for (u64 x = (u64)sl * blockDim.x + threadIdx.x; x < n; x += (u64)slices * blockDim.x) dst[x] = src[x];
+    }
     // launched early (programmatic dependence on the wave launch): the first
     // round's descriptor and coin-launch scalars are loaded before waiting
     // for the waves; v1 and the partials only after
@@ -1131,17 +1145,6 @@ __global__ void __launch_bounds__(256) k_final(Globals *Gs, const RoundRef *roun
             for (u32 v = 0; v < 2; v++) h2[v] = wred(h2[v] + R.part2_pos[(u64)q * 2 + v]);
         for (u32 v = 0; v < 2; v++) h2[v] = wcanon(h2[v]);
         final_round(Gs, R, S, h, h2);
-    }
-    // the outputs open each transcript: a CTA per circuit (grid-stride over
-    // the circuits), its threads over the outputs; the proof's in-place input
-    // pointer is cleared (later evaluations read the input layer)
-    for (int j = blockIdx.x; j < nouts; j += gridDim.x) {
-        Globals &G = Gs[outs[j]];
-        if (threadIdx.x == 0) G.in = nullptr;
-        const u64 n = G.S0;
-        const u64 *__restrict__ src = G.out_src;
-        u64 *__restrict__ dst = G.tr;
-        for (u64 x = threadIdx.x; x < n; x += blockDim.x) dst[x] = src[x];
     }
 }
 

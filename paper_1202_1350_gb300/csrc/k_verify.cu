@@ -319,7 +319,11 @@ __device__ void wiring_warp(u32 kind, u32 si, u32 sn, const u64 *p, const u64 *w
     }
 }
 
+// Threads of a check CTA: 64 warps over the cluster for up to 31 layers, whose
+// 2 d + 1 warp items they take one each, else 128 (with two or three items one
+// after the other the launch took 15 us at 68 layers).
 #define VC_NT 256
+#define VC_NT_DEEP 512
 #define VC_CL 8  // CTAs of the check launch: one thread-block cluster
 
 // All checks of the verifier in one cluster of VC_CL CTAs; the accept bit is
@@ -338,13 +342,14 @@ __device__ void wiring_warp(u32 kind, u32 si, u32 sn, const u64 *p, const u64 *w
 // form.  The
 // accept bit is the conjunction of exactly the sequential verifier's checks.
 // tr_arg: the transcript and accept pointer given directly (NULL: from V.vp).
-__global__ void __cluster_dims__(VC_CL, 1, 1) __launch_bounds__(VC_NT)
+template <int NT>
+__global__ void __cluster_dims__(VC_CL, 1, 1) __launch_bounds__(NT)
     k_vcheck(Globals G, VerifyDev V, const u64 *tr_arg, int *accept_arg)
 {
     namespace cg = cooperative_groups;
     const u64 *const tr = tr_arg ? tr_arg : V.vp->tr;
     const u32 lane = threadIdx.x & 31;
-    const u32 g = blockIdx.x * VC_NT + threadIdx.x, nthreads = VC_CL * VC_NT;
+    const u32 g = blockIdx.x * NT + threadIdx.x, nthreads = VC_CL * NT;
     u32 fail = 0;
     // warp items: [0, d) a layer's starting claim and its round 0 (with the
     // end of the layer when it has no rounds, whose claim is the start);
@@ -490,6 +495,14 @@ const void *vparams_in_kernel() { return reinterpret_cast<const void *>(k_vparam
 // Entries per CTA (log2) of the MLE partial sums for a point of n coordinates.
 u32 vmle_log(u32 n) { return n < 11 ? n : 11; }
 
+static void launch_vcheck(const Globals &G, const VerifyDev &V, const u64 *tr, int *accept, cudaStream_t st)
+{
+    if (2 * V.d + 1 <= VC_CL * VC_NT / 32)
+        k_vcheck<VC_NT><<<VC_CL, VC_NT, 0, st>>>(G, V, tr, accept);
+    else
+        k_vcheck<VC_NT_DEEP><<<VC_CL, VC_NT_DEEP, 0, st>>>(G, V, tr, accept);
+}
+
 void launch_verify(const Globals *Gd, const Globals &G, const VerifyDev &V, u32 nd, u32 n0, const VwireItem *wire_items,
                    int n_wire, cudaStream_t st_mle, cudaEvent_t ev_join, cudaStream_t st)
 {
@@ -501,7 +514,7 @@ void launch_verify(const Globals *Gd, const Globals &G, const VerifyDev &V, u32 
     cudaEventRecord(ev_join, st_mle);
     cudaStreamWaitEvent(st, ev_join, 0);
     if (n_wire > 0) k_vwire<<<n_wire, VM_NT, 0, st>>>(G, wire_items, V);
-    k_vcheck<<<VC_CL, VC_NT, 0, st>>>(G, V, nullptr, nullptr);
+    launch_vcheck(G, V, nullptr, nullptr, st);
 }
 
 void launch_verify_input(const Globals *Gd, const Globals &G, const VerifyDev &V, u32 nd, u32 n0, cudaStream_t st)
@@ -518,5 +531,5 @@ void launch_verify_transcript(const Globals *Gd, const Globals &G, const VerifyD
         k_vmle<<<V.mle_out_blocks, VM_NT, 0, st>>>(Gd, V.vp, nd, vmle_log(nd), n0, vmle_log(n0), V.mle_blocks,
                                                    V.mle_blocks, tr, V.mle_part, G.status, V.result);
     if (n_wire > 0) k_vwire<<<n_wire, VM_NT, 0, st>>>(G, wire_items, V);
-    k_vcheck<<<VC_CL, VC_NT, 0, st>>>(G, V, tr, accept);
+    launch_vcheck(G, V, tr, accept, st);
 }

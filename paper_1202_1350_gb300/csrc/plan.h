@@ -318,7 +318,7 @@ struct LayerEval {
     u32 layer;
 };
 
-// Work item of k_build23: 256 entries of layer i+1's phase-2/3 tables.
+// Work item of k_build23: BUILD_ENTRIES entries of layer i+1's phase-2/3 tables.
 struct BuildItem {
     u32 circ;
     u32 layer;
@@ -387,7 +387,9 @@ void launch_mm_tables(const Globals *Gs, const BuildItem *items, int nitems, cud
 // its sums to part[2 piece ..], and the last to finish (ctr) adds them all to
 // the entry's tables.
 #define BUILD_HEAVY 32u
-#define BUILD_PIECE 4096u
+#define BUILD_PIECE 512u
+#define BUILD_LANES 8u    // k_build23: threads per entry
+#define BUILD_ENTRIES (256u / BUILD_LANES)
 struct HeavyItem {
     u32 circ, layer, w, kind;
     u32 piece, npieces, pad0, pad1;

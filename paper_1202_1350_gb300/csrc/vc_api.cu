@@ -209,6 +209,10 @@ static void plan_eval(vc_circuit *c)
                 const int ne = e + (int)c->s[j] - (int)c->s[j + 1];
                 if (ne < 0 || ne > 11) break;
                 if (c->kind[j] == W_F0_PAIR && ne < 1) break;
+                // a power chain is a serial 59 layers a CTA: blocks that have
+                // shrunk below half a chain's chunk start a run of their own
+                // (pattern matching 2^14: 1024 CTAs of 16 pairs took 64 us)
+                if (c->kind[j] == W_F0_FIRST && j < i && e < EV_PAIR_CHUNK - 1 && s_in > cl_) break;
                 pairs |= c->kind[j] == W_F0_PAIR;
                 e = ne;
                 i_lo = j;
@@ -240,10 +244,11 @@ static void plan_eval(vc_circuit *c)
         S.nchunks = 1u << (s_in - cl);
         S.check_input = (u32)(i + 1 == (int)c->d);
         // tail: narrow local layers below the run (outputs <= 2^11, first
-        // input <= 2^16) go to the CTA that finishes last
+        // input <= 2^16) go to the CTA that finishes last, up to a power chain
+        // (which one CTA would take layer by layer, 1.5 us each)
         S.tail_lo = S.i_lo;
         if (S.nchunks > 1 && c->s[i_lo] <= 16)
-            for (int j = i_lo - 1; j >= 0 && local(j) && !flush[j] && c->s[j] <= 11; j--) {
+            for (int j = i_lo - 1; j >= 0 && local(j) && !flush[j] && c->s[j] <= 11 && c->kind[j] != W_F0_FIRST; j--) {
                 S.tail_lo = (u32)j;
                 maxblock = std::max(maxblock, 1u << c->s[j]);
             }
@@ -621,7 +626,7 @@ static size_t layout(vc_circuit *c, uintptr_t base, uintptr_t hbase)
         }
     }
 
-    // phase-2/3 table builds of explicit layers: one thread per entry of layer
+    // phase-2/3 table builds of explicit layers: eight threads per entry of layer
     // i+1, and a CTA per entry that more than BUILD_HEAVY gates read; and the
     // phase-2 factors of MATMULT layers, a warp per row
     P.builds.clear();
@@ -631,7 +636,7 @@ static size_t layout(vc_circuit *c, uintptr_t base, uintptr_t hbase)
         if (c->kind[i] == W_MATMULT)
             for (u32 b = 0; b < ((1u << (c->s[i] / 3)) + MM_ROWS - 1) / MM_ROWS; b++) P.mms.push_back({0u, i, b, 0u});
         if (!needs_tables(c->kind[i])) continue;
-        const u64 blocks = (S(i + 1) + 255) / 256;
+        const u64 blocks = (S(i + 1) + BUILD_ENTRIES - 1) / BUILD_ENTRIES;
         for (u64 b = 0; b < blocks; b++) P.builds.push_back({0u, i, (u32)b, 0u});
         for (u64 w = 0; w < S(i + 1); w++)
             for (u32 kind = 1; kind <= 2; kind++) {
@@ -863,11 +868,12 @@ static size_t layout(vc_circuit *c, uintptr_t base, uintptr_t hbase)
     c->Vd.mle_out_blocks = S(0) <= VC_OUT_INLINE ? 0u : (u32)mbo;  // few outputs: formed in the check launch
     c->Vd.mle_part = A.take<u64>(mb + mbo);
     c->Vd.wire = A.take<u64>(2 * d + 2);
-    // the verifier's wiring sums: about 4096 gates per CTA, at most 1024 CTAs a layer
+    // the verifier's wiring sums: about 512 gates per CTA (two a thread: each is
+    // a chain of dependent loads), at most 1024 CTAs a layer
     c->vwire.clear();
     u32 nparts = 0;
     for (u32 i : c->explicit_layers) {
-        const u32 nb = (u32)std::min<u64>(1024, std::max<u64>(1, S(i) / 4096));
+        const u32 nb = (u32)std::min<u64>(1024, std::max<u64>(1, S(i) / 512));
         for (u32 b = 0; b < nb; b++) c->vwire.push_back({i, b, nb, nparts});
         nparts += nb;
     }
