@@ -210,42 +210,32 @@ __device__ __forceinline__ void eval_warp_layers(LayerFn layer, int hi, int lo, 
 }
 
 // A chain of F0_PAIR layers (gate 2j = v_2j^2, gate 2j+1 = v_2j+1 v_2j): every
-// pair of entries evolves on its own, so a thread keeps its pairs in registers
+// pair of entries evolves on its own, so a thread keeps a pair in registers
 // through the whole chain, writes each layer with 16-byte stores and needs no
-// barrier between the layers.  `cur` holds the block below layer hi (B
-// entries); the pairs after layer lo go to `nxt`.
-template <class LayerFn>
-__device__ __forceinline__ void eval_pair_chain(LayerFn layer, int hi, int lo, const u64 *cur, u64 *nxt, u32 B,
-                                                u32 chunk)
+// barrier between the layers.  Bound by the latency of one product per layer:
+// the pair stays in W (the product and one fold; the canonical form of what is
+// stored is off the chain) and the layers' pointers are read one ahead (388
+// cycles a layer before, with canonical products and four pairs' slots a
+// thread).  `cur` holds the block below layer hi (B entries); the pairs after
+// layer lo go to `nxt`.
+template <class PtrFn>
+__device__ __forceinline__ void eval_pair_chain(PtrFn ptr, int hi, int lo, const u64 *cur, u64 *nxt, u32 B, u32 chunk)
 {
-    constexpr int PP = EV_MAXB / 2 / EV_NT;  // pairs a thread holds
     const u32 np = B >> 1;
-    u64 x0[PP], x1[PP];
-#pragma unroll
-    for (int h = 0; h < PP; h++) {
-        const u32 q = threadIdx.x + h * EV_NT;
-        x0[h] = (q < np) ? cur[2 * q] : 0;
-        x1[h] = (q < np) ? cur[2 * q + 1] : 0;
-    }
-    for (int i = hi; i >= lo; i--) {
-        ulonglong2 *__restrict__ out = reinterpret_cast<ulonglong2 *>(layer((u32)i).V + (u64)chunk * B);
-#pragma unroll
-        for (int h = 0; h < PP; h++) {
-            const u32 q = threadIdx.x + h * EV_NT;
-            if (q < np) {  // the shorter-latency product: the chain is latency-bound
-                x1[h] = f_mul_wide(x1[h], x0[h]);
-                x0[h] = f_mul_wide(x0[h], x0[h]);
-                out[q] = make_ulonglong2(x0[h], x1[h]);
-            }
+    for (u32 q = threadIdx.x; q < np; q += EV_NT) {
+        u64 x0 = cur[2 * q], x1 = cur[2 * q + 1];
+        const u64 at = (u64)chunk * np + q;
+        ulonglong2 *out = reinterpret_cast<ulonglong2 *>(ptr((u32)hi)) + at;
+#pragma unroll 2
+        for (int i = hi; i >= lo; i--) {
+            ulonglong2 *const next = reinterpret_cast<ulonglong2 *>(ptr((u32)(i > lo ? i - 1 : lo))) + at;
+            x1 = wmul(x1, x0);
+            x0 = wmul(x0, x0);
+            *out = make_ulonglong2(wcanon(x0), wcanon(x1));
+            out = next;
         }
-    }
-#pragma unroll
-    for (int h = 0; h < PP; h++) {
-        const u32 q = threadIdx.x + h * EV_NT;
-        if (q < np) {
-            nxt[2 * q] = x0[h];
-            nxt[2 * q + 1] = x1[h];
-        }
+        nxt[2 * q] = wcanon(x0);
+        nxt[2 * q + 1] = wcanon(x1);
     }
 }
 
@@ -336,9 +326,21 @@ __global__ void __launch_bounds__(EV_NT, EV_MINB) k_eval_seg(const Globals *Gs, 
         if (i == (int)S.warp_from) break;
         const EvLayer L = layer((u32)i);
         if (L.kind == W_F0_PAIR) {  // the chain of pair layers from here, in registers
+            // (its length found 32 layers at a time; layer by layer took 4 us)
             int lo = i;
-            while (lo - 1 >= (int)S.i_lo && lo - 1 != (int)S.warp_from && layer((u32)(lo - 1)).kind == W_F0_PAIR) lo--;
-            eval_pair_chain(layer, i, lo, cur, nxt, B, chunk);
+            const u32 lane = threadIdx.x & 31;
+            while (true) {
+                const int j = lo - 1 - (int)lane;
+                const bool more = j >= (int)S.i_lo && j != (int)S.warp_from && layer((u32)j).kind == W_F0_PAIR;
+                const u32 m = __ballot_sync(0xffffffffu, more);
+                if (m != 0xffffffffu) {
+                    lo -= __ffs(~m) - 1;
+                    break;
+                }
+                lo -= 32;
+            }
+            eval_pair_chain([&](u32 j) { return S.i_hi - j < EV_LC ? s_V[S.i_hi - j] : Ls[j].V; }, i, lo, cur, nxt, B,
+                            chunk);
             __syncthreads();
             u64 *t = cur; cur = nxt; nxt = t;
             i = lo;
