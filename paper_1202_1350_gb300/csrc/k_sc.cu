@@ -488,13 +488,13 @@ __device__ __forceinline__ void bil_run(u64 Aa, u64 Ab, ulonglong2 va, ulonglong
 }
 
 // In-register rounds for e in 2..5: runs of 4 entries (rounds 0, 1), then
-// rounds 2.. on the runs' folded triples, combined like a binary counter.
-// SQUARE's and F0's P carries eq(r_P, .) = lo hi of its split table, and the
-// thread's entries share one hi (2^e entries, e at most half the coordinates),
-// so P is formed with lo alone and hi multiplies the thread's sums and its
-// folded P once.
-__device__ __forceinline__ void gen_regs_runs(const Globals &G, const GenWave &W, u64 x0, u32 e, bool hasB,
-                                              GenSmem &sm, u64 (&h)[15], u64 &pv, u64 &vv, u64 &bv)
+// rounds 2.. on the runs' folded triples, combined like a binary counter.  A
+// first wave's P (and B) carries a factor lo hi of a split table, and the
+// thread's entries share one hi (2^e entries, within one block of the table),
+// so they are formed with lo alone and hi multiplies the thread's sums and
+// its folded P and B once.
+__device__ __forceinline__ void gen_regs_runs(const GenWave &W, u64 x0, u32 e, bool hasB, GenSmem &sm, u64 (&h)[15],
+                                              u64 &pv, u64 &vv, u64 &bv)
 {
     const u32 nruns = 1u << (e - 2), src = W.src;
     const bool b_run = hasB || src == GS_FIRST2;
@@ -503,21 +503,20 @@ __device__ __forceinline__ void gen_regs_runs(const Globals &G, const GenWave &W
     acc128 a[6];
 #pragma unroll
     for (int j = 0; j < 6; j++) acc_zero(a[j]);
-    const bool lohi = src == GS_SQ2 || src == GS_PAIR2 || src == GS_FINAL2;
     const u64 *lo = nullptr;
     u64 hi = 1;
-    if (lohi) {
-        const EqTab &T = G.layers[W.layer].trp;
-        const u64 x = src == GS_FINAL2 ? x0 >> 1 : x0;
-        lo = T.lo + (x & ((1ull << T.h) - 1));
-        hi = T.hi[x >> T.h];
+    if (src != GS_NONE) {
+        const u64 x = src == GS_FINAL2 ? x0 >> 1 : src == GS_FIRST2 ? 2 * x0 : x0;
+        lo = W.inP + (x & ((1ull << W.th) - 1));
+        hi = W.inB[x >> W.th];
     }
     // the second line of each of the thread's tables (32 entries are two)
     // comes while the first is used
     if (nruns > 4) {
         prefetch_l1(W.inV + x0 + 16);
-        if (lohi) prefetch_l1(lo + (src == GS_FINAL2 ? 8 : 16));
-        if (src == GS_NONE) {
+        if (src != GS_NONE) {
+            prefetch_l1(lo + (src == GS_FINAL2 ? 8 : 16));
+        } else {
             prefetch_l1(W.inP + x0 + 16);
             if (hasB) prefetch_l1(W.inB + x0 + 16);
         }
@@ -547,16 +546,20 @@ __device__ __forceinline__ void gen_regs_runs(const Globals &G, const GenWave &W
                 const ulonglong2 *sv = reinterpret_cast<const ulonglong2 *>(W.inV + x0 + 4 * sub);
                 const ulonglong2 va = __ldg(sv), vb = __ldg(sv + 1);
                 v[0] = va.x, v[1] = va.y, v[2] = vb.x, v[3] = vb.y;
-                if (src == GS_SQ2) {
-                    const ulonglong2 *sl = reinterpret_cast<const ulonglong2 *>(lo) + 2 * sub;
-                    const ulonglong2 l = __ldg(sl), l2 = __ldg(sl + 1);
-                    p[0] = wmul(l.x, v[0]), p[1] = wmul(l.y, v[1]), p[2] = wmul(l2.x, v[2]), p[3] = wmul(l2.y, v[3]);
-                } else {
+                const ulonglong2 *sl = reinterpret_cast<const ulonglong2 *>(lo) + (src == GS_FIRST2 ? 4 * sub : 2 * sub);
+                if (src == GS_FIRST2) {
 #pragma unroll
                     for (int q = 0; q < 4; q++) {
-                        const ulonglong2 t = gen_source(G, W, x0 + 4 * sub + q, v[q], v[q & 2]);
-                        p[q] = t.x;
-                        b[q] = t.y;
+                        const ulonglong2 l = __ldg(sl + q);
+                        p[q] = wred(wmul(l.x, v[q]) + l.y);
+                        b[q] = wmul(l.y, v[q]);
+                    }
+                } else {
+                    const ulonglong2 l = __ldg(sl), l2 = __ldg(sl + 1);
+                    p[0] = l.x, p[1] = l.y, p[2] = l2.x, p[3] = l2.y;
+                    if (src == GS_SQ2) {
+#pragma unroll
+                        for (int q = 0; q < 4; q++) p[q] = wmul(p[q], v[q]);
                     }
                 }
             }
@@ -587,10 +590,11 @@ __device__ __forceinline__ void gen_regs_runs(const Globals &G, const GenWave &W
     for (int j = 0; j < 6; j++) h[j] = acc_red(a[j]);
 #pragma unroll
     for (int j = 0; j < 9; j++) h[6 + j] = sm.hs[j][threadIdx.x];
-    if (lohi) {  // every sum and P are linear in it (B = 0)
+    if (src != GS_NONE) {  // every sum, P and B are linear in it
 #pragma unroll
         for (int j = 0; j < 15; j++) h[j] = wmul(hi, h[j]);
         tp = wmul(hi, tp);
+        if (b_run) tb = wmul(hi, tb);
     }
     pv = tp;
     vv = tv;
@@ -649,6 +653,7 @@ __device__ __noinline__ int gen_chunk(const Globals &G, const GenWave &W, u32 ch
     const u32 na = 1u << (nr - e);
     const u64 base = (u64)chunk << nr;
     const bool hasB = (W.flags & WF_HASB) != 0;
+    if (e > 0 && tid < na) prefetch_l1(W.inV + base + ((u64)tid << e));  // while the challenges come
     if (tid < nr) sm.r[tid] = G.chal[W.chal_off + tid];
     __syncthreads();
     u64 pv = 0, vv = 0, bv = 0;
@@ -658,7 +663,7 @@ __device__ __noinline__ int gen_chunk(const Globals &G, const GenWave &W, u32 ch
         for (int i = 0; i < 15; i++) h[i] = 0;
         if (tid < na) {
             const u64 x0 = base + ((u64)tid << e);
-            gen_regs_runs(G, W, x0, e, hasB, sm, h, pv, vv, bv);
+            gen_regs_runs(W, x0, e, hasB, sm, h, pv, vv, bv);
         }
         u64 h16[16];
 #pragma unroll

@@ -45,7 +45,7 @@ struct LayerDev {
     u64 tr_q;         // transcript offset of q(0..s_{i+1})
     EqTab trp, tr1, tr2;  // eq tables of r_P, r1, r2 (r1, r2: table-built layers, verifier)
     u64 *P2, *B2, *P3, *B3;   // EXPLICIT: phase-2/3 tables over layer i+1 (B* NULL if !has_add)
-    u64 *mu, *mei;            // MATMULT: tables of k_mm_tables (n entries each)
+    u64 *mu, *mei;            // MATMULT: tables of k_mm_tables (n entries each; mei then n zeros)
     const unsigned char *type;  // EXPLICIT only
     const u32 *in1, *in2;
     const u32 *by1_off, *by1_g;  // gates grouped by in1: offsets [S_{i+1}+1], gate ids [S_i]
@@ -197,6 +197,9 @@ struct GenWave {
     u32 layer;
     u32 chal_off;
     u32 pad;
+    u32 th;            // first wave with a source: its factor of entry x (SQ2, PAIR2, MM2), x / 2 (FINAL2)
+                       // or 2 x (FIRST2) is lo[index mod 2^th] hi[index >> th]; lo is inP, hi is inB
+    u32 pad2;
     const u64 *inP, *inV, *inB;
     u64 *outP, *outV, *outB;
     u64 *part;         // partials: part[(k * nchunks + chunk) * 3 + t]

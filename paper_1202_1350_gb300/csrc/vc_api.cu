@@ -549,7 +549,7 @@ static size_t layout(vc_circuit *c, uintptr_t base, uintptr_t hbase)
         }
         if (L.kind == W_MATMULT) {
             L.mu = A.take<u64>(u64(1) << (L.s / 3));
-            L.mei = A.take<u64>(u64(1) << (L.s / 3));
+            L.mei = A.take<u64>(u64(2) << (L.s / 3));
         }
         L.P2 = tabs ? A.take<u64>(S(i + 1)) : nullptr;
         L.P3 = tabs ? A.take<u64>(S(i + 1)) : nullptr;
@@ -584,6 +584,8 @@ static size_t layout(vc_circuit *c, uintptr_t base, uintptr_t hbase)
         if (grp.size() <= g) grp.resize(g + 1);
         for (u32 ch = 0; ch < nchunks; ch++) grp[g].push_back({type, idx, ch, 0u});
     };
+    u32 line_smax = 0;
+    for (u32 i = 0; i <= d; i++) line_smax = std::max(line_smax, c->s[i]);
     for (u32 i = 0; i < d; i++) {
         const u32 n = c->s[i + 1];
         u32 l0 = 0, g = 0;
@@ -593,6 +595,10 @@ static size_t layout(vc_circuit *c, uintptr_t base, uintptr_t hbase)
             // first chunks of more than 20 coordinates take up to two more, so
             // that the next wave is their last (a third was a launch of its own)
             u32 cap = (w == 0) ? c->cfg.ln_chunk0 : LN_CHUNKW_LOG;
+            // circuits of up to 2^16 entries a layer: halves of the default chunk,
+            // whose chain is half as long (F2 2^14 38.9 -> 33.1 us; in wider ones the
+            // load decides: F0 2^16 199 -> 216, F2 2^20 91 -> 94)
+            if (w == 0 && cap == LN_CHUNK0_LOG && n >= LN_CHUNK0_LOG && line_smax <= 16) cap = LN_CHUNK0_LOG - 1;
             if (w == 0 && cap == LN_CHUNK0_LOG && n > cap + LN_CHUNKW_LOG)
                 cap = std::min(LN_CHUNK0_LOG + LN_XTRA, n - LN_CHUNKW_LOG);
             const u32 nl = std::min(cap, n - l0);
@@ -705,7 +711,7 @@ static size_t layout(vc_circuit *c, uintptr_t base, uintptr_t hbase)
             } else {
                 // F0 pair and final layers: the first wave's round 0 leaves a
                 // factor out of P if it runs in registers (applied by k_final)
-                const bool regs = std::min(c->cfg.gn_chunk, n) > WV_LOG;
+                const bool regs = std::min(c->cfg.gn_chunk, n) > WV_LOG;  // (a smaller default chunk is above WV_LOG too)
                 Sc.kind = PK_GEN_EZ;
                 switch (L.kind) {
                 case W_SQUARE: src = GS_SQ2; break;
@@ -732,6 +738,14 @@ static size_t layout(vc_circuit *c, uintptr_t base, uintptr_t hbase)
                     break;
                 }
             }
+            u32 th = 0;
+            if (src == GS_MM2) {
+                th = L.s / 3;
+            } else if (src != GS_NONE) {
+                inP = L.trp.lo;
+                inB = L.trp.hi;
+                th = L.trp.h;
+            }
             const u32 sci = (u32)P.scis.size();
             const bool prod = Sc.kind < PK_GEN_FIRST;
             if (prod && ph != 4) {
@@ -746,6 +760,12 @@ static size_t layout(vc_circuit *c, uintptr_t base, uintptr_t hbase)
             const u32 split = (c->cfg.pr_split == VC_SPLIT_WIDEST) ? smax : c->cfg.pr_split;
             u32 C = prod ? ((n < split && c->cfg.pr_chunk > 1) ? c->cfg.pr_chunk - 1 : c->cfg.pr_chunk)
                          : c->cfg.gn_chunk;
+            // With the default shapes general instances of few coordinates take
+            // smaller chunks: a lone thread's 32 entries are a chain of about
+            // 2,700 cycles per 4 (F0 2^11 44.8 us with 2^12, F0 2^14 90 against 85
+            // with 2^11; under load 2^12 wins: F0 2^16 199 against 222).
+            const u32 gsmall = n <= 12 ? 10u : n <= 15 ? 11u : GN_CHUNK_LOG;
+            if (!prod && c->cfg.gn_chunk == GN_CHUNK_LOG) C = gsmall;
             // with the default shapes wide PROD instances take larger chunks
             // (about 7,000 cycles of a chunk do not depend on its size): 2^13
             // from 14 coordinates, 2^14 from 19.  F2 2^22 waves 206 us with 2^12
@@ -825,6 +845,7 @@ static size_t layout(vc_circuit *c, uintptr_t base, uintptr_t hbase)
                               (has_tail ? WF_TAIL : 0);
                     W.layer = i;
                     W.chal_off = Sc.chal_off + r0;
+                    W.th = th;
                     W.inP = inP;
                     W.inV = inV;
                     W.inB = inB;
@@ -993,6 +1014,8 @@ bool plan_valid(const Plan &P)
     for (size_t k = 0; k < P.gw.size(); k++) {
         const GenWave &W = P.gw[k];
         if (W.circ >= nc || W.sci >= P.scis.size() || P.scis[W.sci].circ != W.circ) return false;
+        // a thread's entries share one upper factor of the source's split table
+        if (W.src != GS_NONE && W.e && W.e + (W.src == GS_FIRST2) - (W.src == GS_FINAL2) > W.th) return false;
         if (W.nr > GN_CHUNK_LOG || W.e > (u32)GN_M || W.e > W.nr || W.nr - W.e > WV_LOG || (W.e && W.e < 2))
             return false;
         if ((W.flags & WF_TAIL) && (k + 1 >= P.gw.size() || P.gw[k + 1].nchunks != 1 || P.gw[k + 1].sci != W.sci ||
