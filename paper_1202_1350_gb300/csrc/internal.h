@@ -119,6 +119,7 @@ struct Plan {
     std::vector<u32> seg_maxblock;                         // per step: largest block of its runs
     std::vector<LineWaveDev> lw;
     std::vector<BuildItem> builds, mms;  // k_build23 (EXPLICIT), k_mm_tables (MATMULT)
+    bool mm_inputs = true;  // every MATMULT layer reads its circuit's inputs
     std::vector<HeavyItem> heavy;  // explicit layers' entries with long gate lists (k_build_heavy)
     std::vector<SciDev> scis;
     std::vector<ProdWave> pw;
@@ -148,7 +149,7 @@ struct Plan {
     // execution
     cudaStream_t aux = nullptr;  // eq tables and product weights, concurrent with evaluation
     cudaStream_t cap = nullptr;  // private stream: graph capture, creation work
-    cudaEvent_t ev_fork = nullptr, ev_tables = nullptr;
+    cudaEvent_t ev_fork = nullptr, ev_tables = nullptr, ev_checked = nullptr;
     cudaEvent_t ev_params = nullptr;  // a batch's parameter table was copied
     // stage events are recorded on a side branch of the graph (evs), so that
     // timing a stage adds no node between two launches (and keeps the final

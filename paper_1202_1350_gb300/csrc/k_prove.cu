@@ -76,19 +76,37 @@ void launch_params_batch(Globals *Gs, const CallParams *cp, int n, cudaStream_t 
 
 
 // Layer evaluation: V_i[g] = V_{i+1}[in1] op V_{i+1}[in2] (Sec. 6.2.4); an
-// item covers 256 gates of one layer of one circuit.
+// item covers 256 `reps` gates of one layer of one circuit, `reps` (<= EVL_REPS)
+// a thread with their operands' loads in flight together (a gate a thread,
+// each CTA spent most of its life on descriptors: 17 us for MATMULT 128's 2^21,
+// now 12; a 2^15-gate layer stays at a gate a thread: 31.8 us of evaluation
+// stage for the pattern circuit of 2^14, 38.0 with eight).
 __global__ void __launch_bounds__(256) k_eval_layer(const Globals *Gs, const LayerEval *le, const Item *items)
 {
+    constexpr u32 R = EVL_REPS;
     const Item it = items[blockIdx.x];
     const LayerEval E = le[it.wave];
-    const LayerDev &L = Gs[E.circ].layers[E.layer];
-    const u64 g = (u64)it.chunk * 256 + threadIdx.x;
-    if (g < (1ull << L.s)) {
-        u64 a, b;
-        u32 mul;
-        gate_wiring(L, g, a, b, mul);
-        const u64 x = L.Vn[a], y = L.Vn[b];
-        L.V[g] = mul ? f_mul(x, y) : f_add(x, y);
+    const LayerDev L = Gs[E.circ].layers[E.layer];
+    const u64 n = 1ull << L.s, g0 = (u64)it.chunk * (256 * E.reps) + threadIdx.x;
+    u64 x[R], y[R];
+    u32 muls = 0;
+#pragma unroll
+    for (u32 r = 0; r < R; r++) {
+        const u64 g = g0 + 256 * r;
+        x[r] = y[r] = 0;
+        if (r < E.reps && g < n) {
+            u64 a, b;
+            u32 mul;
+            gate_wiring(L, g, a, b, mul);
+            x[r] = L.Vn[a];
+            y[r] = L.Vn[b];
+            muls |= mul << r;
+        }
+    }
+#pragma unroll
+    for (u32 r = 0; r < R; r++) {
+        const u64 g = g0 + 256 * r;
+        if (r < E.reps && g < n) L.V[g] = (muls >> r) & 1 ? f_mul_wide(x[r], y[r]) : f_add(x[r], y[r]);
     }
 }
 

@@ -1136,7 +1136,8 @@ __global__ void __launch_bounds__(256) k_final(Globals *Gs, const RoundRef *roun
         }
         if (lane == 0) final_round(Gs, R, S, h, h2);
     }
-    for (u64 t = gt; t < (u64)(nrounds - nbig); t += nthreads) {
+    // (from the grid's end: the CTAs that had no round to themselves first)
+    for (u64 t = nthreads - 1 - gt; t < (u64)(nrounds - nbig); t += nthreads) {
         const RoundRef R = rounds[nbig + t];
         RoundScalars S = round_scalars_pre(R);
         if (R.kind < PK_GEN_FIRST) S.v1 = *R.v1;
@@ -1157,7 +1158,7 @@ void launch_final(Globals *Gs, const RoundRef *rounds, int nrounds, int nbig, co
                   cudaStream_t st)
 {
     const u64 warp_blocks = ((u64)nbig * 32 + 255) / 256, thread_blocks = ((u64)(nrounds - nbig) + 255) / 256;
-    u64 blocks = warp_blocks > thread_blocks ? warp_blocks : thread_blocks;
+    u64 blocks = warp_blocks + thread_blocks;
     if (blocks < (u64)nouts) blocks = (u64)nouts;
     if (blocks < 64) blocks = 64;
     if (blocks > (u64)device_sms() * 8) blocks = (u64)device_sms() * 8;

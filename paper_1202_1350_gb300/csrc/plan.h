@@ -315,10 +315,15 @@ struct EvalSeg {
     u32 pad2;
 };
 
-// A layer evaluated on its own (MATMULT or EXPLICIT wiring).
+// A layer evaluated on its own (MATMULT or EXPLICIT wiring), by items of 256
+// `reps` gates: about 1024 CTAs for wide layers, a gate a thread below 2^19.
+#define EVL_REPS 8u
+__host__ __device__ __forceinline__ u32 eval_reps(u32 s) { return s <= 18 ? 1u : s >= 21 ? EVL_REPS : 1u << (s - 18); }
 struct LayerEval {
     u32 circ;
     u32 layer;
+    u32 reps;
+    u32 pad;
 };
 
 // Work item of k_build23: BUILD_ENTRIES entries of layer i+1's phase-2/3 tables.
@@ -405,8 +410,9 @@ void launch_waves(const Globals *Gs, const LineWaveDev *lw, const ProdWave *pw, 
                   int ntasks, u32 *ctr, cudaStream_t st);
 // Rounds [0, nbig) are reduced a warp each: all rounds when there are at most
 // FINAL_ALL_WARPS (the warps of one full launch), else those with more than
-// FINAL_WARP_MIN chunk partials; the rest a thread each.
-#define FINAL_WARP_MIN 8u
+// FINAL_WARP_MIN chunk partials; the rest a thread each (those with up to 8 a
+// thread: 196.6 us for the 56-circuit batch, so 194.3).
+#define FINAL_WARP_MIN 2u
 #define FINAL_ALL_WARPS ((u32)device_sms() * 8u * 8u)
 void launch_final(Globals *Gs, const RoundRef *rounds, int nrounds, int nbig, const u32 *outs, int nouts,
                   cudaStream_t st);

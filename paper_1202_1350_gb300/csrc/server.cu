@@ -205,6 +205,7 @@ vc_status launch(vc_server *s, Slot &sl)
     sl.P.cap = res.cap;
     sl.P.ev_fork = res.ev_fork;
     sl.P.ev_tables = res.ev_tables;
+    sl.P.ev_checked = res.ev_checked;
     sl.P.ev_params = res.ev_params;
     const int n = (int)cs.size();
     const size_t need = plan_bytes(sl.P, true) + (size_t)n * sizeof(CallParams) + 512;

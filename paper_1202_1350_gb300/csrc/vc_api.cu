@@ -292,8 +292,9 @@ static void plan_eval(vc_circuit *c)
         } else {
             const u32 layer = (u32)(-step - 1);
             const u32 idx = (u32)P.levs.size();
-            P.levs.push_back({0u, layer});
-            const u64 blocks = ((u64(1) << c->s[layer]) + 255) / 256;
+            const u32 reps = eval_reps(c->s[layer]);
+            P.levs.push_back({0u, layer, reps, 0u});
+            const u64 blocks = ((u64(1) << c->s[layer]) + 256 * reps - 1) / (256 * reps);
             for (u64 b = 0; b < blocks; b++) P.lev_items[k].push_back({idx, (u32)b});
         }
     }
@@ -389,7 +390,7 @@ static void staged_partition(vc_circuit *c, Arena &A)
     for (const BuildItem &b : P.mms) c->stMm[list_of(b.layer)].push_back(b);
     c->stEval.assign(d, {});
     for (u32 i = 0; i < d; i++) {
-        const u64 blocks = ((u64(1) << c->s[i]) + 255) / 256;
+        const u64 per = 256 * eval_reps(c->s[i]), blocks = ((u64(1) << c->s[i]) + per - 1) / per;
         for (u64 b = 0; b < blocks; b++) c->stEval[i].push_back({i, (u32)b});
     }
     c->st_evalstep.assign(d, -1);
@@ -431,7 +432,7 @@ static void staged_partition(vc_circuit *c, Arena &A)
 static cudaError_t staged_upload(vc_circuit *c)
 {
     std::vector<LayerEval> lev(c->d);
-    for (u32 i = 0; i < c->d; i++) lev[i] = {0u, i};
+    for (u32 i = 0; i < c->d; i++) lev[i] = {0u, i, eval_reps(c->s[i]), 0u};
     cudaError_t e = upload(c->d_stLev, lev);
     for (size_t i = 0; e == cudaSuccess && i < c->stA.size(); i++)
         for (size_t g = 0; e == cudaSuccess && g < c->stA[i].size(); g++) e = upload(c->d_stA[i][g], c->stA[i][g]);
@@ -879,6 +880,9 @@ static size_t layout(vc_circuit *c, uintptr_t base, uintptr_t hbase)
         P.rounds[t.round].nchunks2 = t.nchunks;
     }
     P.outs.assign(1, 0u);
+    // every MATMULT layer reads the circuit's inputs, which are in layer d before the launches
+    P.mm_inputs = true;
+    for (u32 i = 0; i + 1 < d; i++) P.mm_inputs &= c->kind[i] != W_MATMULT;
     sort_tasks(P);
 
     // verifier scratch
@@ -1156,7 +1160,7 @@ cudaError_t plan_resources(Plan &P)
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&P.cap, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&P.evs, cudaStreamNonBlocking);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&P.evs_aux, cudaStreamNonBlocking);
-    for (cudaEvent_t *ev : {&P.ev_fork, &P.ev_tables, &P.ev_params, &P.ev_mark})
+    for (cudaEvent_t *ev : {&P.ev_fork, &P.ev_tables, &P.ev_checked, &P.ev_params, &P.ev_mark})
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
     return e;
 }
@@ -1173,7 +1177,7 @@ void plan_drop_graph(Plan &P)
 void plan_release(Plan &P)
 {
     plan_drop_graph(P);
-    for (cudaEvent_t *ev : {&P.ev_fork, &P.ev_tables, &P.ev_params, &P.ev_mark}) {
+    for (cudaEvent_t *ev : {&P.ev_fork, &P.ev_tables, &P.ev_checked, &P.ev_params, &P.ev_mark}) {
         if (*ev) cudaEventDestroy(*ev);
         *ev = nullptr;
     }
@@ -1247,6 +1251,7 @@ void plan_merge(Plan &B, const std::vector<vc_circuit *> &cs)
             b.circ = cj;
             B.mms.push_back(b);
         }
+        B.mm_inputs &= P.mm_inputs;
         for (HeavyItem b : P.heavy) {
             b.circ = cj;
             B.heavy.push_back(b);
@@ -1328,19 +1333,25 @@ void enqueue_plan(Plan &P, cudaStream_t st)
                          P.own_params && k == 0);
         launch_eval_layers(Gs, P.d_levs, P.d_lev_items[k], (int)P.lev_items[k].size(), st);
     }
-    // inputs not checked by an evaluation segment: the check only latches a
-    // status read after the proof, so it need not delay the evaluation
-    launch_check_inputs(Gs, P.d_checks, (int)P.checks.size(), st);
     mark(VC_STAGE_EVAL, 1, st);
     cudaStreamWaitEvent(sa, P.ev_fork, 0);
     mark(VC_STAGE_TABLES, 0, sa);
     launch_coins(Gs, P.d_setups, (int)P.setups.size(), P.d_eqjobs, (int)P.eqjobs.size(), P.d_scis, P.d_pw, (int)P.pw.size(),
                  P.d_lw, (int)P.lw.size(), sa);
     mark(VC_STAGE_TABLES, 1, sa);
+    // MATMULT layers' phase-2 factors need the coins and the layer's inputs:
+    // beside the evaluation if those are the circuit's (with the wider
+    // evaluation items: MATMULT 128 from 108 to 100 us, pattern 2^14 163 to 158)
+    if (P.mm_inputs) launch_mm_tables(Gs, P.d_mms, (int)P.mms.size(), sa);
     cudaEventRecord(P.ev_tables, sa);
+    // inputs not checked by an evaluation segment: the check only latches a
+    // status read after the proof, so nothing but the end waits for it
+    if (!P.checks.empty()) {
+        launch_check_inputs(Gs, P.d_checks, (int)P.checks.size(), sa);
+        cudaEventRecord(P.ev_checked, sa);
+    }
     cudaStreamWaitEvent(st, P.ev_tables, 0);
-    // MATMULT layers' phase-2 factors (they need the coins and the layer's inputs)
-    launch_mm_tables(Gs, P.d_mms, (int)P.mms.size(), st);
+    if (!P.mm_inputs) launch_mm_tables(Gs, P.d_mms, (int)P.mms.size(), st);
     // line reductions, product-weighted and on-the-fly general waves
     mark(VC_STAGE_WAVES, 0, st);
     if (nA) waves(P.groupsA[0], P.d_groupsA[0], 0);
@@ -1365,6 +1376,7 @@ void enqueue_plan(Plan &P, cudaStream_t st)
     mark(VC_STAGE_FINAL, 0, st);
     launch_final(P.d_G, P.d_rounds, (int)P.rounds.size(), (int)P.nbig, P.d_outs, (int)P.outs.size(), st);
     mark(VC_STAGE_FINAL, 1, st);
+    if (!P.checks.empty()) cudaStreamWaitEvent(st, P.ev_checked, 0);
     mark(VC_STAGE_PROOF, 1, st);
     // the branches join the stream at the end
     for (int k = 0; k < 2; k++)
