@@ -280,7 +280,7 @@ typedef enum {
                                and on-the-fly general sum-checks (their single-chunk
                                later waves run inside it)                                */
     VC_STAGE_WAVESN = 4,    /* later persistent launches of the same kinds (wide layers) */
-    VC_STAGE_BUILD = 5,     /* phase-2/3 wiring tables (MATMULT, F0, EXPLICIT layers)    */
+    VC_STAGE_BUILD = 5,     /* phase-2/3 wiring tables (EXPLICIT layers)                 */
     VC_STAGE_TABWAVES = 6,  /* general sum-checks over the built tables                  */
     VC_STAGE_FINAL = 7,     /* per-round reductions into the transcript                  */
     VC_NUM_STAGES = 8

@@ -55,26 +55,6 @@ __device__ __forceinline__ u64 warp_sum16(u64 (&v)[16])
     return wred(r);
 }
 
-// Sum over the warp of 32 values per lane: afterwards lane l holds the total
-// of value index l.  Inputs in W.
-__device__ __forceinline__ u64 warp_sum32(u64 (&v)[32])
-{
-    const u32 lane = threadIdx.x & 31;
-#pragma unroll
-    for (int step = 0; step < 5; step++) {
-        const int o = 16 >> step, half = 16 >> step;
-        const bool up = (lane & o) != 0;
-#pragma unroll
-        for (int i = 0; i < half; i++) {
-            const u64 send = up ? v[i] : v[i + half];
-            const u64 keep = up ? v[i + half] : v[i];
-            v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
-            if (step & 1) v[i] = wred(v[i]);
-        }
-    }
-    return wred(v[0]);
-}
-
 // (The per-wave weight tables of the PROD waves are built with the coins, in
 // k_coins.cu.)
 
@@ -154,12 +134,6 @@ __device__ __forceinline__ void cp_wait()
 
 // Bring the line holding p into L1 ahead of its load (no register cost).
 __device__ __forceinline__ void prefetch_l1(const void *p) { asm volatile("prefetch.global.L1 [%0];" ::"l"(p)); }
-
-// Sum of the four warps' per-warp round sums (W values).
-__device__ __forceinline__ u64 cta_sum4(const u64 *a, const u64 *b, const u64 *c, const u64 *d)
-{
-    return wred(*a + *b + *c + *d);
-}
 
 // The next task of the CTA (thread 0; ctr NULL: the CTA keeps the one it has).
 __device__ __forceinline__ int claim_task(u32 *ctr)
@@ -445,7 +419,7 @@ __device__ __forceinline__ void gen_run(const u64 (&p)[4], const u64 (&v)[4], co
 }
 
 // P (and B, for FIRST2) of one entry x of a first wave whose tables follow
-// from the wiring (GS_*); v = V[x], ve = V[x with bit 0 cleared]// (.x: P, .y: B).
+// from the wiring (GS_*); v = V[x], ve = V[x with bit 0 cleared] (.x: P, .y: B).
 __device__ __noinline__ ulonglong2 gen_source(const Globals &G, const GenWave &W, u64 x, u64 v, u64 ve)
 {
     u64 p, b = 0;
