@@ -57,7 +57,7 @@ constexpr u32 VC_VALUES_SLOTTED = VC_VALUES_STAGED | VC_VALUES_WINDOWED;
 // Layers whose phases 2 and 3 run over tables built by k_build23, and those
 // whose phase 2 looks up eq(r_P, .).
 inline bool needs_tables(u32 kind) { return kind == W_EXPLICIT; }
-inline bool needs_eq_rp(u32 kind) { return kind != W_TREE && kind != W_MATMULT; }
+inline bool needs_eq_rp(u32 kind, bool host) { return kind == W_TREE ? host : kind != W_MATMULT; }
 
 // Bump allocator over one device allocation (base 0: sizing pass).
 struct Arena {

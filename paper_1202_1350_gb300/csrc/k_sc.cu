@@ -418,9 +418,13 @@ __device__ __forceinline__ void gen_run(const u64 (&p)[4], const u64 (&v)[4], co
     }
 }
 
-// P (and B, for FIRST2) of one entry x of a first wave whose tables follow
-// from the wiring (GS_*); v = V[x], ve = V[x with bit 0 cleared] (.x: P, .y: B).
-__device__ __noinline__ ulonglong2 gen_source(const Globals &G, const GenWave &W, u64 x, u64 v, u64 ve)
+// First waves whose B follows from the wiring too.
+__device__ __forceinline__ bool source_b(u32 src) { return src == GS_FIRST2 || src == GS_TREE2; }
+
+// P (and B, for FIRST2 and TREE2) of one entry x of a first wave whose tables
+// follow from the wiring (GS_*); v = V[x], vn = V[x with bit 0 cleared] (PAIR2)
+// or set (TREE2) (.x: P, .y: B).
+__device__ __noinline__ ulonglong2 gen_source(const Globals &G, const GenWave &W, u64 x, u64 v, u64 vn)
 {
     u64 p, b = 0;
     if (W.src == GS_MM2) {
@@ -431,8 +435,12 @@ __device__ __noinline__ ulonglong2 gen_source(const Globals &G, const GenWave &W
     const EqTab &T = G.layers[W.layer].trp;
     switch (W.src) {
     case GS_SQ2: p = wmul(eq_at(T, x), v); break;
-    case GS_PAIR2: p = wmul(eq_at(T, x), ve); break;
+    case GS_PAIR2: p = wmul(eq_at(T, x), vn); break;
     case GS_FINAL2: p = (x & 1) ? wmul(eq_at(T, x >> 1), v) : 0; break;
+    case GS_TREE2:
+        p = (x & 1) ? 0 : eq_at(T, x >> 1);
+        b = wmul(p, vn);
+        break;
     default: {  // GS_FIRST2
         const u64 wa = eq_at(T, 2 * x + 1);
         b = wmul(wa, v);
@@ -471,7 +479,7 @@ __device__ __forceinline__ void gen_regs_runs(const GenWave &W, u64 x0, u32 e, b
                                               u64 &pv, u64 &vv, u64 &bv)
 {
     const u32 nruns = 1u << (e - 2), src = W.src;
-    const bool b_run = hasB || src == GS_FIRST2;
+    const bool b_run = hasB || source_b(src), half = src == GS_FINAL2 || src == GS_TREE2;
 #pragma unroll
     for (int j = 0; j < 9; j++) sm.hs[j][threadIdx.x] = 0;
     acc128 a[6];
@@ -480,7 +488,7 @@ __device__ __forceinline__ void gen_regs_runs(const GenWave &W, u64 x0, u32 e, b
     const u64 *lo = nullptr;
     u64 hi = 1;
     if (src != GS_NONE) {
-        const u64 x = src == GS_FINAL2 ? x0 >> 1 : src == GS_FIRST2 ? 2 * x0 : x0;
+        const u64 x = half ? x0 >> 1 : src == GS_FIRST2 ? 2 * x0 : x0;
         lo = W.inP + (x & ((1ull << W.th) - 1));
         hi = W.inB[x >> W.th];
     }
@@ -489,7 +497,7 @@ __device__ __forceinline__ void gen_regs_runs(const GenWave &W, u64 x0, u32 e, b
     if (nruns > 4) {
         prefetch_l1(W.inV + x0 + 16);
         if (src != GS_NONE) {
-            prefetch_l1(lo + (src == GS_FINAL2 ? 8 : 16));
+            prefetch_l1(lo + (half ? 8 : 16));
         } else {
             prefetch_l1(W.inP + x0 + 16);
             if (hasB) prefetch_l1(W.inB + x0 + 16);
@@ -520,7 +528,7 @@ __device__ __forceinline__ void gen_regs_runs(const GenWave &W, u64 x0, u32 e, b
                 const ulonglong2 *sv = reinterpret_cast<const ulonglong2 *>(W.inV + x0 + 4 * sub);
                 const ulonglong2 va = __ldg(sv), vb = __ldg(sv + 1);
                 v[0] = va.x, v[1] = va.y, v[2] = vb.x, v[3] = vb.y;
-                const ulonglong2 *sl = reinterpret_cast<const ulonglong2 *>(lo) + (src == GS_FIRST2 ? 4 * sub : 2 * sub);
+                const ulonglong2 *sl = reinterpret_cast<const ulonglong2 *>(lo) + (src == GS_FIRST2 ? 4 * sub : half ? sub : 2 * sub);
                 if (src == GS_FIRST2) {
 #pragma unroll
                     for (int q = 0; q < 4; q++) {
@@ -528,6 +536,10 @@ __device__ __forceinline__ void gen_regs_runs(const GenWave &W, u64 x0, u32 e, b
                         p[q] = wred(wmul(l.x, v[q]) + l.y);
                         b[q] = wmul(l.y, v[q]);
                     }
+                } else if (src == GS_TREE2) {
+                    const ulonglong2 l = __ldg(sl);
+                    p[0] = l.x, p[1] = 0, p[2] = l.y, p[3] = 0;
+                    b[0] = wmul(l.x, v[1]), b[1] = 0, b[2] = wmul(l.y, v[3]), b[3] = 0;
                 } else {
                     const ulonglong2 l = __ldg(sl), l2 = __ldg(sl + 1);
                     p[0] = l.x, p[1] = l.y, p[2] = l2.x, p[3] = l2.y;
@@ -652,13 +664,14 @@ __device__ __noinline__ int gen_chunk(const Globals &G, const GenWave &W, u32 ch
             pv = ld_in(W.inP + x, ext);
             bv = hasB ? ld_in(W.inB + x, ext) : 0;
         } else {
-            const ulonglong2 t = gen_source(G, W, x, vv, W.src == GS_PAIR2 ? ld_in(W.inV + (x & ~1ull), ext) : vv);
+            const u64 xn = W.src == GS_TREE2 ? x | 1 : W.src == GS_PAIR2 ? x & ~1ull : x;
+            const ulonglong2 t = gen_source(G, W, x, vv, xn != x ? ld_in(W.inV + xn, ext) : vv);
             pv = t.x;
             bv = t.y;
         }
     }
     const int next = claim_task(ctr);
-    gen_cross(hasB || W.src == GS_FIRST2, pv, vv, bv, e, tid, nr, sm);
+    gen_cross(hasB || source_b(W.src), pv, vv, bv, e, tid, nr, sm);
     __syncthreads();
     // four threads a value: in-register rounds from the warps' sums, cross
     // rounds from their pairs' terms

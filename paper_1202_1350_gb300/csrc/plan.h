@@ -116,7 +116,8 @@ enum : u32 {
     PK_TREE2 = 7,
     PK_TREE2B = 8,
     PK_GEN_FIRST = 16,
-    PK_GEN_EZ = 16,    // phase 2 of SQUARE and F0 layers, P and B formed from the wiring (times eq(z, rP))
+    PK_GEN_EZ = 16,    // phase 2 of SQUARE, F0 and (values in host memory) TREE layers, P and B formed from
+                       // the wiring (times eq(z, rP))
     PK_GEN_PAIR2 = 17,   // phase 2 of F0_PAIR and
     PK_GEN_FINAL2 = 18,  // F0_FINAL layers with a first wave in registers (bil_run)
     PK_GEN_TAB = 19    // tables built by k_build23 (EXPLICIT) or k_mm_tables (MATMULT)
@@ -128,7 +129,10 @@ enum : u32 {
 //   FINAL2  P[2q+1] = eq(rP, q) V[2q+1], P[2q] = 0
 //   FIRST2  P[x] = eq(rP, 2x) V[x] + eq(rP, 2x+1), B[x] = eq(rP, 2x+1) V[x]
 //   MM2     P[(k, i, 0)] = u[k] ei[i] (inP, inB: the tables of k_mm_tables), P[(., ., 1)] = 0
-enum : u32 { GS_NONE = 0, GS_SQ2 = 1, GS_PAIR2 = 2, GS_FINAL2 = 3, GS_FIRST2 = 4, GS_MM2 = 5 };
+//   TREE2   P[2g] = eq(rP, g), B[2g] = P[2g] V[2g+1], P and B 0 at odd entries
+//           (values in host memory only: one pass over V, where PK_TREE2 and
+//           PK_TREE2B are two and the odd entries' sectors cross the link twice)
+enum : u32 { GS_NONE = 0, GS_SQ2 = 1, GS_PAIR2 = 2, GS_FINAL2 = 3, GS_FIRST2 = 4, GS_MM2 = 5, GS_TREE2 = 6 };
 
 // PROD: a chunk of more than 2^PR_C entries is a matrix of 2^kr rows of 2^PR_C
 // columns, kr <= PR_R (128 threads per CTA)
@@ -197,7 +201,7 @@ struct GenWave {
     u32 layer;
     u32 chal_off;
     u32 pad;
-    u32 th;            // first wave with a source: its factor of entry x (SQ2, PAIR2, MM2), x / 2 (FINAL2)
+    u32 th;            // first wave with a source: its factor of entry x (SQ2, PAIR2, MM2), x / 2 (FINAL2, TREE2)
                        // or 2 x (FIRST2) is lo[index mod 2^th] hi[index >> th]; lo is inP, hi is inB
     u32 pad2;
     const u64 *inP, *inV, *inB;

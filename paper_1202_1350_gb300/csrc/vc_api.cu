@@ -538,7 +538,7 @@ static size_t layout(vc_circuit *c, uintptr_t base, uintptr_t hbase)
         L.tr_msg = c->tr_msg[i];
         L.tr_q = c->tr_q[i];
         const u64 *r = G.chal + L.chal_off;
-        if (needs_eq_rp(L.kind)) {
+        if (needs_eq_rp(L.kind, host)) {
             L.trp = take_eq(A, r, L.s);
             P.eqjobs.push_back({L.trp, 0u, L.chal_off});
         }
@@ -678,7 +678,7 @@ static size_t layout(vc_circuit *c, uintptr_t base, uintptr_t hbase)
             // ph 4: the second instance of a TREE layer's phase 2 (PK_TREE2B),
             // over the odd entries of layer i+1; its round j belongs to round
             // j + 1 of phase 2
-            if (ph == 4 && L.kind != W_TREE) continue;
+            if (ph == 4 && (L.kind != W_TREE || host)) continue;
             const u32 n = (ph == 1) ? c->s[i] : (ph == 4) ? c->s[i + 1] - 1 : c->s[i + 1];
             if (n == 0) continue;
             const u32 roff = (ph == 1) ? 0 : (ph == 2) ? c->s[i] : (ph == 4) ? c->s[i] + 1 : c->s[i] + c->s[i + 1];
@@ -716,7 +716,15 @@ static size_t layout(vc_circuit *c, uintptr_t base, uintptr_t hbase)
                 Sc.kind = PK_GEN_EZ;
                 switch (L.kind) {
                 case W_SQUARE: src = GS_SQ2; break;
-                case W_TREE: Sc.kind = PK_TREE2; break;
+                case W_TREE:
+                    // with values in host memory every read crosses the link, which
+                    // bounds the launch: one pass over V, formed like the others
+                    // (F2 2^20 1.07 ms with the two product-weighted passes)
+                    if (host)
+                        src = GS_TREE2;
+                    else
+                        Sc.kind = PK_TREE2;
+                    break;
                 case W_F0_PAIR:
                     src = GS_PAIR2;
                     if (regs) Sc.kind = PK_GEN_PAIR2;
@@ -775,7 +783,7 @@ static size_t layout(vc_circuit *c, uintptr_t base, uintptr_t hbase)
             if (prod && c->cfg.pr_chunk == PR_CHUNK_LOG && c->cfg.pr_split == VC_SPLIT_WIDEST && n >= 14)
                 C = n >= 19 ? PR_CHUNK_WIDE : PR_CHUNK_LOG;
             const bool tab = needs_tables(L.kind) && ph != 1;  // waits for k_build23
-            const bool anyB = (tab && L.has_add) || src == GS_FIRST2;
+            const bool anyB = (tab && L.has_add) || src == GS_FIRST2 || src == GS_TREE2;
             const u64 *inV = (ph == 1) ? L.V : L.Vn;
             u32 r0 = 0, g = 0;
             bool tail = false;
@@ -1019,7 +1027,7 @@ bool plan_valid(const Plan &P)
         const GenWave &W = P.gw[k];
         if (W.circ >= nc || W.sci >= P.scis.size() || P.scis[W.sci].circ != W.circ) return false;
         // a thread's entries share one upper factor of the source's split table
-        if (W.src != GS_NONE && W.e && W.e + (W.src == GS_FIRST2) - (W.src == GS_FINAL2) > W.th) return false;
+        if (W.src != GS_NONE && W.e && W.e + (W.src == GS_FIRST2) - (W.src == GS_FINAL2 || W.src == GS_TREE2) > W.th) return false;
         if (W.nr > GN_CHUNK_LOG || W.e > (u32)GN_M || W.e > W.nr || W.nr - W.e > WV_LOG || (W.e && W.e < 2))
             return false;
         if ((W.flags & WF_TAIL) && (k + 1 >= P.gw.size() || P.gw[k + 1].nchunks != 1 || P.gw[k + 1].sci != W.sci ||

@@ -164,3 +164,21 @@ def test_f2sp_row_groups(v, h):
         assert ok and f2 == sum(int(t) * int(t) for t in a) % P
     finally:
         vc.vc_f2sp_destroy(s)
+
+
+# values in host memory: addition layers of a part of a warp, one and several
+# registers' runs, one and several chunks; against every other kind's layers
+@pytest.mark.parametrize("family,logn", [("f2", n) for n in (1, 2, 3, 7, 8, 9, 10, 12, 13, 14, 16)] +
+                         [("f0", 9), ("matmult", 4)])
+def test_host_values_addition_layers(family, logn):
+    w, k = circuits.by_name(family, logn)
+    x = elements(logn, 1 << w[-1])
+    h = vc.vc_circuit_create(w, k, host_values=True)
+    try:
+        tr = torch.empty(vc.vc_transcript_len(h), dtype=torch.int64, device="cuda")
+        vc.vc_prove(h, dev(x), 51, tr)
+        vc.vc_circuit_sync(h)
+        assert (to_np(tr) == oracle_prove(w, k, x, 51)).all()
+        assert vc.vc_verify(h, dev(x), 51, tr)
+    finally:
+        vc.vc_circuit_destroy(h)
