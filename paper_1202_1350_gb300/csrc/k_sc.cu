@@ -115,6 +115,14 @@ extern __shared__ __align__(16) unsigned char wv_dyn[];  // a WaveSmem
 __device__ __forceinline__ ulonglong2 ld_in(const ulonglong2 *p, bool ext) { return ext ? __ldg(p) : __ldcg(p); }
 __device__ __forceinline__ u64 ld_in(const u64 *p, bool ext) { return ext ? __ldg(p) : __ldcg(p); }
 
+// Four entries of a first wave's values, a whole sector in one load (p 32-byte
+// aligned: a layer's values are, and runs are multiples of four): half the load
+// instructions (F2 2^22 212 -> 210 us).
+__device__ __forceinline__ void ldg4(const u64 *p, u64 &a, u64 &b, u64 &c, u64 &d)
+{
+    asm("ld.global.nc.v4.b64 {%0, %1, %2, %3}, [%4];" : "=l"(a), "=l"(b), "=l"(c), "=l"(d) : "l"(p));
+}
+
 // Asynchronous copies to shared memory: 16 bytes through L2 (also what other
 // CTAs of this launch wrote), or 8 bytes through L1 (a first wave's input).
 __device__ __forceinline__ void cp16(void *dst, const void *src)
@@ -509,8 +517,9 @@ __device__ __forceinline__ void gen_regs_runs(const GenWave &W, u64 x0, u32 e, b
 #pragma unroll 1
     for (u32 sub = 0; sub < nruns; sub++) {
         if (src == GS_PAIR2 || src == GS_FINAL2) {
-            const ulonglong2 *sv = reinterpret_cast<const ulonglong2 *>(W.inV + x0 + 4 * sub);
-            const ulonglong2 va = __ldg(sv), vb = __ldg(sv + 1);
+            u64 w4[4];
+            ldg4(W.inV + x0 + 4 * sub, w4[0], w4[1], w4[2], w4[3]);
+            const ulonglong2 va = make_ulonglong2(w4[0], w4[1]), vb = make_ulonglong2(w4[2], w4[3]);
             const ulonglong2 *sl = reinterpret_cast<const ulonglong2 *>(lo) + (src == GS_PAIR2 ? 2 * sub : sub);
             ulonglong2 l = __ldg(sl);
             if (src == GS_PAIR2) {
@@ -525,9 +534,7 @@ __device__ __forceinline__ void gen_regs_runs(const GenWave &W, u64 x0, u32 e, b
             if (src == GS_NONE) {
                 gen_load<4>(W, x0 + 4 * sub, hasB, p, v, b);
             } else {
-                const ulonglong2 *sv = reinterpret_cast<const ulonglong2 *>(W.inV + x0 + 4 * sub);
-                const ulonglong2 va = __ldg(sv), vb = __ldg(sv + 1);
-                v[0] = va.x, v[1] = va.y, v[2] = vb.x, v[3] = vb.y;
+                ldg4(W.inV + x0 + 4 * sub, v[0], v[1], v[2], v[3]);
                 const ulonglong2 *sl = reinterpret_cast<const ulonglong2 *>(lo) + (src == GS_FIRST2 ? 4 * sub : half ? sub : 2 * sub);
                 if (src == GS_FIRST2) {
 #pragma unroll
@@ -745,7 +752,6 @@ __device__ __forceinline__ void line_run8(const u64 *v, const u64 *la, const u64
 // sm.part[0..e][tid].
 __device__ __forceinline__ void line_regs(const u64 *entries, u32 e, LineSmem &sm)
 {
-    const ulonglong2 *src = reinterpret_cast<const ulonglong2 *>(entries);
     const u32 tid = threadIdx.x, nruns = 1u << (e - 3);
     u64 la[3], lb[3];
 #pragma unroll
@@ -761,14 +767,10 @@ __device__ __forceinline__ void line_regs(const u64 *entries, u32 e, LineSmem &s
     };
 #pragma unroll 1
     for (u32 run = 0; run < nruns; run++) {
-        if (!(run & 1) && run + 2 < nruns) prefetch_l1(src + 4 * (run + 2));  // the next line
+        if (!(run & 1) && run + 2 < nruns) prefetch_l1(entries + 8 * (run + 2));  // the next line
         u64 v[8];
-#pragma unroll
-        for (int t = 0; t < 4; t++) {
-            const ulonglong2 w = __ldg(src + 4 * run + t);
-            v[2 * t] = w.x;
-            v[2 * t + 1] = w.y;
-        }
+        ldg4(entries + 8 * run, v[0], v[1], v[2], v[3]);
+        ldg4(entries + 8 * run + 4, v[4], v[5], v[6], v[7]);
         u64 c[4];
         line_run8(v, la, lb, c);
         if (nruns == 1) store(dst, c);
