@@ -129,6 +129,13 @@ __device__ __forceinline__ void cp16(void *dst, const void *src)
 {
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((u32)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
 }
+// The same through L1, for values in host memory: copies that bypass it took
+// every sector across the link twice (F2 2^20: 4.19 M sectors read by the wave
+// launch, 2.91 M needed; 915 us a proof, so 740).
+__device__ __forceinline__ void cp16_l1(void *dst, const void *src)
+{
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"((u32)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
+}
 __device__ __forceinline__ void cp8(void *dst, const void *src)
 {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"((u32)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
@@ -227,6 +234,10 @@ __device__ __noinline__ int prod_chunk(const ProdWave &W, u32 chunk, u32 *ctr)
                     cp8(&dst[q * WV_NT].x, &src[32 * q].y);
                     cp8(&dst[q * WV_NT].y, &src[32 * q + 1].y);
                 }
+            } else if (W.flags & WF_HOST) {
+                src += row * 64 + c;
+#pragma unroll
+                for (int q = 0; q < 4; q++) cp16_l1(&dst[q * WV_NT], &src[16 * q]);
             } else {
                 src += row * 64 + c;
 #pragma unroll

@@ -83,8 +83,9 @@ __device__ __forceinline__ void gate_wiring(const LayerDev &L, u64 g, u64 &a, u6
 
 // Flags of a sum-check wave.  WF_TAIL: the next descriptor (a single chunk)
 // is run by the CTA that finishes this wave's last chunk.
-// WF_ODD: a PROD wave over the odd entries of its input table.
-enum : u32 { WF_HASB = 2, WF_LAST = 4, WF_TAIL = 8, WF_ODD = 16 };
+// WF_ODD: a PROD wave over the odd entries of its input table; WF_HOST: over
+// values in host memory.
+enum : u32 { WF_HASB = 2, WF_LAST = 4, WF_TAIL = 8, WF_ODD = 16, WF_HOST = 32 };
 
 // Kinds of sum-check instance (SCI).  Product-weighted ones (< PK_GEN_FIRST)
 // keep P = sigma prod_m L_m(x_m) implicit; general ones fold P, V, B tables.

@@ -830,7 +830,8 @@ static size_t layout(vc_circuit *c, uintptr_t base, uintptr_t hbase)
                     W.kc = std::min(nr, (u32)PR_C);
                     W.kr = nr - W.kc;
                     W.nchunks = nchunks;
-                    W.flags = (last ? WF_LAST : 0) | (has_tail ? WF_TAIL : 0) | (ph == 4 && w == 0 ? WF_ODD : 0);
+                    W.flags = (last ? WF_LAST : 0) | (has_tail ? WF_TAIL : 0) | (ph == 4 && w == 0 ? WF_ODD : 0) |
+                              (host && w == 0 ? WF_HOST : 0);
                     W.no = n - r0 - nr;
                     W.ho = (W.no + 1) / 2;
                     W.in = inV;
