@@ -118,46 +118,40 @@ def algorithmic_work(widths, kinds):
     return mul, byts
 
 
-def executed_work(widths, kinds, first_wave_log=12):
-    """Field multiplications the wave launch actually performs on circuits of
-    SQUARE and TREE layers (products of W values, 64-bit or in 31-bit limbs):
+def executed_work(widths, kinds, line_log=13):
+    """Field multiplications (exact 64-bit multiply-adds) the wave launch
+    performs on circuits of SQUARE and TREE layers, per entry of first chunks:
       * product-weighted instance over n variables (phase 1 of every layer,
-        phase 3 of SQUARE and TREE layers; P stays implicit): per pair of
-        entries of every round h(0), h(1) and the fold of V: 3 (2^n - 1);
-      * general instance (phase 2): per pair P V at t = 0, 1, 2 and the folds
-        of P and V (and B for TREE): 5 (6) per pair; SQUARE forms P = eq V at
-        2 per entry; TREE with a first wave in registers (n > 7) does its
-        round 0 at 5 per pair (eq(r_P, g), w (v0 + v1), w (3 v1 - v0), the V
-        fold and B = w v1), smaller TREE instances form P and B at 2 per gate;
-      * line reduction over n = s_{i+1} coordinates: folding coordinate j turns
-        pairs of degree-j polynomials into one of degree j + 1 at 2 (j + 1)
-        multiplications: sum_j 2^(n-j-1) 2 (j + 1)."""
+        phase 3, and phase 2 of TREE layers, whose second part runs over the
+        odd entries): two an entry, for the columns' and the rows' sums (the
+        rounds' own sums are over 2^7 values a chunk and not counted);
+      * general instance (phase 2 of SQUARE): P = eq V at one an entry, then
+        per pair P V at 0 and 1, the leading coefficient and two folds: 5;
+      * line reduction over n = s_{i+1} coordinates: folding coordinate j < e
+        in registers turns pairs of degree-j polynomials into one of degree
+        j + 1 at 2 (j + 1), sum_j 2^(n-j-1) 2 (j + 1); the threads' polynomials
+        (e + 1 coefficients) times weight polynomials of 8: 8 (e + 1) a thread."""
     mul = 0
     for i, k in enumerate(kinds):
         si, sn = widths[i], widths[i + 1]
         assert k in (0, 1), "counted for SQUARE and TREE layers"
-        for ph, n in ((1, si), (2, sn), (3, sn)):
-            if n == 0:
-                continue
-            if ph == 2 and k == 0:
-                mul += 5 * ((1 << n) - 1) + 2 * (1 << n)
-            elif ph == 2 and min(n, first_wave_log) > 7:
-                mul += 5 * (1 << (n - 1)) + 6 * ((1 << (n - 1)) - 1)
-            elif ph == 2:
-                mul += 6 * ((1 << n) - 1) + (1 << n)
-            else:
-                mul += 3 * ((1 << n) - 1)
-        mul += sum((1 << (sn - j - 1)) * 2 * (j + 1) for j in range(sn))
+        mul += 2 * (1 << si) + 2 * (1 << sn)
+        if k == 0:
+            mul += (1 << sn) + 5 * ((1 << sn) - 1)
+        else:
+            mul += 2 * (1 << sn) + 2 * (1 << (sn - 1))
+        e = max(3, min(line_log, sn) - 7) if sn > 7 else 0
+        mul += sum((1 << (sn - j - 1)) * 2 * (j + 1) for j in range(e)) + (1 << (sn - e)) * 8 * (e + 1)
     return mul
 
 
 # DRAM bytes (read + write) of one k_waves launch on this workload, from an ncu
 # capture of the current kernel; the V tables are mostly served from L2, so
 # this is below the algorithmic bytes
-K_WAVES_DRAM_BYTES = 25_572_096
+K_WAVES_DRAM_BYTES = 25_881_856
 # The same launch's integer pipes (ncu, % of peak sustained while active):
-# the multiply pipe (fmaheavy) cycles, ALU instructions, issue slots
-K_WAVES_PIPES = {"fmaheavy_cycles_pct": 52.4, "alu_inst_pct": 49.9, "issue_active_pct": 48.7}
+# the multiply pipe (fmaheavy) cycles, ALU pipe cycles, issue slots
+K_WAVES_PIPES = {"fmaheavy_cycles_pct": 56.8, "alu_cycles_pct": 35.9, "issue_active_pct": 43.6}
 # ncu: the pair-step microbenchmark keeps the multiply pipe (fmaheavy) busy
 # this fraction of its cycles (83-86 % over its configurations), so the pipe
 # saturated would give its rate / this fraction
@@ -882,7 +876,7 @@ def run_ours(args):
                      "achieved": achieved / 1e12, "peak": rate / 1e12, "unit": "Tmulmod/s",
                      "frac": achieved / rate, "traffic": K_WAVES_DRAM_BYTES,
                      "traffic_unit": "bytes per launch (ncu dram__bytes_read.sum + dram__bytes_write.sum)",
-                     "peak_source": "measured on this GPU: vc_field_mul_rate variant 2, the kernel's own "
+                     "peak_source": "measured on this GPU: vc_field_mul_rate variant 2, a sum-check "
                                     "pair step (2 exact multiply-adds + 1 lazy fold), best of 5 chain-count and "
                                     "register-budget configurations on a one-wave grid; ncu shows that step keeps "
                                     "the integer-multiply (fmaheavy) pipe 83-86 % of its cycles busy "
