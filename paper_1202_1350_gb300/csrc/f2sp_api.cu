@@ -303,10 +303,12 @@ extern "C" vc_status vc_f2sp_prove(vc_f2sp *s, const uint64_t *a, uint64_t *proo
     vc_status err;
     const u64 *da = sp_device_input(s, a, s->v * s->h, st, &err);
     if (!da) return err;
-    // a proof buffer on the device is written in place
-    launch_sp_prove(da, s->v, s->F, s->part, s->nparts, kp ? proof : s->proof, s->status, st);
+    // a proof buffer on the device is written in place where its words are
+    // aligned; any other takes a copy (which has no alignment rule)
+    const bool direct = kp && reinterpret_cast<uintptr_t>(proof) % sizeof(u64) == 0;
+    launch_sp_prove(da, s->v, s->F, s->part, s->nparts, direct ? proof : s->proof, s->status, st);
     cudaError_t e = cudaGetLastError();
-    if (e == cudaSuccess && !kp)
+    if (e == cudaSuccess && !direct)
         e = cudaMemcpyAsync(proof, s->proof, 2 * s->h * sizeof(u64), cudaMemcpyDefault, st);
     if (e != cudaSuccess) return cuda_status(e);
     return sp_status(s, st);
