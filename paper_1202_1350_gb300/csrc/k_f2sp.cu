@@ -66,8 +66,13 @@ struct SpFft {
 // Values between passes are below 3 2^61 (lazy sums of two W values, or a
 // difference plus 2 p): the next pass's sums and differences, below 2^64, are
 // brought back to W.
+// Lines of more than 13 values may be shared by T lanes of a warp (adjacent
+// ones, `mask`; this one is lane t of them): each holds all the sums, then all
+// the differences, and takes every T-th output pair.  Few rows leave few lines,
+// and one of 61 values is 3,600 products one after another.
 template <int Q, bool INV, bool TW>
-__device__ __forceinline__ void sp_line(u64 *p, u32 st, const ulonglong2 *cs, const u64 *__restrict__ tw)
+__device__ __forceinline__ void sp_line(u64 *p, u32 st, const ulonglong2 *cs, const u64 *__restrict__ tw, u32 T,
+                                        u32 t, u32 mask)
 {
     constexpr int N = (Q - 1) / 2;
     const u64 x0 = p[0];
@@ -101,18 +106,23 @@ __device__ __forceinline__ void sp_line(u64 *p, u32 st, const ulonglong2 *cs, co
             put(INV ? k : Q - k, C + (2 * FP_P) - S);
         }
     } else {
-        u64 t = wred(x0);
+        u64 sum = wred(x0);
 #pragma unroll
         for (int j = 0; j < N; j++) {
             const u64 a = p[(j + 1) * st], b = p[(Q - 1 - j) * st];
             s[j] = wred(a + b);
-            p[(Q - 1 - j) * st] = wred(a + (4 * FP_P) - b);
-            t += s[j];
-            if ((j & 3) == 3) t = wred(t);
+            if (T == 1) p[(Q - 1 - j) * st] = wred(a + (4 * FP_P) - b);
+            sum += s[j];
+            if ((j & 3) == 3) sum = wred(sum);
         }
-        put(0, wred(t));
+        if (T > 1) {
+            __syncwarp(mask);  // every lane has its sums
 #pragma unroll 1
-        for (int k = 1; k <= N; k++) {
+            for (u32 k = t + 1; k <= N; k += T) p[(Q - k) * st] = wred(p[k * st] + (4 * FP_P) - p[(Q - k) * st]);
+        }
+        if (t == 0) put(0, wred(sum));
+#pragma unroll 1
+        for (u32 k = t + 1; k <= N; k += T) {
             acc128 c0, c1;  // N <= 30 products of W and canonical values: below 2^128
             c0.lo = x0;
             c0.hi = 0;
@@ -121,10 +131,12 @@ __device__ __forceinline__ void sp_line(u64 *p, u32 st, const ulonglong2 *cs, co
             for (int j = 0; j < N; j++) mac((j & 1) ? c1 : c0, s[j], cs[(k - 1) * N + j].x);
             p[k * st] = wred(acc_red(c0) + acc_red(c1));
         }
+        if (T > 1) __syncwarp(mask);  // the differences are there
 #pragma unroll
-        for (int j = 0; j < N; j++) s[j] = p[(Q - 1 - j) * st];  // the differences
+        for (int j = 0; j < N; j++) s[j] = p[(Q - 1 - j) * st];
+        if (T > 1) __syncwarp(mask);  // and read: their slots take outputs
 #pragma unroll 1
-        for (int k = 1; k <= N; k++) {
+        for (u32 k = t + 1; k <= N; k += T) {
             acc128 e0, e1;
             acc_zero(e0);
             acc_zero(e1);
@@ -142,23 +154,31 @@ __device__ __forceinline__ void sp_line(u64 *p, u32 st, const ulonglong2 *cs, co
 // through shared memory and a barrier in between).
 enum { SP_INV = 0, SP_FWD = 1, SP_MID = 2 };
 
-// One pass over `nrows` rows in buf: a thread per line.  Lines of all the rows
-// are numbered together (line J starts at (J / st) q st + J mod st).
+// One pass over `nrows` rows in buf: a thread per line, or T where the lines of
+// more than 13 values are at most 1/T of the CTA's threads (100 rows of 61, one
+// line a CTA: 31 us, 103 with a thread a line, 39 with a thread a value; 152 of
+// 2501 = 41 61: 79, 141 and 122).  Lines of all the rows are numbered together (line J starts at
+// (J / st) q st + J mod st).
 template <int Q, int KIND, int NT>
 __device__ __forceinline__ void sp_pass_q(u64 *buf, u32 nrows, const SpFft &F, u32 d, const ulonglong2 *cs)
 {
     const u32 st = F.st[d], n = nrows * (F.h / Q);
     const ulonglong2 *w = cs + F.cso[d];
-    for (u32 J = threadIdx.x; J < n; J += NT) {
+    u32 T = 1;
+    if (Q > 13)
+        while (T < 32 && 2 * T * n <= NT) T *= 2;
+    const u32 t = threadIdx.x & (T - 1), mask = (T == 32 ? ~0u : (1u << T) - 1) << (threadIdx.x & 31 & ~(T - 1));
+    for (u32 J = threadIdx.x / T; J < n; J += NT / T) {
         const u32 o = st == 1 ? J : __umulhi(J, F.magic[d]), in = J - o * st;
         u64 *p = buf + o * Q * st + in;
         if (KIND == SP_MID) {  // outermost digit: o is the row, `in` the line's first slot
-            sp_line<Q, true, true>(p, st, w, F.twist + in);
-            sp_line<Q, false, false>(p, st, w, nullptr);
+            sp_line<Q, true, true>(p, st, w, F.twist + in, T, t, mask);
+            if (T > 1) __syncwarp(mask);
+            sp_line<Q, false, false>(p, st, w, nullptr, T, t, mask);
         } else if (KIND == SP_INV) {
-            sp_line<Q, true, false>(p, st, w, nullptr);
+            sp_line<Q, true, false>(p, st, w, nullptr, T, t, mask);
         } else {
-            sp_line<Q, false, false>(p, st, w, nullptr);
+            sp_line<Q, false, false>(p, st, w, nullptr, T, t, mask);
         }
     }
 }

@@ -48,3 +48,62 @@ def test_f2sp_proof_at_any_byte(offset):
     got = buf.cpu().numpy()
     assert (got[offset:offset + 16 * h].view(np.uint64) == want).all()
     assert (got[:offset] == 0x5A).all() and (got[offset + 16 * h:] == 0x5A).all()
+
+
+# lines of 25, 31, 41 and 61 values on 32 lanes, then on 16, 8, 4, 2 and one
+@pytest.mark.parametrize("v,h", [(3, 25), (3, 31), (3, 41), (100, 61), (3040, 61), (6080, 61), (2000, 155), (30400, 61),
+                                 (17176, 123)])
+def test_f2sp_shared_lines(v, h):
+    a = elements(v + h, v * h)
+    s = vc.vc_f2sp_create(v, h)
+    try:
+        out = torch.empty(2 * h, dtype=torch.int64, device="cuda")
+        vc.vc_f2sp_prove(s, dev(a), out)
+    finally:
+        vc.vc_f2sp_destroy(s)
+    assert (out.cpu().numpy().view(np.uint64) == oracle.f2sp_prove(a, v, h)).all()
+
+
+# two and three large factors in one row length: the even points in closed form,
+# and the polynomial through all of them at the verifier's secret points
+@pytest.mark.parametrize("v,h", [(2, 775), (304, 775), (152, 2501), (2, 4575), (3, 6355)])
+def test_f2sp_two_large_factors(v, h):
+    a = elements(v + h, v * h)
+    s = vc.vc_f2sp_create(v, h)
+    try:
+        da, out = dev(a), torch.empty(2 * h, dtype=torch.int64, device="cuda")
+        vc.vc_f2sp_prove(s, da, out)
+        even = out.cpu().numpy().view(np.uint64)[::2]
+        want = (a.astype(object).reshape(v, h) ** 2).sum(axis=0) % P
+        assert [int(t) for t in even] == [int(t) for t in want]
+        for seed in (1, 2):
+            vc.vc_f2sp_verify_begin(s, seed)
+            vc.vc_f2sp_verify_absorb(s, da, 0, v)
+            assert vc.vc_f2sp_verify_end(s, out) == (True, int(want.sum()) % P)
+    finally:
+        vc.vc_f2sp_destroy(s)
+
+
+def prove_us(v, h):
+    """Device time of a special-purpose proof, the least of twenty."""
+    a = dev(elements(1, v * h))
+    out = torch.empty(2 * h, dtype=torch.int64, device="cuda")
+    s = vc.vc_f2sp_create(v, h)
+    try:
+        best = float("inf")
+        for _ in range(20):
+            b, e = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            b.record()
+            vc.vc_f2sp_prove(s, a, out)
+            e.record()
+            e.synchronize()
+            best = min(best, b.elapsed_time(e) * 1e3)
+        return best
+    finally:
+        vc.vc_f2sp_destroy(s)
+
+
+def test_f2sp_few_rows_of_a_large_factor():
+    """One row of 61 a CTA takes about as long as one of 91 = 7 13 (a line of 61
+    in one thread took 3.5 times as long, and twice a thread per value's)."""
+    assert prove_us(100, 61) < 2 * prove_us(100, 91)
