@@ -88,6 +88,7 @@ struct GenSmem {
     u64 lvl[3];
     u64 w[WV_NT / 32][16];  // per-warp sums of the in-register rounds
     u64 hs[9][WV_NT];       // per-thread sums of in-register rounds 2..4 (kept out of registers)
+    u64 pend[9][WV_NT];     // triples waiting for their partner in rounds 2..4
     u64 x[3][WV_NT];        // the threads' folded triples
     u64 c[3][WV_NT + 4];    // cross rounds' pair terms: round kk's at 2 (64 - (64 >> kk)) ..
 };
@@ -442,28 +443,31 @@ __device__ __forceinline__ bool source_b(u32 src) { return src == GS_FIRST2 || s
 
 // P (and B, for FIRST2 and TREE2) of one entry x of a first wave whose tables
 // follow from the wiring (GS_*); v = V[x], vn = V[x with bit 0 cleared] (PAIR2)
-// or set (TREE2) (.x: P, .y: B).
-__device__ __noinline__ ulonglong2 gen_source(const Globals &G, const GenWave &W, u64 x, u64 v, u64 vn)
+// or set (TREE2) (.x: P, .y: B).  The factors come from the wave's own split
+// table, whose pointers are there with the descriptor: through the layer's
+// they were two more loads, one after another.
+__device__ __noinline__ ulonglong2 gen_source(const GenWave &W, u64 x, u64 v, u64 vn)
 {
-    u64 p, b = 0;
-    if (W.src == GS_MM2) {
-        const u32 Lb = G.layers[W.layer].s / 3;
-        const u64 k = x & ((1ull << Lb) - 1), i = x >> Lb;
-        return make_ulonglong2((i >> Lb) ? 0 : wmul(__ldg(W.inP + k), __ldg(W.inB + i)), 0);
-    }
-    const EqTab &T = G.layers[W.layer].trp;
-    switch (W.src) {
-    case GS_SQ2: p = wmul(eq_at(T, x), v); break;
-    case GS_PAIR2: p = wmul(eq_at(T, x), vn); break;
-    case GS_FINAL2: p = (x & 1) ? wmul(eq_at(T, x >> 1), v) : 0; break;
+    const u32 src = W.src, th = W.th;
+    const bool half = src == GS_FINAL2 || src == GS_TREE2;
+    const u64 *lo = W.inP, *hi = W.inB;
+    const u64 t = half ? x >> 1 : src == GS_FIRST2 ? 2 * x : x;
+    const u64 i = t & ((1ull << th) - 1);
+    const u64 h = __ldg(hi + (t >> th));
+    u64 p = wmul(__ldg(lo + i), h), b = 0;
+    switch (src) {
+    case GS_MM2: break;  // (the table ends with n zeros: no weight past the first matrix)
+    case GS_SQ2: p = wmul(p, v); break;
+    case GS_PAIR2: p = wmul(p, vn); break;
+    case GS_FINAL2: p = (x & 1) ? wmul(p, v) : 0; break;
     case GS_TREE2:
-        p = (x & 1) ? 0 : eq_at(T, x >> 1);
+        p = (x & 1) ? 0 : p;
         b = wmul(p, vn);
         break;
     default: {  // GS_FIRST2
-        const u64 wa = eq_at(T, 2 * x + 1);
+        const u64 wa = wmul(__ldg(lo + i + 1), h);
         b = wmul(wa, v);
-        p = wred(wmul(eq_at(T, 2 * x), v) + wa);
+        p = wred(wmul(p, v) + wa);
         break;
     }
     }
@@ -522,7 +526,6 @@ __device__ __forceinline__ void gen_regs_runs(const GenWave &W, u64 x0, u32 e, b
             if (hasB) prefetch_l1(W.inB + x0 + 16);
         }
     }
-    u64 p0 = 0, v0 = 0, b0 = 0, p1 = 0, v1 = 0, b1 = 0, p2 = 0, v2 = 0, b2 = 0;  // pending: rounds 2, 3, 4
     u64 tp = 0, tv = 0, tb = 0;
     // a rolled loop keeps the kernel small (instruction-cache bound when unrolled)
 #pragma unroll 1
@@ -572,23 +575,19 @@ __device__ __forceinline__ void gen_regs_runs(const GenWave &W, u64 x0, u32 e, b
             else
                 gen_run<false>(p, v, b, sm, a, tp, tv, tb);
         }
-        if (!(sub & 1)) {  // wait for the partner run
-            p0 = tp, v0 = tv, b0 = tb;
-            continue;
+        // combined like a binary counter, the pending triples in shared memory
+        u32 lv = 0;
+#pragma unroll 1
+        for (; lv + 2 < e && ((sub >> lv) & 1); lv++) {
+            const u64 *q = &sm.pend[3 * lv][threadIdx.x];
+            gen_pair_acc(b_run, q[0], tp, q[WV_NT], tv, b_run ? q[2 * WV_NT] : 0, tb, sm.r[2 + lv], sm, lv, tp, tv, tb);
         }
-        gen_pair_acc(b_run, p0, tp, v0, tv, b0, tb, sm.r[2], sm, 0, tp, tv, tb);
-        if (nruns == 2) continue;
-        if (!(sub & 2)) {
-            p1 = tp, v1 = tv, b1 = tb;
-            continue;
+        if (lv + 2 < e) {
+            u64 *q = &sm.pend[3 * lv][threadIdx.x];
+            q[0] = tp;
+            q[WV_NT] = tv;
+            if (b_run) q[2 * WV_NT] = tb;
         }
-        gen_pair_acc(b_run, p1, tp, v1, tv, b1, tb, sm.r[3], sm, 1, tp, tv, tb);
-        if (nruns == 4) continue;
-        if (!(sub & 4)) {
-            p2 = tp, v2 = tv, b2 = tb;
-            continue;
-        }
-        gen_pair_acc(b_run, p2, tp, v2, tv, b2, tb, sm.r[4], sm, 2, tp, tv, tb);
     }
 #pragma unroll
     for (int j = 0; j < 6; j++) h[j] = acc_red(a[j]);
@@ -683,7 +682,7 @@ __device__ __noinline__ int gen_chunk(const Globals &G, const GenWave &W, u32 ch
             bv = hasB ? ld_in(W.inB + x, ext) : 0;
         } else {
             const u64 xn = W.src == GS_TREE2 ? x | 1 : W.src == GS_PAIR2 ? x & ~1ull : x;
-            const ulonglong2 t = gen_source(G, W, x, vv, xn != x ? ld_in(W.inV + xn, ext) : vv);
+            const ulonglong2 t = gen_source(W, x, vv, xn != x ? ld_in(W.inV + xn, ext) : vv);
             pv = t.x;
             bv = t.y;
         }
