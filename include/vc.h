@@ -332,9 +332,14 @@ vc_status vc_circuit_get_info(const vc_circuit *c, vc_circuit_info *info);
  * of fewer than 2^pr_split_log entries use chunks half as large (they are
  * dispatched after the larger ones, so finer chunks even out the end of the
  * persistent launch; 0 = never, VC_SPLIT_WIDEST = the circuit's widest
- * layer, else <= 40).  Any choice gives the same transcript; they only
- * change speed. */
+ * layer, else <= 40).  The three chunk sizes may be VC_TILE_BY_SIZE, the
+ * default of circuits created without tiles: each instance's chunk then
+ * follows its own size (product-weighted 13, from 19 coordinates 14, and
+ * VC_SPLIT_WIDEST halves none of 14 coordinates or more; general 10 to 12;
+ * line 12 to 15).  A number is used as it is.  Any choice gives the same
+ * transcript; they only change speed. */
 #define VC_SPLIT_WIDEST 0xFFFFFFFFu
+#define VC_TILE_BY_SIZE 0xFFFFFFFFu
 typedef struct {
     uint32_t pr_chunk_log;
     uint32_t gn_chunk_log;
@@ -369,7 +374,8 @@ vc_status vc_autotune_batch(const vc_circuit_desc *descs, int n, int device, int
 vc_status vc_circuit_create_tiles(const vc_circuit_desc *desc, int device, const vc_tile_config *tiles,
                                   vc_circuit **out);
 
-/* The tile shapes a circuit was planned with. */
+/* The tile shapes a circuit was planned with (VC_TILE_BY_SIZE where its chunks
+ * follow their instances' sizes). */
 vc_status vc_circuit_get_tiles(const vc_circuit *c, vc_tile_config *tiles);
 
 /* Batches (Sec. 6.2.3 runs many independent proofs; here they share launches).

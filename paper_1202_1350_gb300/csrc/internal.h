@@ -11,22 +11,23 @@
 
 constexpr u32 WV_LOG = 7;                  // log2 of the threads of a wave CTA
 constexpr u32 PR_CHUNK_LOG = 13;             // rounds of one PROD chunk, and
-constexpr u32 PR_CHUNK_WIDE = PR_C + PR_R;   // of one in a wide instance
+constexpr u32 PR_CHUNK_WIDE = PR_C + PR_R;   // of one in a wide instance (chunks by size only)
 constexpr u32 GN_CHUNK_LOG = GN_M + WV_LOG;  // rounds of one GEN chunk (2^GN_M entries per thread)
 constexpr u32 LN_CHUNK0_LOG = 6 + WV_LOG;    // coordinates of a first line-wave chunk (64 entries per thread)
 constexpr u32 LN_XTRA = 2;                   // more coordinates of a first line-wave chunk (256 entries per thread)
 constexpr u32 LN_CHUNKW_LOG = WV_LOG;        // coordinates of a later line-wave chunk (one polynomial per thread)
 
 // Tile shapes of a circuit's plan (the autotuner's knobs): rounds folded
-// by a first PROD / GEN chunk, coordinates folded by a first line-wave chunk,
-// the smallest evaluation chunk (log2 entries), and the size below which PROD
-// instances use half-size chunks.
+// by a first PROD / GEN chunk, coordinates folded by a first line-wave chunk
+// (VC_TILE_BY_SIZE: by the instance's size, the rules of pr_chunk_of,
+// gn_chunk_of and ln_chunk_of), the smallest evaluation chunk (log2 entries),
+// and the size below which PROD instances use half-size chunks.
 struct PlanConfig {
-    u32 pr_chunk = PR_CHUNK_LOG;
-    u32 gn_chunk = GN_CHUNK_LOG;
-    u32 ln_chunk0 = LN_CHUNK0_LOG;
+    u32 pr_chunk = VC_TILE_BY_SIZE;
+    u32 gn_chunk = VC_TILE_BY_SIZE;
+    u32 ln_chunk0 = VC_TILE_BY_SIZE;
     u32 ev_chunk = 11;  // evaluation chunk: 2^11 inputs per CTA
-    u32 pr_split = VC_SPLIT_WIDEST;  // PROD instances below 2^pr_split entries: chunks of 2^(pr_chunk - 1)
+    u32 pr_split = VC_SPLIT_WIDEST;  // PROD instances below 2^pr_split entries: chunks half as large
 };
 
 // Every device and page-locked host allocation of the library goes through

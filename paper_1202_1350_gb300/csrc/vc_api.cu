@@ -450,6 +450,44 @@ static cudaError_t staged_upload(vc_circuit *c)
     return e;
 }
 
+// Rounds of a first chunk of a product-weighted instance of n coordinates (the
+// circuit's widest layer: smax).  By size: 2^13, and 2^14 from 19 coordinates,
+// since about 7,000 cycles of a chunk do not depend on its size (F2 2^22 waves
+// 206 us with 2^12 and 2^13, 194 with 2^13, 182 with these; 2^14 from 17: 182,
+// but MATMULT 128 71 against 67).  Instances below the split, dispatched after
+// the larger ones, take half of it, which evens out the end of the launch; by
+// size, VC_SPLIT_WIDEST halves only what fits one chunk.
+static u32 pr_chunk_of(const PlanConfig &f, u32 n, u32 smax)
+{
+    const bool by_size = f.pr_chunk == VC_TILE_BY_SIZE, widest = f.pr_split == VC_SPLIT_WIDEST;
+    const u32 C = !by_size ? f.pr_chunk : n >= 19 ? PR_CHUNK_WIDE : PR_CHUNK_LOG;
+    if (by_size && widest && n > PR_CHUNK_LOG) return C;
+    return (n < (widest ? smax : f.pr_split) && C > 1) ? C - 1 : C;
+}
+
+// The same of a general instance.  By size few coordinates take smaller
+// chunks: a lone thread's 32 entries are a chain of about 2,700 cycles per 4
+// (F0 2^11 44.8 us with 2^12, F0 2^14 90 against 85 with 2^11; under load 2^12
+// wins: F0 2^16 199 against 222).
+static u32 gn_chunk_of(const PlanConfig &f, u32 n)
+{
+    if (f.gn_chunk != VC_TILE_BY_SIZE) return f.gn_chunk;
+    return n <= 12 ? 10u : n <= 15 ? 11u : GN_CHUNK_LOG;
+}
+
+// Coordinates of a first line chunk over n coordinates.  By size: 13; in
+// circuits of up to 2^16 entries a layer 12, whose chain is half as long (F2
+// 2^14 38.9 -> 33.1 us; in wider ones the load decides: F0 2^16 199 -> 216, F2
+// 2^20 91 -> 94); beyond 20 coordinates up to two more, so that the next wave
+// is the last (a third was a launch of its own).
+static u32 ln_chunk_of(const PlanConfig &f, u32 n, u32 smax)
+{
+    if (f.ln_chunk0 != VC_TILE_BY_SIZE) return f.ln_chunk0;
+    if (n >= LN_CHUNK0_LOG && smax <= 16) return LN_CHUNK0_LOG - 1;
+    if (n > LN_CHUNK0_LOG + LN_CHUNKW_LOG) return std::min(LN_CHUNK0_LOG + LN_XTRA, n - LN_CHUNKW_LOG);
+    return LN_CHUNK0_LOG;
+}
+
 // Lay out every buffer and descriptor relative to `base` (0 for sizing) and
 // fill the circuit's single-circuit plan (circ = 0).
 static size_t layout(vc_circuit *c, uintptr_t base, uintptr_t hbase)
@@ -593,15 +631,7 @@ static size_t layout(vc_circuit *c, uintptr_t base, uintptr_t hbase)
         const u64 *in = c->V[i + 1];
         bool tail = false;
         for (u32 w = 0;; w++) {
-            // first chunks of more than 20 coordinates take up to two more, so
-            // that the next wave is their last (a third was a launch of its own)
-            u32 cap = (w == 0) ? c->cfg.ln_chunk0 : LN_CHUNKW_LOG;
-            // circuits of up to 2^16 entries a layer: halves of the default chunk,
-            // whose chain is half as long (F2 2^14 38.9 -> 33.1 us; in wider ones the
-            // load decides: F0 2^16 199 -> 216, F2 2^20 91 -> 94)
-            if (w == 0 && cap == LN_CHUNK0_LOG && n >= LN_CHUNK0_LOG && line_smax <= 16) cap = LN_CHUNK0_LOG - 1;
-            if (w == 0 && cap == LN_CHUNK0_LOG && n > cap + LN_CHUNKW_LOG)
-                cap = std::min(LN_CHUNK0_LOG + LN_XTRA, n - LN_CHUNKW_LOG);
+            const u32 cap = (w == 0) ? ln_chunk_of(c->cfg, n, line_smax) : LN_CHUNKW_LOG;
             const u32 nl = std::min(cap, n - l0);
             LineWaveDev W{};
             W.circ = 0;
@@ -712,7 +742,7 @@ static size_t layout(vc_circuit *c, uintptr_t base, uintptr_t hbase)
             } else {
                 // F0 pair and final layers: the first wave's round 0 leaves a
                 // factor out of P if it runs in registers (applied by k_final)
-                const bool regs = std::min(c->cfg.gn_chunk, n) > WV_LOG;  // (a smaller default chunk is above WV_LOG too)
+                const bool regs = std::min(gn_chunk_of(c->cfg, n), n) > WV_LOG;
                 Sc.kind = PK_GEN_EZ;
                 switch (L.kind) {
                 case W_SQUARE: src = GS_SQ2; break;
@@ -764,24 +794,7 @@ static size_t layout(vc_circuit *c, uintptr_t base, uintptr_t hbase)
             }
             P.scis.push_back(Sc);
             const u32 nv = prod ? 2 : 3;
-            // smaller PROD instances (dispatched after the larger ones) use
-            // half-size chunks, which evens out the end of the launch
-            const u32 split = (c->cfg.pr_split == VC_SPLIT_WIDEST) ? smax : c->cfg.pr_split;
-            u32 C = prod ? ((n < split && c->cfg.pr_chunk > 1) ? c->cfg.pr_chunk - 1 : c->cfg.pr_chunk)
-                         : c->cfg.gn_chunk;
-            // With the default shapes general instances of few coordinates take
-            // smaller chunks: a lone thread's 32 entries are a chain of about
-            // 2,700 cycles per 4 (F0 2^11 44.8 us with 2^12, F0 2^14 90 against 85
-            // with 2^11; under load 2^12 wins: F0 2^16 199 against 222).
-            const u32 gsmall = n <= 12 ? 10u : n <= 15 ? 11u : GN_CHUNK_LOG;
-            if (!prod && c->cfg.gn_chunk == GN_CHUNK_LOG) C = gsmall;
-            // with the default shapes wide PROD instances take larger chunks
-            // (about 7,000 cycles of a chunk do not depend on its size): 2^13
-            // from 14 coordinates, 2^14 from 19.  F2 2^22 waves 206 us with 2^12
-            // and 2^13, 194 with 2^13, 182 with these (2^14 from 17: 182, but
-            // MATMULT 128 71 against 67).
-            if (prod && c->cfg.pr_chunk == PR_CHUNK_LOG && c->cfg.pr_split == VC_SPLIT_WIDEST && n >= 14)
-                C = n >= 19 ? PR_CHUNK_WIDE : PR_CHUNK_LOG;
+            const u32 C = prod ? pr_chunk_of(c->cfg, n, smax) : gn_chunk_of(c->cfg, n);
             const bool tab = needs_tables(L.kind) && ph != 1;  // waits for k_build23
             const bool anyB = (tab && L.has_add) || src == GS_FIRST2 || src == GS_TREE2;
             const u64 *inV = (ph == 1) ? L.V : L.Vn;
@@ -1672,8 +1685,9 @@ static std::map<std::vector<u32>, PlanConfig> g_tuned;  // size class -> fastest
 
 static bool config_ok(const PlanConfig &f)
 {
-    return f.pr_chunk >= 1 && f.pr_chunk <= PR_CHUNK_LOG && f.gn_chunk >= 1 && f.gn_chunk <= GN_CHUNK_LOG &&
-           f.ln_chunk0 >= 1 && f.ln_chunk0 <= LN_CHUNK0_LOG && f.ev_chunk >= 1 && f.ev_chunk <= 11 &&
+    auto chunk_ok = [](u32 c, u32 max) { return (c >= 1 && c <= max) || c == VC_TILE_BY_SIZE; };
+    return chunk_ok(f.pr_chunk, PR_CHUNK_LOG) && chunk_ok(f.gn_chunk, GN_CHUNK_LOG) &&
+           chunk_ok(f.ln_chunk0, LN_CHUNK0_LOG) && f.ev_chunk >= 1 && f.ev_chunk <= 11 &&
            (f.pr_split <= 40 || f.pr_split == VC_SPLIT_WIDEST);
 }
 
@@ -2517,9 +2531,10 @@ extern "C" vc_status vc_autotune(const vc_circuit_desc *desc, int device, int re
     // below half of its size, never)
     u32 smax = 0;
     for (u32 i = 0; i <= desc->n_layers; i++) smax = std::max(smax, desc->log_width[i]);
-    const u32 cand[5][4] = {{11, 12, 13, 0}, {10, 11, 12, 0}, {11, 12, 13, 0}, {8, 9, 10, 11},
+    const u32 by = VC_TILE_BY_SIZE;
+    const u32 cand[5][4] = {{by, 11, 12, 13}, {by, 10, 11, 12}, {by, 11, 12, 13}, {8, 9, 10, 11},
                             {VC_SPLIT_WIDEST, smax ? smax - 1 : 0, 0, VC_SPLIT_WIDEST}};
-    const int ncand[5] = {3, 3, 3, 4, 3};
+    const int ncand[5] = {4, 4, 4, 4, 3};
     for (int knob = 0; knob < 5 && s == VC_OK; knob++)
         for (int j = 0; j < ncand[knob]; j++) {
             PlanConfig f = cur;
@@ -2635,9 +2650,10 @@ extern "C" vc_status vc_autotune_batch(const vc_circuit_desc *descs, int n, int 
     // coordinate descent over the knobs, one configuration for every member,
     // timed on the merged batch itself (the split threshold below the widest
     // layer of the batch, below 2^13 and 2^11, or never)
-    const u32 cand[5][4] = {{11, 12, 13, 0}, {10, 11, 12, 0}, {11, 12, 13, 0}, {8, 9, 10, 11},
+    const u32 by = VC_TILE_BY_SIZE;
+    const u32 cand[5][4] = {{by, 11, 12, 13}, {by, 10, 11, 12}, {by, 11, 12, 13}, {8, 9, 10, 11},
                             {VC_SPLIT_WIDEST, 13, 11, smax ? smax - 1 : 0}};
-    const int ncand[5] = {3, 3, 3, 4, 4};
+    const int ncand[5] = {4, 4, 4, 4, 4};
     for (int pass = 0; pass < 2 && s == VC_OK; pass++) {
         bool moved = false;
         for (int knob = 0; knob < 5 && s == VC_OK; knob++)

@@ -81,6 +81,7 @@ class ServerStats(ctypes.Structure):
 
 
 VC_SPLIT_WIDEST = 0xFFFFFFFF
+VC_TILE_BY_SIZE = 0xFFFFFFFF  # a chunk size: by each instance's size (the default)
 
 
 class TileConfig(ctypes.Structure):
@@ -681,6 +682,8 @@ def vc_autotune_batch(shapes, device: int = 0, reps: int = 3):
 
 
 def vc_circuit_create_tiles(log_width, wiring, tiles: dict, device: int = 0):
+    """A circuit with explicit tile shapes; each chunk size a number, used as it
+    is, or VC_TILE_BY_SIZE."""
     desc, keep = _desc_struct(log_width, wiring)
     t = TileConfig(tiles["pr_chunk_log"], tiles["gn_chunk_log"], tiles["line_chunk_log"], tiles["eval_chunk_log"],
                    tiles.get("pr_split_log", VC_SPLIT_WIDEST))

@@ -5,8 +5,8 @@ import numpy as np
 import pytest
 
 import oracle
-from gpu_util import ensure_built
-from paper_1202_1350_gb300 import vc
+from gpu_util import ensure_built, oracle_prove, to_np
+from paper_1202_1350_gb300 import SQUARE, circuits, vc
 
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
@@ -107,3 +107,80 @@ def test_f2sp_few_rows_of_a_large_factor():
     """One row of 61 a CTA takes about as long as one of 91 = 7 13 (a line of 61
     in one thread took 3.5 times as long, and twice a thread per value's)."""
     assert prove_us(100, 61) < 2 * prove_us(100, 91)
+
+
+W, BY_SIZE = vc.VC_SPLIT_WIDEST, vc.VC_TILE_BY_SIZE
+
+
+def tiles_of(pr, gn, ln, ev, split):
+    return {"pr_chunk_log": pr, "gn_chunk_log": gn, "line_chunk_log": ln, "eval_chunk_log": ev, "pr_split_log": split}
+
+
+def first_chunks(widths, kinds, pr, gn, ln, split):
+    """Chunks of every instance's and line's first wave (SQUARE and TREE
+    layers), by the documented meaning of the tile shapes."""
+    widest = max(widths)
+    split = widest if split == W else split
+
+    def chunks(n, c):
+        return 1 << (n - min(n, c)) if n > 0 else 0
+
+    total = 0
+    for i, kind in enumerate(kinds):
+        si, sn = widths[i], widths[i + 1]
+        prod = [si, sn] if kind == SQUARE else [si, sn, sn - 1, sn]
+        total += sum(chunks(n, pr - 1 if n < split and pr > 1 else pr) for n in prod)
+        total += chunks(sn, gn) if kind == SQUARE else 0
+        total += 1 << (sn - min(sn, ln))
+    return total
+
+
+# numbers at the top of their range, below it, and with each kind of split
+@pytest.mark.parametrize("shape", [(13, 12, 13, 11, W), (13, 12, 13, 11, 0), (13, 12, 13, 11, 15), (12, 11, 12, 11, W),
+                                   (13, 10, 9, 10, 14), (1, 7, 7, 11, W)])
+@pytest.mark.parametrize("logn", [12, 15, 17, 21])
+def test_explicit_tiles_are_used_as_they_are(shape, logn):
+    w, k = circuits.f2(logn)
+    pr, gn, ln, ev, split = shape
+    h = vc.vc_circuit_create_tiles(w, k, tiles_of(*shape))
+    try:
+        assert vc.vc_circuit_get_tiles(h) == tiles_of(*shape)
+        assert vc.vc_circuit_get_info(h)["wave_tasks"] == first_chunks(w, k, pr, gn, ln, split)
+    finally:
+        vc.vc_circuit_destroy(h)
+
+
+@pytest.mark.parametrize("logn", [12, 20])
+def test_default_tiles_are_named_by_size(logn):
+    """What a circuit without tiles reports is what it was planned with: the
+    same shapes again give the same plan, and a numeric split leaves the sizes
+    of wider instances' chunks alone."""
+    w, k = circuits.f2(logn)
+    hs = [vc.vc_circuit_create(w, k)]
+    try:
+        t = vc.vc_circuit_get_tiles(hs[0])
+        assert t == tiles_of(BY_SIZE, BY_SIZE, BY_SIZE, 11, W)
+        hs.append(vc.vc_circuit_create_tiles(w, k, t))
+        hs.append(vc.vc_circuit_create_tiles(w, k, dict(t, pr_split_log=0)))
+        tasks = [vc.vc_circuit_get_info(h)["wave_tasks"] for h in hs]
+        assert tasks[0] == tasks[1] and tasks[2] <= tasks[0]
+    finally:
+        for h in hs:
+            vc.vc_circuit_destroy(h)
+
+
+# explicit shapes whose general first waves form their tables with one entry, 4
+# and 32 entries a thread, from split tables with several upper factors
+@pytest.mark.parametrize("family,logn", [("f0", 11), ("f2", 12), ("matmult", 6)])
+@pytest.mark.parametrize("gn", [7, 9, 12])
+def test_explicit_general_chunks(family, logn, gn):
+    w, k = circuits.by_name(family, logn)
+    x = elements(gn, 1 << w[-1])
+    h = vc.vc_circuit_create_tiles(w, k, tiles_of(13, gn, 13, 11, W))
+    try:
+        tr = torch.empty(vc.vc_transcript_len(h), dtype=torch.int64, device="cuda")
+        vc.vc_prove(h, dev(x), 61, tr)
+        vc.vc_circuit_sync(h)
+        assert (to_np(tr) == oracle_prove(w, k, x, 61)).all()
+    finally:
+        vc.vc_circuit_destroy(h)
