@@ -465,13 +465,19 @@ static u32 pr_chunk_of(const PlanConfig &f, u32 n, u32 smax)
     return (n < (widest ? smax : f.pr_split) && C > 1) ? C - 1 : C;
 }
 
-// The same of a general instance.  By size few coordinates take smaller
-// chunks: a lone thread's 32 entries are a chain of about 2,700 cycles per 4
-// (F0 2^11 44.8 us with 2^12, F0 2^14 90 against 85 with 2^11; under load 2^12
-// wins: F0 2^16 199 against 222).
-static u32 gn_chunk_of(const PlanConfig &f, u32 n)
+// The same of a general instance, in a circuit whose general instances hold
+// `entries` in all.  By size few coordinates take smaller chunks: a lone
+// thread's 32 entries are a chain of about 2,700 cycles per 4 (F0 2^11 44.8 us
+// with 2^12, F0 2^14 90 against 85 with 2^11; under load 2^12 wins: F0 2^16 199
+// against 222).  11 coordinates, the least that do not fit one chunk of 2^10,
+// take 2^8 where the circuit has at most 2^12 such entries, so that the launch
+// is short of work anyway and only rounds 0 and 1 run in registers (F2 2^11
+// 26.7 -> 24.7 us, 43.0 -> 37.1 with the L2 flushed, MATMULT 32 52.7 -> 48.7;
+// at 12 as well, 576 merged circuits lose 0.6 %, so 0.2 %).
+static u32 gn_chunk_of(const PlanConfig &f, u32 n, u64 entries)
 {
     if (f.gn_chunk != VC_TILE_BY_SIZE) return f.gn_chunk;
+    if (n == 11 && entries <= (u64(1) << 12)) return 8;
     return n <= 12 ? 10u : n <= 15 ? 11u : GN_CHUNK_LOG;
 }
 
@@ -701,6 +707,9 @@ static size_t layout(vc_circuit *c, uintptr_t base, uintptr_t hbase)
     u64 part_total = 0;
     u32 smax = 0;
     for (u32 i = 0; i <= d; i++) smax = std::max(smax, c->s[i]);
+    u64 gen_entries = 0;  // of the circuit's general instances
+    for (u32 i = 0; i < d; i++)
+        if (c->kind[i] != W_TREE || host) gen_entries += (c->kind[i] == W_EXPLICIT ? 2 : 1) * S(i + 1);
     for (u32 i = 0; i < d; i++) {
         const LayerDev &L = c->L[i];
         u64 tree2_rounds = 0;  // index of phase 2's first round
@@ -742,7 +751,7 @@ static size_t layout(vc_circuit *c, uintptr_t base, uintptr_t hbase)
             } else {
                 // F0 pair and final layers: the first wave's round 0 leaves a
                 // factor out of P if it runs in registers (applied by k_final)
-                const bool regs = std::min(gn_chunk_of(c->cfg, n), n) > WV_LOG;
+                const bool regs = std::min(gn_chunk_of(c->cfg, n, gen_entries), n) > WV_LOG;
                 Sc.kind = PK_GEN_EZ;
                 switch (L.kind) {
                 case W_SQUARE: src = GS_SQ2; break;
@@ -794,7 +803,7 @@ static size_t layout(vc_circuit *c, uintptr_t base, uintptr_t hbase)
             }
             P.scis.push_back(Sc);
             const u32 nv = prod ? 2 : 3;
-            const u32 C = prod ? pr_chunk_of(c->cfg, n, smax) : gn_chunk_of(c->cfg, n);
+            const u32 C = prod ? pr_chunk_of(c->cfg, n, smax) : gn_chunk_of(c->cfg, n, gen_entries);
             const bool tab = needs_tables(L.kind) && ph != 1;  // waits for k_build23
             const bool anyB = (tab && L.has_add) || src == GS_FIRST2 || src == GS_TREE2;
             const u64 *inV = (ph == 1) ? L.V : L.Vn;

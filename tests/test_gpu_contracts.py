@@ -6,7 +6,7 @@ import pytest
 
 import oracle
 from gpu_util import ensure_built, oracle_prove, to_np
-from paper_1202_1350_gb300 import SQUARE, circuits, vc
+from paper_1202_1350_gb300 import SQUARE, TREE, circuits, vc
 
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
@@ -184,3 +184,18 @@ def test_explicit_general_chunks(family, logn, gn):
         assert (to_np(tr) == oracle_prove(w, k, x, 61)).all()
     finally:
         vc.vc_circuit_destroy(h)
+
+
+# a single general instance of 10 .. 13 coordinates, in a circuit and beside others
+@pytest.mark.parametrize("logn", [10, 11, 12, 13])
+def test_lone_general_instances(logn):
+    for w, k in (circuits.f2(logn), ([logn - 1, logn], [TREE]), ([logn, logn], [SQUARE]),
+                 ([logn] * 4, [SQUARE] * 3)):
+        x = elements(logn, 1 << w[-1])
+        h = vc.vc_circuit_create(w, k)
+        try:
+            tr = torch.empty(vc.vc_transcript_len(h), dtype=torch.int64, device="cuda")
+            assert vc.vc_prove_verify(h, dev(x), 71, tr)
+            assert (to_np(tr) == oracle_prove(w, k, x, 71)).all()
+        finally:
+            vc.vc_circuit_destroy(h)
