@@ -118,7 +118,19 @@ def algorithmic_work(widths, kinds):
     return mul, byts
 
 
-def executed_work(widths, kinds, line_log=13):
+def line_chunk_log(n, widest, tiles=None):
+    """Coordinates of the first line-reduction chunk over n coordinates in a
+    circuit whose widest layer has 2^widest entries: `tiles`' number, else
+    (the default) the library's choice by size."""
+    from paper_1202_1350_gb300 import vc
+    if tiles is not None and tiles["line_chunk_log"] != vc.VC_TILE_BY_SIZE:
+        return tiles["line_chunk_log"]
+    if n >= 13 and widest <= 16:
+        return 12
+    return min(15, n - 7) if n > 20 else 13
+
+
+def executed_work(widths, kinds, tiles=None):
     """Field multiplications (exact 64-bit multiply-adds) the wave launch
     performs on circuits of SQUARE and TREE layers, per entry of first chunks:
       * product-weighted instance over n variables (phase 1 of every layer,
@@ -130,7 +142,8 @@ def executed_work(widths, kinds, line_log=13):
       * line reduction over n = s_{i+1} coordinates: folding coordinate j < e
         in registers turns pairs of degree-j polynomials into one of degree
         j + 1 at 2 (j + 1), sum_j 2^(n-j-1) 2 (j + 1); the threads' polynomials
-        (e + 1 coefficients) times weight polynomials of 8: 8 (e + 1) a thread."""
+        (e + 1 coefficients) times weight polynomials of 8: 8 (e + 1) a thread.
+    `tiles`: the circuit's tile shapes (vc_circuit_get_tiles), None the default."""
     mul = 0
     for i, k in enumerate(kinds):
         si, sn = widths[i], widths[i + 1]
@@ -140,7 +153,8 @@ def executed_work(widths, kinds, line_log=13):
             mul += (1 << sn) + 5 * ((1 << sn) - 1)
         else:
             mul += 2 * (1 << sn) + 2 * (1 << (sn - 1))
-        e = max(3, min(line_log, sn) - 7) if sn > 7 else 0
+        chunk = min(line_chunk_log(sn, max(widths), tiles), sn)
+        e = max(3, chunk - 7) if chunk > 7 else 0
         mul += sum((1 << (sn - j - 1)) * 2 * (j + 1) for j in range(e)) + (1 << (sn - e)) * 8 * (e + 1)
     return mul
 
@@ -855,7 +869,7 @@ def run_ours(args):
     # which runs every sum-check round and line reduction of the F2 circuit
     wave_launch_ms = statistics.mean(wave_ms)
     mul, byts = algorithmic_work(widths, kinds)
-    executed = executed_work(widths, kinds, vc.vc_circuit_get_tiles(h)["gn_chunk_log"])
+    executed = executed_work(widths, kinds, vc.vc_circuit_get_tiles(h))
     rate = vc.vc_field_mul_rate(local, 2, 1 << 12)
     achieved = mul / (wave_launch_ms / 1000)
     stages = {name: round(statistics.mean(v), 4) for name, v in stage_ms.items()}
