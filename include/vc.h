@@ -274,16 +274,22 @@ vc_status vc_prove_verify(vc_circuit *c, const uint64_t *inputs, uint64_t seed, 
 typedef enum {
     VC_STAGE_PROOF = 0,     /* the whole proof                                           */
     VC_STAGE_TABLES = 1,    /* one launch: coins, layer points, eq(z_i, r_P), split eq
-                               tables, product weights                   (helper stream) */
+                               tables, product weights; then the phase-2 factors of
+                               MATMULT layers over the inputs            (helper stream) */
     VC_STAGE_EVAL = 2,      /* layer-by-layer evaluation                                  */
     VC_STAGE_WAVES = 3,     /* first persistent launch: line reductions, product-weighted
                                and on-the-fly general sum-checks (their single-chunk
                                later waves run inside it)                                */
     VC_STAGE_WAVESN = 4,    /* later persistent launches of the same kinds (wide layers) */
-    VC_STAGE_BUILD = 5,     /* phase-2/3 wiring tables (EXPLICIT layers)                 */
+    VC_STAGE_BUILD = 5,     /* phase-2/3 wiring tables of EXPLICIT layers; without any,
+                               the phase-2 factors of MATMULT layers over computed
+                               values, before the waves (with both, those factors are
+                               part of VC_STAGE_WAVES)                                   */
     VC_STAGE_TABWAVES = 6,  /* general sum-checks over the built tables                  */
     VC_STAGE_FINAL = 7,     /* per-round reductions into the transcript                  */
     VC_NUM_STAGES = 8
+    /* the check of inputs that no evaluation launch reads first runs beside
+       the waves on the helper stream: part of VC_STAGE_PROOF alone */
 } vc_stage;
 
 /* Record CUDA events around the stages of every later vc_prove on this

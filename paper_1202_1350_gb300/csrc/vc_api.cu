@@ -1369,11 +1369,11 @@ void enqueue_plan(Plan &P, cudaStream_t st)
     mark(VC_STAGE_TABLES, 0, sa);
     launch_coins(Gs, P.d_setups, (int)P.setups.size(), P.d_eqjobs, (int)P.eqjobs.size(), P.d_scis, P.d_pw, (int)P.pw.size(),
                  P.d_lw, (int)P.lw.size(), sa);
-    mark(VC_STAGE_TABLES, 1, sa);
     // MATMULT layers' phase-2 factors need the coins and the layer's inputs:
     // beside the evaluation if those are the circuit's (with the wider
     // evaluation items: MATMULT 128 from 108 to 100 us, pattern 2^14 163 to 158)
     if (P.mm_inputs) launch_mm_tables(Gs, P.d_mms, (int)P.mms.size(), sa);
+    mark(VC_STAGE_TABLES, 1, sa);
     cudaEventRecord(P.ev_tables, sa);
     // inputs not checked by an evaluation segment: the check only latches a
     // status read after the proof, so nothing but the end waits for it
@@ -1382,9 +1382,16 @@ void enqueue_plan(Plan &P, cudaStream_t st)
         cudaEventRecord(P.ev_checked, sa);
     }
     cudaStreamWaitEvent(st, P.ev_tables, 0);
-    if (!P.mm_inputs) launch_mm_tables(Gs, P.d_mms, (int)P.mms.size(), st);
+    // over computed values: a stage of its own, or part of the waves' where
+    // explicit layers' tables are the build stage
+    if (!P.mm_inputs && !has_build) {
+        mark(VC_STAGE_BUILD, 0, st);
+        launch_mm_tables(Gs, P.d_mms, (int)P.mms.size(), st);
+        mark(VC_STAGE_BUILD, 1, st);
+    }
     // line reductions, product-weighted and on-the-fly general waves
     mark(VC_STAGE_WAVES, 0, st);
+    if (!P.mm_inputs && has_build) launch_mm_tables(Gs, P.d_mms, (int)P.mms.size(), st);
     if (nA) waves(P.groupsA[0], P.d_groupsA[0], 0);
     mark(VC_STAGE_WAVES, 1, st);
     if (has_wavesn) {

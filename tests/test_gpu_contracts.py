@@ -6,7 +6,7 @@ import pytest
 
 import oracle
 from gpu_util import ensure_built, oracle_prove, to_np
-from paper_1202_1350_gb300 import SQUARE, TREE, circuits, vc
+from paper_1202_1350_gb300 import EXPLICIT, SQUARE, TREE, circuits, vc
 
 pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
@@ -199,3 +199,47 @@ def test_lone_general_instances(logn):
             assert (to_np(tr) == oracle_prove(w, k, x, 71)).all()
         finally:
             vc.vc_circuit_destroy(h)
+
+
+def stage_times(widths, kinds, x, explicit=None):
+    """(start, end) of every stage in ms after the proof's start, negative for
+    a stage that the proof did not mark."""
+    h = vc.vc_circuit_create(widths, kinds, explicit)
+    try:
+        evs = [torch.cuda.Event(enable_timing=True) for _ in range(2 * vc.NUM_STAGES)]
+        for e in evs:
+            e.record()
+        torch.cuda.synchronize()
+        vc.vc_circuit_set_stage_events(h, evs)
+        tr = torch.empty(vc.vc_transcript_len(h), dtype=torch.int64, device="cuda")
+        xd = dev(x)
+        for _ in range(2):
+            vc.vc_prove(h, xd, 81, tr)
+        vc.vc_circuit_sync(h)
+        torch.cuda.synchronize()
+        assert (to_np(tr) == oracle_prove(widths, kinds, x, 81, explicit)).all()
+        t = [evs[0].elapsed_time(e) for e in evs]
+        return list(zip(t[::2], t[1::2]))
+    finally:
+        vc.vc_circuit_destroy(h)
+
+
+PROOF, TABLES, EVAL, WAVES, WAVESN, BUILD, TABWAVES, FINAL = range(8)
+
+
+def test_stages_of_matrix_products():
+    """The launch that forms MATMULT layers' factors is inside a marked stage,
+    wherever it runs (the marks of one stream are ordered among themselves)."""
+    L = 4
+    w, k = circuits.matmult(L)
+    t = stage_times(w, k, elements(1, 1 << w[-1]))  # over the inputs: beside the evaluation
+    assert t[BUILD][0] < 0 and 0 <= t[TABLES][0] <= t[TABLES][1] and 0 <= t[EVAL][1] <= t[WAVES][0]
+    w, k = w + [2 * L + 1], k + [SQUARE]  # over computed values: a stage before the waves
+    t = stage_times(w, k, elements(2, 1 << w[-1]))
+    assert t[EVAL][1] <= t[BUILD][0] <= t[BUILD][1] <= t[WAVES][0] <= t[WAVES][1] <= t[FINAL][0]
+    S = 1 << w[-1]  # with explicit layers, whose tables come after the waves
+    ex = [None] * len(k) + [(np.arange(S, dtype=np.uint8) % 2, np.arange(S, dtype=np.uint32),
+                             np.arange(S, dtype=np.uint32)[::-1].copy())]
+    w, k = w + [2 * L + 1], k + [EXPLICIT]
+    t = stage_times(w, k, elements(3, 1 << w[-1]), ex)
+    assert t[WAVES][1] <= t[BUILD][0] <= t[BUILD][1] <= t[TABWAVES][0] <= t[FINAL][0]
