@@ -1100,7 +1100,8 @@ void sort_tasks(Plan &P)
     if (P.rounds.size() <= FINAL_ALL_WARPS) {
         P.nbig = (u32)P.rounds.size();
     } else {
-        auto many = [](const RoundRef &R) { return R.nchunks > FINAL_WARP_MIN; };
+        // (a round of TREE phase 2 has the partials of two instances)
+        auto many = [](const RoundRef &R) { return std::max(R.nchunks, R.nchunks2) > FINAL_WARP_MIN; };
         P.nbig = (u32)(std::stable_partition(P.rounds.begin(), P.rounds.end(), many) - P.rounds.begin());
     }
     auto rank = [&](const Task &t) { return t.type == TK_LINE ? 0 : (t.type == TK_GEN ? 1 : 2); };
