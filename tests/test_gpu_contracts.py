@@ -243,3 +243,43 @@ def test_stages_of_matrix_products():
     w, k = w + [2 * L + 1], k + [EXPLICIT]
     t = stage_times(w, k, elements(3, 1 << w[-1]), ex)
     assert t[WAVES][1] <= t[BUILD][0] <= t[BUILD][1] <= t[TABWAVES][0] <= t[FINAL][0]
+
+
+# layers of 22 and 23 coordinates: line chunks of 8 coordinates a thread and a
+# third line wave, product-weighted chunks of 2^14 whose next wave has one or two
+# row coordinates over values that the same launch wrote; with explicit shapes two
+# to four
+@pytest.mark.parametrize("widths,kinds,shapes", [
+    ([21, 22], [TREE], [None, (11, 12, 13, 11, 0), (12, 11, 12, 11, W)]),
+    ([22, 22], [SQUARE], [None, (9, 12, 13, 11, 0)]),
+    ([22, 23], [TREE], [None])])
+def test_wide_layers(widths, kinds, shapes):
+    x = elements(sum(widths), 1 << widths[-1])
+    want = oracle_prove(widths, kinds, x, 91)
+    xd = dev(x)
+    for shape in shapes:
+        h = vc.vc_circuit_create(widths, kinds) if shape is None else \
+            vc.vc_circuit_create_tiles(widths, kinds, tiles_of(*shape))
+        try:
+            tr = torch.empty(vc.vc_transcript_len(h), dtype=torch.int64, device="cuda")
+            for _ in range(2):
+                assert vc.vc_prove_verify(h, xd, 91, tr), shape
+                assert (to_np(tr) == want).all(), shape
+                tr.zero_()
+        finally:
+            vc.vc_circuit_destroy(h)
+
+
+# later product-weighted waves of 2^8 chunks (one row coordinate) and of a part
+@pytest.mark.parametrize("pr,logn", [(8, 17), (8, 16), (9, 18), (10, 15)])
+def test_later_waves_with_rows(pr, logn):
+    w, k = circuits.f2(logn)
+    x = elements(pr, 1 << logn)
+    h = vc.vc_circuit_create_tiles(w, k, tiles_of(pr, 12, 13, 11, 0))
+    try:
+        tr = torch.empty(vc.vc_transcript_len(h), dtype=torch.int64, device="cuda")
+        vc.vc_prove(h, dev(x), 101, tr)
+        vc.vc_circuit_sync(h)
+        assert (to_np(tr) == oracle_prove(w, k, x, 101)).all()
+    finally:
+        vc.vc_circuit_destroy(h)
