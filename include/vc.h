@@ -588,12 +588,13 @@ vc_status vc_field_mul(const uint64_t *a, const uint64_t *b, uint64_t *out, uint
  * CUDA events after a warm-up launch, and returns units per second in *rate.
  * variant 0: canonical 32-bit-limb Mersenne product + add (8 chains; units:
  * field products); 1: canonical 64x64->128 product, fold, add (8 chains;
- * field products); 2: the product-weighted sum-check pair step of the
- * dominant kernel (two exact 128-bit multiply-adds and one lazily reduced
- * fold, counted as three field products), the best of 2, 4 and 8 pairs per
- * thread at several register budgets; 3: 32-bit integer multiply-adds (8
- * chains; units: multiply-adds); 4: exact 64x64->128-bit multiply-accumulates
- * (8 accumulators; units: multiply-accumulates).  Synchronous; VC_EINVAL for
+ * field products); 2: a sum-check pair step of a prover that folds round by
+ * round (two exact 128-bit multiply-adds and one lazily reduced fold, counted
+ * as three field products), the best of 2, 4 and 8 pairs per thread at several
+ * register budgets; 3: 32-bit integer multiply-adds (8 chains; units:
+ * multiply-adds); 4: exact 64x64->128-bit multiply-accumulates, what the
+ * product-weighted chunks of the dominant kernel consist of (8 accumulators;
+ * units: multiply-accumulates).  Synchronous; VC_EINVAL for
  * another variant or iters = 0, VC_ECUDA on a CUDA error. */
 vc_status vc_field_mul_rate(int device, int variant, uint64_t iters, double *rate);
 

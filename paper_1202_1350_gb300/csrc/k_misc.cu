@@ -70,8 +70,9 @@ __global__ void __launch_bounds__(256) k_mul_rate(u64 iters, u64 *sink)
     if (s == 0x12345) sink[0] = s;  // keeps the chains alive
 }
 
-// The sum-check pair primitive of the product-weighted waves: per step two
-// multiply-adds into 128-bit accumulators and one lazy fold (3 products).
+// The pair step of a sum-check that folds round by round (the general chunks'
+// kind of work): per step two multiply-adds into 128-bit accumulators and one
+// lazy fold (3 products).
 // CH independent pairs per thread; MINB resident CTAs per SM the register
 // allocation is sized for.
 template <int CH, int MINB>
@@ -131,14 +132,16 @@ __global__ void __launch_bounds__(256) k_imad_rate(u64 iters, u64 *sink)
 }
 
 // Exact 64x64 -> 128-bit multiply-accumulate rate (the `mac` of the sum-check
-// waves): CH independent accumulators per thread.
+// waves): CH independent accumulators per thread.  One operand changes every
+// step: with both fixed the compiler takes parts of the products out of the loop
+// (1.1 wide products a step by the pipe's counters, where an exact one has four).
 template <int CH>
 __global__ void __launch_bounds__(256) k_mac_rate(u64 iters, u64 *sink)
 {
     acc128 a[CH];
     u64 x[CH];
     const u64 t = blockIdx.x * (u64)blockDim.x + threadIdx.x;
-    const u64 y = (t * 0xBF58476D1CE4E5B9ull) & FP_P;
+    u64 y = t * 0xBF58476D1CE4E5B9ull + 1;
 #pragma unroll
     for (int c = 0; c < CH; c++) {
         acc_zero(a[c]);
@@ -147,6 +150,7 @@ __global__ void __launch_bounds__(256) k_mac_rate(u64 iters, u64 *sink)
     for (u64 k = 0; k < iters; k++) {
 #pragma unroll
         for (int c = 0; c < CH; c++) mac(a[c], x[c], y);
+        y = (y << 7) | (y >> 57);
     }
     u64 s = 0;
 #pragma unroll

@@ -283,3 +283,13 @@ def test_later_waves_with_rows(pr, logn):
         assert (to_np(tr) == oracle_prove(w, k, x, 101)).all()
     finally:
         vc.vc_circuit_destroy(h)
+
+
+def test_multiply_accumulate_rate_is_of_whole_products():
+    """Variant 4's exact multiply-accumulates against variant 2's pair steps
+    (three products each).  The multiply pipe bounds both: a product is four
+    wide ones, eight of the 10.5 pipe cycles a product of the pair step takes
+    by the counters, so a multiply-accumulate is at most 10.5 / 8 = 1.31 times as
+    fast (1.5 times when parts of the products left the loop)."""
+    pair, mac = (max(vc.vc_field_mul_rate(0, v, 1 << 12) for _ in range(3)) for v in (2, 4))
+    assert mac < 1.35 * pair
