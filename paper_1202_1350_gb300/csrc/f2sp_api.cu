@@ -51,8 +51,9 @@ u64 h_pow(u64 b, u64 e)
 u64 h_inv(u64 a) { return h_pow(a, FP_P - 2); }
 
 // The factors of h for the prime-factor transform: pairwise coprime prime
-// powers, each a divisor of p - 1 and at most 61 (so that a length-q DFT sums
-// at most 61 exact products in 128 bits).  False if h has another factor.
+// powers, each a divisor of p - 1 and at most 61 (a thread keeps the (q - 1) / 2
+// sums or differences of a line in registers, and the kernel has code for these
+// sizes alone).  False if h has another factor.
 bool sp_factor(u64 h, std::vector<u32> &q)
 {
     static const u32 primes[] = {3, 5, 7, 11, 13, 31, 41, 61};

@@ -169,10 +169,9 @@ __device__ __forceinline__ u64 wmul(u64 x, u64 y)
 }
 
 // u0 + a d for u0 in W, d < 1.5 2^62 (a lazy difference u1 + 2p - u0 of W
-// values) and canonical a: an exact 128-bit product, below 1.5 2^123 (so u0 + the
-// remainder + the quotient stay below 2^64), reduced once.  (In 31/30-bit limbs, without carries between the partial
-// products, the same took about half as many instructions again, which bound
-// the folds.)
+// values) and canonical a.  The exact product is below 1.5 2^123, so u0, its
+// remainder and its quotient add up below 2^64 and are reduced once.  (In 31-
+// and 30-bit limbs the same took half as many instructions again.)
 __device__ __forceinline__ u64 wlin1(u64 u0, u64 d, u64 a)
 {
     const unsigned __int128 t = (unsigned __int128)a * d;

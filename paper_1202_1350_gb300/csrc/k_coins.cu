@@ -7,8 +7,9 @@
 // splitmix64 stream, Sec. 3.1's "verifier picks at random", made
 // reproducible), so each CTA derives the challenges its job needs itself and
 // no CTA waits for another.  A draw equal to p is rejected and the stream
-// shifts (probability 2^-61 per draw): each CTA checks all of its circuit's
-// draws and then takes the shifted sequence the slow way.
+// shifts (probability 2^-61 per draw): each CTA finds out whether any of its
+// circuit's draws is (eight products, draws_rejected) and then walks the
+// stream to each of its challenges.
 #include <cuda_runtime.h>
 #include "coins.cuh"
 

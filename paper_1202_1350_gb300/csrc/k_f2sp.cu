@@ -41,7 +41,8 @@
 // Prover CTA: 1024 threads (64 registers each) when every dimension is at most
 // 13, whose lines fit that; 512 (128 registers) otherwise.  A line's products
 // are dependent chains, so warps in flight matter: at 4995 x 5005 16 warps an
-// SM issued in 42 % of the cycles.
+// SM issued in 42 % of the cycles.  (Both spill a few words around the calls of
+// the passes, once a pass; the lines' loops do not.)
 #define SP_PNT 1024
 #define SP_PNT_BIG 512
 
