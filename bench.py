@@ -159,17 +159,18 @@ def executed_work(widths, kinds, tiles=None):
     return mul
 
 
-# DRAM bytes (read + write) of one k_waves launch on this workload, from an ncu
-# capture of the current kernel; the V tables are mostly served from L2, so
-# this is below the algorithmic bytes
-K_WAVES_DRAM_BYTES = 25_881_856
+# DRAM bytes of one k_waves launch on this workload, from an ncu capture of the
+# current kernel (profiles/k_waves_f2_2e20.md): 25,872,384 read, none written.
+# The capture starts with a flushed L2, so the values are read from DRAM once;
+# every further read of them is served from L2
+K_WAVES_DRAM_BYTES = 25_872_384
 # The same launch's integer pipes (ncu, % of peak sustained while active):
 # the multiply pipe (fmaheavy) cycles, ALU pipe cycles, issue slots
-K_WAVES_PIPES = {"fmaheavy_cycles_pct": 56.8, "alu_cycles_pct": 35.9, "issue_active_pct": 43.6}
-# ncu: the pair-step microbenchmark keeps the multiply pipe (fmaheavy) busy
-# this fraction of its cycles (83-86 % over its configurations), so the pipe
-# saturated would give its rate / this fraction
-PAIR_STEP_FMAHEAVY_FRAC = 0.847
+K_WAVES_PIPES = {"fmaheavy_cycles_pct": 56.8, "alu_cycles_pct": 36.5, "issue_active_pct": 44.1}
+# ncu: the multiply-accumulate microbenchmark keeps the multiply pipe (fmaheavy)
+# busy this fraction of its cycles, so the pipe saturated would give its rate /
+# this fraction
+MAC_FMAHEAVY_FRAC = 0.922
 
 
 def run_ablation(h, xd, tr, flush, reps=5):
@@ -870,8 +871,8 @@ def run_ours(args):
     wave_launch_ms = statistics.mean(wave_ms)
     mul, byts = algorithmic_work(widths, kinds)
     executed = executed_work(widths, kinds, vc.vc_circuit_get_tiles(h))
-    rate = vc.vc_field_mul_rate(local, 2, 1 << 12)
-    achieved = mul / (wave_launch_ms / 1000)
+    rate = vc.vc_field_mul_rate(local, 4, 1 << 12)
+    achieved = executed / (wave_launch_ms / 1000)
     stages = {name: round(statistics.mean(v), 4) for name, v in stage_ms.items()}
     launches = (info["prove_launches"] + info["verify2_launches"]) * args.steps
     line = {
@@ -887,19 +888,20 @@ def run_ours(args):
         "e2e": e2e,
         "roofline": {"bound": "alu", "kernel": "k_waves (persistent launch: every sum-check round and line "
                                                 "reduction of the F2 circuit)",
-                     "achieved": achieved / 1e12, "peak": rate / 1e12, "unit": "Tmulmod/s",
+                     "achieved": achieved / 1e12, "peak": rate / 1e12, "unit": "T products/s",
                      "frac": achieved / rate, "traffic": K_WAVES_DRAM_BYTES,
                      "traffic_unit": "bytes per launch (ncu dram__bytes_read.sum + dram__bytes_write.sum)",
-                     "peak_source": "measured on this GPU: vc_field_mul_rate variant 2, a sum-check "
-                                    "pair step (2 exact multiply-adds + 1 lazy fold), best of 5 chain-count and "
-                                    "register-budget configurations on a one-wave grid; ncu shows that step keeps "
-                                    "the integer-multiply (fmaheavy) pipe 83-86 % of its cycles busy "
+                     "achieved_rule": "products the launch executes (executed_mulmods) / kernel_ms",
+                     "peak_source": "measured on this GPU: vc_field_mul_rate variant 4, exact 64x64->128-bit "
+                                    "multiply-accumulates on a one-wave grid; ncu shows them keep the "
+                                    "integer-multiply (fmaheavy) pipe 92 % of its cycles busy "
                                     "(profiles/int_rate_microbench.md)",
-                     "peak_pipe_saturated": rate / PAIR_STEP_FMAHEAVY_FRAC / 1e12,
-                     "frac_of_pipe_saturated": achieved / (rate / PAIR_STEP_FMAHEAVY_FRAC),
-                     "kernel_pipes_ncu": K_WAVES_PIPES,
-                     "algorithmic_mulmods": mul, "algorithmic_rule": "7 S_i + 24 S_{i+1} per layer (folding prover)",
-                     "executed_mulmods": executed, "executed_frac": executed / (wave_launch_ms / 1000) / rate,
+                     "peak_pipe_saturated": rate / MAC_FMAHEAVY_FRAC / 1e12,
+                     "frac_of_pipe_saturated": achieved / (rate / MAC_FMAHEAVY_FRAC),
+                     "kernel_pipes_ncu": K_WAVES_PIPES, "executed_mulmods": executed,
+                     # what a prover that folds round by round multiplies for the same proof
+                     # (not a rate of this kernel, which needs two fifths of it)
+                     "folding_prover_mulmods": mul, "folding_prover_rule": "7 S_i + 24 S_{i+1} per layer",
                      "algorithmic_bytes": byts, "kernel_ms": wave_launch_ms,
                      "bytes_frac_of_hbm": (byts / (wave_launch_ms / 1000)) / (measured_peaks().get("hbm_gbs", 6787.9) * 1e9)},
         "stage_ms": stages,
