@@ -150,11 +150,12 @@ def test_explicit_tiles_are_used_as_they_are(shape, logn):
         vc.vc_circuit_destroy(h)
 
 
-@pytest.mark.parametrize("logn", [12, 20])
+@pytest.mark.parametrize("logn", [13, 20])
 def test_default_tiles_are_named_by_size(logn):
     """What a circuit without tiles reports is what it was planned with: the
     same shapes again give the same plan, and a numeric split leaves the sizes
-    of wider instances' chunks alone."""
+    of wider instances' chunks alone.  (Sizes that no test has tuned: a recorded
+    choice would be what such a circuit reports.)"""
     w, k = circuits.f2(logn)
     hs = [vc.vc_circuit_create(w, k)]
     try:
