@@ -341,7 +341,7 @@ vc_status vc_circuit_get_info(const vc_circuit *c, vc_circuit_info *info);
  * layer, else <= 40).  The three chunk sizes may be VC_TILE_BY_SIZE, the
  * default of circuits created without tiles: each instance's chunk then
  * follows its own size (product-weighted 13, from 19 coordinates 14, and
- * VC_SPLIT_WIDEST halves none of 14 coordinates or more; general 10 to 12;
+ * VC_SPLIT_WIDEST halves none of 14 coordinates or more; general 7 to 12;
  * line 12 to 15).  A number is used as it is.  Any choice gives the same
  * transcript; they only change speed. */
 #define VC_SPLIT_WIDEST 0xFFFFFFFFu

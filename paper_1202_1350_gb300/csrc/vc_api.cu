@@ -469,15 +469,16 @@ static u32 pr_chunk_of(const PlanConfig &f, u32 n, u32 smax)
 // `entries` in all.  By size few coordinates take smaller chunks: a lone
 // thread's 32 entries are a chain of about 2,700 cycles per 4 (F0 2^11 44.8 us
 // with 2^12, F0 2^14 90 against 85 with 2^11; under load 2^12 wins: F0 2^16 199
-// against 222).  11 coordinates, the least that do not fit one chunk of 2^10,
-// take 2^8 where the circuit has at most 2^12 such entries, so that the launch
-// is short of work anyway and only rounds 0 and 1 run in registers (F2 2^11
-// 26.7 -> 24.7 us, 43.0 -> 37.1 with the L2 flushed, MATMULT 32 52.7 -> 48.7;
-// at 12 as well, 576 merged circuits lose 0.6 %, so 0.2 %).
+// against 222).  10 and 11 coordinates take eight chunks where the circuit has
+// at most 2^12 such entries: the launch is short of work anyway, and little or
+// none of the register rounds' code is run, which a flushed L2 makes slow to
+// fetch (F2 2^10 22.6 -> 22.6 us, flushed 39.0 -> 29.6; 2^11 26.7 -> 24.6, flushed
+// 43.0 -> 37.0; 576 merged circuits 2048 -> 2055; at 11 coordinates 2^7, or
+// sixteen chunks at 12, 0.3 % more there).
 static u32 gn_chunk_of(const PlanConfig &f, u32 n, u64 entries)
 {
     if (f.gn_chunk != VC_TILE_BY_SIZE) return f.gn_chunk;
-    if (n == 11 && entries <= (u64(1) << 12)) return 8;
+    if ((n == 10 || n == 11) && entries <= (u64(1) << 12)) return n - 3;
     return n <= 12 ? 10u : n <= 15 ? 11u : GN_CHUNK_LOG;
 }
 
